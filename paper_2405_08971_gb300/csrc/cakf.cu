@@ -375,7 +375,7 @@ int plan_and_alloc(cakf_ctx* c, const cakf_problem* p) {
   if ((rc = c->alloc(c->GV, mm * std::max(B, 1) * es))) return rc;
   if ((rc = c->alloc(c->GS, mm * std::max(B, 1) * es))) return rc;
   if ((rc = c->alloc(c->Qa, mm * std::max(B, 1) * es))) return rc;
-  if ((rc = c->alloc(c->part, mm * std::max(32, gram_matvec_slots((int)mm)) * es))) return rc;
+  if ((rc = c->alloc(c->part, gram_matvec_part_elems((int)mm) * es))) return rc;
   if ((rc = c->alloc(c->tv, std::max<size_t>(c->rmax, 1) * ((mm + 1023) / 1024 + 1) * es))) return rc;
   if ((rc = c->alloc(c->dots, (B + 8) * sizeof(double)))) return rc;
   if ((rc = c->alloc(c->dots2, (B + 8) * sizeof(double)))) return rc;
@@ -725,7 +725,7 @@ struct Runner {
         rtol2 = c->cg_rtol * c->cg_rtol * r0sq;
         use_rtol = 1;
       }
-      const int nsplit = gram_matvec_slots(m);
+      const int nsplit = gram_matvec_slots(m, sizeof(T));
       const double* rep = (c->replay && !recompute) ? c->rep + c->off_rep[k] : nullptr;
       T* Qa = (T*)c->Qa;       // orthonormal basis of the previous actions (CG policy only)
       // Re-orthogonalising each action against the previous ones leaves span(S) -- and so every

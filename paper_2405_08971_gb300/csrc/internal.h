@@ -39,8 +39,10 @@ template <class T>
 // partials of Mo^T s (Mo: m x rp, ld ldm) into tpart for cg_combine
 void gram_matvec(int ker, const C4<T>* Xo, const T* s, int m, T sf2, T* part, const T* Mo, int ldm, int rp, T* tpart,
                  const int* active, cudaStream_t st);
-// number of partial slots (rows of part, each m long) gram_matvec writes for m observations
-int gram_matvec_slots(int m);
+// number of partial slots (rows of part, each m long) gram_matvec writes for m observations of the
+// given element size, and the elements that part needs for every step with up to mmax observations
+int gram_matvec_slots(int m, int elem_size);
+size_t gram_matvec_part_elems(int mmax);
 template <class T>
 void gram_block_simt(int ker, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, const T* B, int ldb, int width,
                      T sf2, T* Out, int ldo, cudaStream_t st);

@@ -65,38 +65,48 @@ __global__ void k_gather_coords(const C4<T>* __restrict__ X, const int* __restri
 // chunk of GV_CHUNK rows), which k_cg_combine needs next: one launch for both.
 constexpr int MVS_T = 128, MVS_R = MVS_T / 32, MVS_W = MVS_T / 32;
 constexpr int GV_CHUNK = 1024;
-template <int KER, class T>
+
+// Partials of t = Mo^T s: block b of the first ngv blocks of a matvec launch.
+template <class T>
+__device__ __forceinline__ void gv_block(const T* __restrict__ Mo, int ldm, int rp, const T* __restrict__ s, int m,
+                                         T* __restrict__ tpart) {
+  const int per_chunk = (rp + MVS_W - 1) / MVS_W;
+  const int z = blockIdx.x / per_chunk;
+  const int col = (blockIdx.x - z * per_chunk) * MVS_W + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (col >= rp) return;
+  const int i0 = z * GV_CHUNK, i1 = min(m, i0 + GV_CHUNK);
+  const T* a = Mo + (size_t)col * ldm;
+  T acc = T(0);
+#pragma unroll 8
+  for (int i = i0 + lane; i < i1; i += 32) acc = fma(a[i], s[i], acc);
+  acc = warp_sum(acc);
+  if (lane == 0) tpart[(size_t)z * rp + col] = acc;
+}
+
+// The FP64 matvec on TILE x TILE tiles, R = TILE / 32 rows per lane, TILE / MVS_W columns per warp.
+template <int KER, class T, int R>
 __global__ void __launch_bounds__(MVS_W * 32)
 k_gram_matvec(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int nb, T sf2, T* __restrict__ part,
               const T* __restrict__ Mo, int ldm, int rp, int ngv, T* __restrict__ tpart,
               const int* __restrict__ active) {
+  constexpr int TILE = 32 * R, CW = TILE / MVS_W;
   pdl_wait();
   pdl_trigger();
   if (active && !*active) return;
-  __shared__ C4<T> xs[MVS_T];
-  __shared__ T ss[MVS_T];
-  __shared__ T racc[MVS_W][MVS_T];
+  __shared__ C4<T> xs[TILE];
+  __shared__ T ss[TILE];
+  __shared__ T racc[MVS_W][TILE];
   if ((int)blockIdx.x < ngv) {
-    const int per_chunk = (rp + MVS_W - 1) / MVS_W;
-    const int z = blockIdx.x / per_chunk;
-    const int col = (blockIdx.x - z * per_chunk) * MVS_W + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (col >= rp) return;
-    const int i0 = z * GV_CHUNK, i1 = min(m, i0 + GV_CHUNK);
-    const T* a = Mo + (size_t)col * ldm;
-    T acc = T(0);
-#pragma unroll 8
-    for (int i = i0 + lane; i < i1; i += 32) acc = fma(a[i], s[i], acc);
-    acc = warp_sum(acc);
-    if (lane == 0) tpart[(size_t)z * rp + col] = acc;
+    gv_block(Mo, ldm, rp, s, m, tpart);
     return;
   }
   int idx = blockIdx.x - ngv, I = 0;
   while (idx >= nb - I) { idx -= nb - I; ++I; }
   const int J = I + idx;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = threadIdx.x; t < MVS_T; t += blockDim.x) {
-    const int j = J * MVS_T + t;
+  for (int t = threadIdx.x; t < TILE; t += blockDim.x) {
+    const int j = J * TILE + t;
     C4<T> x;
     x.x = x.y = x.z = x.w = T(0);
     T v = T(0);
@@ -104,11 +114,11 @@ k_gram_matvec(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int 
     xs[t] = x;
     ss[t] = v;
   }
-  C4<T> xi[MVS_R];
-  T si[MVS_R], acc[MVS_R];
+  C4<T> xi[R];
+  T si[R], acc[R];
 #pragma unroll
-  for (int r = 0; r < MVS_R; ++r) {
-    const int i = I * MVS_T + lane + 32 * r;
+  for (int r = 0; r < R; ++r) {
+    const int i = I * TILE + lane + 32 * r;
     xi[r].x = xi[r].y = xi[r].z = xi[r].w = T(0);
     si[r] = T(0);
     if (i < m) { xi[r] = Xo[i]; si[r] = s[i]; }
@@ -118,20 +128,20 @@ k_gram_matvec(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int 
   T cacc = T(0);
   if (I == J) {
 #pragma unroll 4
-    for (int jj = 0; jj < 32; ++jj) {
-      const C4<T> xj = xs[warp * 32 + jj];
-      const T sj = ss[warp * 32 + jj];
+    for (int jj = 0; jj < CW; ++jj) {
+      const C4<T> xj = xs[warp * CW + jj];
+      const T sj = ss[warp * CW + jj];
 #pragma unroll
-      for (int r = 0; r < MVS_R; ++r) acc[r] = fma(kval<KER>(dist2(xi[r], xj), sf2), sj, acc[r]);
+      for (int r = 0; r < R; ++r) acc[r] = fma(kval<KER>(dist2(xi[r], xj), sf2), sj, acc[r]);
     }
   } else {
 #pragma unroll 4
-    for (int jj = 0; jj < 32; ++jj) {
-      const C4<T> xj = xs[warp * 32 + jj];
-      const T sj = ss[warp * 32 + jj];
+    for (int jj = 0; jj < CW; ++jj) {
+      const C4<T> xj = xs[warp * CW + jj];
+      const T sj = ss[warp * CW + jj];
       T cp = T(0);
 #pragma unroll
-      for (int r = 0; r < MVS_R; ++r) {
+      for (int r = 0; r < R; ++r) {
         const T kv = kval<KER>(dist2(xi[r], xj), sf2);
         acc[r] = fma(kv, sj, acc[r]);
         cp = fma(kv, si[r], cp);
@@ -141,19 +151,55 @@ k_gram_matvec(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int 
     }
   }
 #pragma unroll
-  for (int r = 0; r < MVS_R; ++r) racc[warp][lane + 32 * r] = acc[r];
+  for (int r = 0; r < R; ++r) racc[warp][lane + 32 * r] = acc[r];
   __syncthreads();
-  for (int t = threadIdx.x; t < MVS_T; t += blockDim.x) {
-    const int i = I * MVS_T + t;
+  for (int t = threadIdx.x; t < TILE; t += blockDim.x) {
+    const int i = I * TILE + t;
     if (i >= m) continue;
     T v = racc[0][t];
 #pragma unroll
     for (int w = 1; w < MVS_W; ++w) v += racc[w][t];
     part[(size_t)J * m + i] = v;
   }
-  if (I != J) {
-    const int j = J * MVS_T + warp * 32 + lane;
+  if (I != J && lane < CW) {
+    const int j = J * TILE + warp * CW + lane;
     if (j < m) part[(size_t)I * m + j] = cacc;
+  }
+}
+
+// The FP64 matvec for few observations, where even 32 x 32 tiles leave most SMs idle: every entry is
+// evaluated (no symmetry), a block takes 32 rows (one per lane) and MVS_W * cpw columns (cpw per
+// warp), and its sum goes to the slot of its column group, so the slots per row number
+// ceil(m / (MVS_W cpw)) and no column sums are needed.  An FP64 Matern value is about 60 dependent
+// FP64 operations (a warp-wide one takes 19 cycles of the SM's FP64 pipe), so what counts is how many
+// SMs share the values.
+template <int KER, class T>
+__global__ void __launch_bounds__(MVS_W * 32)
+k_gram_matvec_rows(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int nslot, int cpw, T sf2,
+                   T* __restrict__ part, const T* __restrict__ Mo, int ldm, int rp, int ngv, T* __restrict__ tpart,
+                   const int* __restrict__ active) {
+  pdl_wait();
+  pdl_trigger();
+  if (active && !*active) return;
+  __shared__ T racc[MVS_W][32];
+  if ((int)blockIdx.x < ngv) {
+    gv_block(Mo, ldm, rp, s, m, tpart);
+    return;
+  }
+  const int b = blockIdx.x - ngv, rt = b / nslot, slot = b - rt * nslot;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = rt * 32 + lane;
+  const C4<T> xi = Xo[min(i, m - 1)];
+  const int j0 = (slot * MVS_W + warp) * cpw;
+  T acc = T(0);
+  for (int j = j0; j < min(m, j0 + cpw); ++j) acc = fma(kval<KER>(dist2(xi, Xo[j]), sf2), s[j], acc);
+  racc[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && i < m) {
+    T v = racc[0][lane];
+#pragma unroll
+    for (int w = 1; w < MVS_W; ++w) v += racc[w][lane];
+    part[(size_t)slot * m + i] = v;
   }
 }
 
@@ -174,17 +220,7 @@ k_gram_matvec_f2(const C4<float>* __restrict__ Xo, const float* __restrict__ s, 
   __shared__ float racc[MVS_W][MVS_T];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if ((int)blockIdx.x < ngv) {
-    const int per_chunk = (rp + MVS_W - 1) / MVS_W;
-    const int z = blockIdx.x / per_chunk;
-    const int col = (blockIdx.x - z * per_chunk) * MVS_W + warp;
-    if (col >= rp) return;
-    const int i0 = z * GV_CHUNK, i1 = min(m, i0 + GV_CHUNK);
-    const float* a = Mo + (size_t)col * ldm;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int i = i0 + lane; i < i1; i += 32) acc = fmaf(a[i], s[i], acc);
-    acc = warp_sum(acc);
-    if (lane == 0) tpart[(size_t)z * rp + col] = acc;
+    gv_block(Mo, ldm, rp, s, m, tpart);
     return;
   }
   int idx = blockIdx.x - ngv, I = 0;
@@ -837,6 +873,138 @@ k_gemm_tn_part(const T* __restrict__ A, int lda, int na, const T* __restrict__ B
     }
 }
 
+// The FP64 factor products.  GB300's FP64 pipe takes 19 cycles of its SM per warp-wide FMA, so a tile
+// needs no register blocking to keep it busy (one or two shared loads per FMA are free); what the
+// products of the FP64 mode need is blocks on every SM and no padding: outputs are taken 32 rows by
+// single columns, and the columns per warp (1, 2, 4) shrink until the grid fills the GPU.
+// Measured in the gradient pass of the 1,024-point model (M = 1,024): N = 256, K = 288 takes 133 us
+// against 318 us with 64 x 64 tiles (64 blocks), N = 33 about 22 us against 150 us (16 blocks).
+constexpr int G64_WARPS = 8;
+// C[M x N] = alpha A[M x K] B[K x N] + beta C: lane = row, CPW columns per warp, the next 4 values of k
+// loaded while the current ones are used.  Every output sums over k in ascending order.
+template <int CPW>
+__global__ void __launch_bounds__(G64_WARPS * 32)
+k_gemm_nn_f64(int M, int N, int K, double alpha, const double* __restrict__ A, int lda, const double* __restrict__ B,
+              int ldb, double beta, double* __restrict__ C, int ldc) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = blockIdx.x * 32 + lane;
+  const int n0 = (blockIdx.y * G64_WARPS + warp) * CPW;
+  if (n0 >= N) return;
+  const double* a = A + min(row, M - 1);
+  const double* b[CPW];
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) b[c] = B + (size_t)min(n0 + c, N - 1) * ldb;
+  double acc[CPW];
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) acc[c] = 0.0;
+  constexpr int U = 4;
+  double av[U], bv[CPW][U];
+  const int K4 = K / U * U;
+  if (K4 > 0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      av[u] = a[(size_t)u * lda];
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) bv[c][u] = b[c][u];
+    }
+  }
+  for (int k = 0; k < K4; k += U) {
+    double an[U], bn[CPW][U];
+    const int kn = k + U < K4 ? k + U : 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      an[u] = a[(size_t)(kn + u) * lda];
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) bn[c][u] = b[c][kn + u];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) acc[c] = fma(av[u], bv[c][u], acc[c]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      av[u] = an[u];
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) bv[c][u] = bn[c][u];
+    }
+  }
+  for (int k = K4; k < K; ++k) {
+    const double x = a[(size_t)k * lda];
+#pragma unroll
+    for (int c = 0; c < CPW; ++c) acc[c] = fma(x, b[c][k], acc[c]);
+  }
+  if (row >= M) return;
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) {
+    if (n0 + c >= N) break;
+    double* p = C + (size_t)(n0 + c) * ldc + row;
+    *p = beta == 0.0 ? alpha * acc[c] : fma(alpha, acc[c], beta * *p);
+  }
+}
+
+// part[z][a + b*na] = sum_{t in chunk z} A[t, a] B[t, b] (A: K x na, B: K x nb): 32 columns of A by
+// G64_WARPS * CPW columns of B per block, 32 values of t staged through shared memory at a time
+// (their loads in flight while the previous ones are used).  With one chunk the output is written
+// directly (C = alpha sum + beta C).
+template <int CPW>
+__global__ void __launch_bounds__(G64_WARPS * 32)
+k_gemm_tn_f64(const double* __restrict__ A, int lda, int na, const double* __restrict__ B, int ldb, int nb, int K,
+              int chunk, double* __restrict__ part, double alpha, double beta, double* __restrict__ C, int ldc) {
+  constexpr int NBC = G64_WARPS * CPW;
+  __shared__ double As[32][33], Bs[32][NBC + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int a0 = blockIdx.x * 32, b0 = blockIdx.y * NBC;
+  const int kb = blockIdx.z * chunk, ke = min(K, kb + chunk);
+  double ra[4], rb[CPW], acc[CPW];
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) acc[c] = 0.0;
+  // lane = t within the stage, warp w loads columns w, w + 8, ... of both operands
+  auto load = [&](int k0) {
+    const int t = k0 + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int col = a0 + warp + G64_WARPS * u;
+      ra[u] = (t < ke && col < na) ? A[(size_t)col * lda + t] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) {
+      const int col = b0 + warp + G64_WARPS * u;
+      rb[u] = (t < ke && col < nb) ? B[(size_t)col * ldb + t] : 0.0;
+    }
+  };
+  load(kb);
+  for (int k0 = kb; k0 < ke; k0 += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) As[lane][warp + G64_WARPS * u] = ra[u];
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) Bs[lane][warp + G64_WARPS * u] = rb[u];
+    __syncthreads();
+    if (k0 + 32 < ke) load(k0 + 32);
+    if (b0 + warp * CPW < nb) {
+#pragma unroll 8
+      for (int t = 0; t < 32; ++t) {
+        const double x = As[t][lane];
+#pragma unroll
+        for (int c = 0; c < CPW; ++c) acc[c] = fma(x, Bs[t][warp * CPW + c], acc[c]);
+      }
+    }
+  }
+  const int a = a0 + lane;
+  if (a >= na) return;
+#pragma unroll
+  for (int c = 0; c < CPW; ++c) {
+    const int b = b0 + warp * CPW + c;
+    if (b >= nb) break;
+    if (part) {
+      part[blockIdx.z * (size_t)na * nb + (size_t)b * na + a] = acc[c];
+    } else {
+      double* o = C + (size_t)b * ldc + a;
+      *o = alpha * acc[c] + (beta != 0.0 ? beta * *o : 0.0);
+    }
+  }
+}
+
 // C[a + b*ldc] = alpha * sum_z part[z][a + b*na]  (+ beta * C)
 template <class OutT>
 __global__ void k_reduce_splits(const double* __restrict__ part, int nsplit, int na, int nb, double alpha,
@@ -1477,27 +1645,54 @@ void gather_coords(const C4<T>* X, const int* idx, int m, C4<T>* out, cudaStream
   k_gather_coords<T><<<cdiv(m, 256), 256, 0, st>>>(X, idx, m, out); note_launch();
 }
 
-int gram_matvec_slots(int m) { return std::max(1, (m + MVS_T - 1) / MVS_T); }
+// Tiling of the FP64 matvec by the observation count (Matern-5/2; a 128 x 128 tile costs 185 us on its
+// SM whatever the others do, a 32 x 32 one about 18 us):
+//   m <= 416        every entry, one row per lane: 5.7 us a launch at m = 128 against 185 us for the one
+//                   128-wide tile.  Its cost grows as m^2 / 152 SMs and meets the one wave of 32 x 32
+//                   tiles (m <= 544: 152 blocks) between m = 400 and 500
+//   m <= 2048       32 x 32 tiles of the upper triangle: m = 2048 has 2,080 of them, the block count of
+//                   m = 8,192 with 128 x 128 tiles, and the same 64 slots
+//   above           128 x 128 tiles, whose slots grow as m / 128
+constexpr int MV64_ROWS_MAX = 416, MV64_SMALL_TILE_MAX = 2048;
+static int mv64_cpw(int m) { return std::max(1, (m + 255) / 256); }   // columns per warp: at most 64 slots
+int gram_matvec_slots(int m, int elem_size) {
+  if (m <= 0) return 1;
+  if (elem_size == 8 && m <= MV64_ROWS_MAX) return (m + MVS_W * mv64_cpw(m) - 1) / (MVS_W * mv64_cpw(m));
+  if (elem_size == 8 && m <= MV64_SMALL_TILE_MAX) return (m + 31) / 32;
+  return (m + MVS_T - 1) / MVS_T;
+}
+size_t gram_matvec_part_elems(int mmax) {
+  return (size_t)std::max(mmax, 1) * std::max(64, (mmax + MVS_T - 1) / MVS_T);
+}
 
+template <int KER, class T>
+static void launch_matvec(const C4<T>* Xo, const T* s, int m, T sf2, T* part, const T* Mo, int ldm, int rp, T* tpart,
+                          const int* active, cudaStream_t st) {
+  const int nb = gram_matvec_slots(m, sizeof(T));
+  const int ngv = rp > 0 ? (int)cdiv(m, GV_CHUNK) * (int)cdiv(rp, MVS_W) : 0;
+  const int grid = ngv + nb * (nb + 1) / 2;
+  if constexpr (sizeof(T) == 4) {
+    launch_pdl(k_gram_matvec_f2<KER>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv,
+               tpart, active);
+  } else if (m <= MV64_ROWS_MAX) {
+    launch_pdl(k_gram_matvec_rows<KER, T>, dim3(ngv + nb * (int)cdiv(m, 32)), dim3(MVS_W * 32), 0, st, Xo, s, m, nb,
+               mv64_cpw(m), sf2, part, Mo, ldm, rp, ngv, tpart, active);
+  } else if (m <= MV64_SMALL_TILE_MAX) {
+    launch_pdl(k_gram_matvec<KER, T, 1>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp,
+               ngv, tpart, active);
+  } else {
+    launch_pdl(k_gram_matvec<KER, T, MVS_R>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp,
+               ngv, tpart, active);
+  }
+}
 template <class T>
 void gram_matvec(int ker, const C4<T>* Xo, const T* s, int m, T sf2, T* part, const T* Mo, int ldm, int rp, T* tpart,
                  const int* active, cudaStream_t st) {
   if (m <= 0) return;
-  const int nb = gram_matvec_slots(m);
-  const int ngv = rp > 0 ? (int)cdiv(m, GV_CHUNK) * (int)cdiv(rp, MVS_W) : 0;
-  const int grid = ngv + nb * (nb + 1) / 2;
-  if constexpr (sizeof(T) == 4) {
-    switch (ker) {
-      case 0: launch_pdl(k_gram_matvec_f2<0>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-      case 1: launch_pdl(k_gram_matvec_f2<1>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-      default: launch_pdl(k_gram_matvec_f2<2>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-    }
-  } else {
-    switch (ker) {
-      case 0: launch_pdl(k_gram_matvec<0, T>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-      case 1: launch_pdl(k_gram_matvec<1, T>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-      default: launch_pdl(k_gram_matvec<2, T>, dim3(grid), dim3(MVS_W * 32), 0, st, Xo, s, m, nb, sf2, part, Mo, ldm, rp, ngv, tpart, active); break;
-    }
+  switch (ker) {
+    case 0: launch_matvec<0, T>(Xo, s, m, sf2, part, Mo, ldm, rp, tpart, active, st); break;
+    case 1: launch_matvec<1, T>(Xo, s, m, sf2, part, Mo, ldm, rp, tpart, active, st); break;
+    default: launch_matvec<2, T>(Xo, s, m, sf2, part, Mo, ldm, rp, tpart, active, st); break;
   }
 }
 
@@ -1622,6 +1817,32 @@ void gemm_tn(const T* A, int lda, int na, const T* B, int ldb, int nb, int K, do
     cudaGetLastError();
   }
   const size_t tile_elems = (size_t)na * nb;
+  if constexpr (sizeof(T) == 8) {
+    // about two blocks per SM: single columns per warp while that alone does not fill the GPU, then
+    // splits of K (at least 64 values each)
+    const int gx = cdiv(na, 32);
+    int cpw = 4;
+    while (cpw > 1 && gx * (int)cdiv(nb, G64_WARPS * cpw) < 2 * 152) cpw /= 2;
+    const int gy = cdiv(nb, G64_WARPS * cpw);
+    int nsplit = std::max(1, std::min({2 * 152 / (gx * gy), K / 64, (int)std::min<size_t>(part_elems / tile_elems, 1 << 20)}));
+    const int chunk = std::max(32, (int)cdiv(cdiv(std::max(K, 1), nsplit), 32) * 32);
+    nsplit = std::max(1, (int)cdiv(std::max(K, 1), chunk));
+    double* out = nsplit > 1 ? part : nullptr;
+    const dim3 grid(gx, gy, nsplit);
+    const double *Ad = (const double*)A, *Bd = (const double*)B;
+    const int Kp = std::max(K, 0);
+    switch (cpw) {
+      case 1: k_gemm_tn_f64<1><<<grid, G64_WARPS * 32, 0, st>>>(Ad, lda, na, Bd, ldb, nb, Kp, chunk, out, alpha, beta, C, ldc); break;
+      case 2: k_gemm_tn_f64<2><<<grid, G64_WARPS * 32, 0, st>>>(Ad, lda, na, Bd, ldb, nb, Kp, chunk, out, alpha, beta, C, ldc); break;
+      default: k_gemm_tn_f64<4><<<grid, G64_WARPS * 32, 0, st>>>(Ad, lda, na, Bd, ldb, nb, Kp, chunk, out, alpha, beta, C, ldc); break;
+    }
+    note_launch();
+    if (out) {
+      k_reduce_splits<double><<<cdiv(tile_elems, 256), 256, 0, st>>>(part, nsplit, na, nb, alpha, beta, C, ldc);
+      note_launch();
+    }
+    return;
+  }
   int gx = cdiv(na, TN_T), gy = cdiv(nb, TN_T);
   int want = std::max(1, (int)(4 * 152 / std::max(1, gx * gy)));
   int chunk_min = 256;
@@ -1685,7 +1906,20 @@ void gemm_nn(int M, int N, int K, T alpha, const T* A, int lda, const TB* B, int
       return;
     cudaGetLastError();
   }
-  k_gemm_nn<T, TB><<<dim3(cdiv(M, NN_BM), cdiv(N, NN_BN)), 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); note_launch();
+  if constexpr (sizeof(T) == 8 && sizeof(TB) == 8) {
+    const int gx = cdiv(M, 32);
+    int cpw = 4;
+    while (cpw > 1 && gx * (int)cdiv(N, G64_WARPS * cpw) < 2 * 152) cpw /= 2;
+    const dim3 grid(gx, cdiv(N, G64_WARPS * cpw));
+    switch (cpw) {
+      case 1: k_gemm_nn_f64<1><<<grid, G64_WARPS * 32, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); break;
+      case 2: k_gemm_nn_f64<2><<<grid, G64_WARPS * 32, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); break;
+      default: k_gemm_nn_f64<4><<<grid, G64_WARPS * 32, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); break;
+    }
+    note_launch();
+  } else {
+    k_gemm_nn<T, TB><<<dim3(cdiv(M, NN_BM), cdiv(N, NN_BN)), 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); note_launch();
+  }
 }
 
 void gemm_small_f64(int ta, int tb, int M, int N, int K, double alpha, const double* A, int lda, const double* B,
