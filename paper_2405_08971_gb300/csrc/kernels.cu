@@ -1,6 +1,5 @@
 // SIMT kernels of the CAKF/CAKS hot path (FP32 and FP64 instantiations):
 //   - Gram matvec of the CG loop:  part[p][i] = sum_{j in split p} k(xo_i, xo_j) s_j
-//   - Gram x block (plain SIMT path): Out = K(Xr, Xc) B, evaluated tile by tile, never stored
 //   - tall-skinny GEMMs (split-K transposed products, tiled NN products)
 //   - the CG / Gram-Schmidt bookkeeping of the iterative update step
 //   - gathers, scatters and row epilogues of the filter and smoother.
@@ -752,71 +751,6 @@ __global__ void k_cg_init(const double* __restrict__ y, const double* __restrict
   }
   double sq = block_sum(val * val);
   if (threadIdx.x == 0) atomicAdd(r0sq, sq);
-}
-
-// ------------------------------------------------------------------------------------------
-// Plain SIMT Gram x block:  Out[i, c] = sum_j k(xr_i, xc_j) B[j, c]   (Out, B column-major)
-constexpr int GB_BM = 64, GB_BN = 64, GB_BK = 32, GB_THREADS = 256;
-
-template <int KER, class T, bool DER = false>
-__global__ void __launch_bounds__(GB_THREADS)
-k_gram_block_simt(const C4<T>* __restrict__ Xr, int nr, const C4<T>* __restrict__ Xc, int nc,
-                  const T* __restrict__ B, int ldb, int width, T sf2, T* __restrict__ Out, int ldo) {
-  __shared__ T Ks[GB_BK][GB_BM + 1];
-  __shared__ T Bs[GB_BK][GB_BN + 1];
-  __shared__ C4<T> xr[GB_BM];
-  const int r0 = blockIdx.x * GB_BM, n0 = blockIdx.y * GB_BN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // 16 x 16 threads, 4 x 4 outputs each
-  if (threadIdx.x < GB_BM) {
-    int rr = r0 + threadIdx.x;
-    if (rr < nr) xr[threadIdx.x] = Xr[rr]; else { C4<T> z; z.x = z.y = z.z = T(1e30); z.w = 0; xr[threadIdx.x] = z; }
-  }
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  __syncthreads();
-  for (int k0 = 0; k0 < nc; k0 += GB_BK) {
-    // kernel tile 64 x 32: 2048 values, 8 per thread
-    for (int e = threadIdx.x; e < GB_BM * GB_BK; e += GB_THREADS) {
-      int rr = e % GB_BM, kk = e / GB_BM;
-      int col = k0 + kk;
-      T kvv = T(0);
-      if (col < nc && r0 + rr < nr)
-        kvv = DER ? kval_dlogl<KER>(dist2(xr[rr], Xc[col]), sf2) : kval<KER>(dist2(xr[rr], Xc[col]), sf2);
-      Ks[kk][rr] = kvv;
-    }
-    for (int e = threadIdx.x; e < GB_BK * GB_BN; e += GB_THREADS) {
-      int kk = e % GB_BK, cc = e / GB_BK;
-      int col = k0 + kk, c = n0 + cc;
-      Bs[kk][cc] = (col < nc && c < width) ? B[(size_t)c * ldb + col] : T(0);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < GB_BK; ++kk) {
-      T ka[4], bb[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) ka[a] = Ks[kk][ty + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bb[b] = Bs[kk][tx + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(ka[a], bb[b], acc[a][b]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    int rr = r0 + ty + 16 * a;
-    if (rr >= nr) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      int c = n0 + tx + 16 * b;
-      if (c < width) Out[(size_t)c * ldo + rr] = acc[a][b];
-    }
-  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1697,31 +1631,6 @@ void gram_matvec(int ker, const C4<T>* Xo, const T* s, int m, T sf2, T* part, co
 }
 
 template <class T>
-void gram_block_simt(int ker, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, const T* B, int ldb, int width,
-                     T sf2, T* Out, int ldo, cudaStream_t st) {
-  if (nr <= 0 || width <= 0) return;
-  dim3 grid(cdiv(nr, GB_BM), cdiv(width, GB_BN));
-  switch (ker) {
-    case 0: k_gram_block_simt<0, T><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-    case 1: k_gram_block_simt<1, T><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-    default: k_gram_block_simt<2, T><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-  }
-}
-
-// Out = dK/dlog(l_x) (Xr, Xc) B  (the derivative Gram matrix, never stored)
-template <class T>
-void gram_block_dlogl_simt(int ker, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, const T* B, int ldb, int width,
-                           T sf2, T* Out, int ldo, cudaStream_t st) {
-  if (nr <= 0 || width <= 0) return;
-  dim3 grid(cdiv(nr, GB_BM), cdiv(width, GB_BN));
-  switch (ker) {
-    case 0: k_gram_block_simt<0, T, true><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-    case 1: k_gram_block_simt<1, T, true><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-    default: k_gram_block_simt<2, T, true><<<grid, GB_THREADS, 0, st>>>(Xr, nr, Xc, nc, B, ldb, width, sf2, Out, ldo); note_launch(); break;
-  }
-}
-
-template <class T>
 void cg_combine(const T* part, int nsplit, const T* s, T sn2, const T* Mo, int ldm, int r, const T* t, T a2, int m,
                 T* g, const T* V, int ldv, int j, const T* r0, const T* v, T* dpart1, const int* active,
                 cudaStream_t st) {
@@ -2310,10 +2219,6 @@ void check_finite(const double* x, size_t n, int* err, cudaStream_t st) {
   template void gather_coords<T>(const C4<T>*, const int*, int, C4<T>*, cudaStream_t);                          \
   template void gram_matvec<T>(int, const C4<T>*, const T*, int, T, T*, const T*, int, int, T*, const int*,     \
                                cudaStream_t);                                                                   \
-  template void gram_block_simt<T>(int, const C4<T>*, int, const C4<T>*, int, const T*, int, int, T, T*, int,    \
-                                   cudaStream_t);                                                                \
-  template void gram_block_dlogl_simt<T>(int, const C4<T>*, int, const C4<T>*, int, const T*, int, int, T, T*,   \
-                                         int, cudaStream_t);                                                     \
   template void cg_combine<T>(const T*, int, const T*, T, const T*, int, int, const T*, T, int, T*, const T*,     \
                               int, int, const T*, const T*, T*, const int*, cudaStream_t);                       \
   template void cg_upd1<T>(int, const T*, double*, T*, T*, int, const T*, const T*, int, T*,                    \
