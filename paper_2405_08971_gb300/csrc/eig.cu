@@ -2,13 +2,14 @@
 // of the (r+i) x (r+i) Gram of the downdate factor).
 //
 //   1. Householder tridiagonalisation, one cooperative kernel; the blocks exchange each column's
-//      matvec and pivot column through epoch-tagged words (no grid barrier), with bounded polling.
+//      matvec and pivot column through write-once words (no grid barrier), with bounded polling.
 //   2. Divide and conquer on the tridiagonal (Cuppen's tearing; deflation of small z components and
 //      close poles by Givens rotations; secular roots by a two-pole rational model guarded by
 //      bisection; eigenvectors from the Loewner-corrected z (Gu-Eisenstat), which keeps them
 //      orthogonal without re-orthogonalisation).
 //   3. Back-transformation of the wanted columns through the Householder reflectors.
 // All arithmetic is FP64; only the final eigenvector block is stored in the caller's precision.
+#include <type_traits>
 #include <vector>
 #include <map>
 #include <mutex>
@@ -36,28 +37,40 @@ __device__ __forceinline__ double nr_rcp(double x) {
   return r;
 }
 
-// Per-step exchange without a grid barrier: every word a block publishes for step k carries the
-// step's epoch (k mod 4), and the consumers poll the words themselves until all carry the epoch they
-// wait for.  A value x travels as a pair of 8-byte words: hi is the bit pattern of x with its two
-// lowest bits replaced by the epoch, lo holds those two original bits in bits 0-1 and the epoch in
-// bits 2-3.  The reader accepts the pair when both epochs match and rebuilds x bit for bit from hi
-// and lo with integer operations (no FP64 arithmetic, nothing lost).  Each 8-byte word is written
-// and read as one access, so a reader sees either the old or the new word; the data dependence of
-// the recursion (no block can publish step k + 2 before every block has published step k + 1, which
-// needs step k consumed) makes two buffers enough.
-__device__ __forceinline__ int epoch_hi(long long h) { return (int)(h & 3LL); }
-__device__ __forceinline__ int epoch_lo(long long l) { return (int)((l >> 2) & 3LL); }
-__device__ __forceinline__ void publish_pair(double* p, double x, int ep) {
-  const long long b = __double_as_longlong(x);
-  const long long hi = (b & ~3LL) | (long long)ep;
-  const long long lo = (b & 3LL) | ((long long)ep << 2);
-  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(hi), "l"(lo) : "memory");
+// sqrt(x) and 1 / sqrt(x), and 1 / x, for normal x > 0, from the hardware's approximations y (about 20 bits,
+// full FP64 exponent range) and one third-order step: with e = 1 - x y^2 the factor 1 + e / 2 + 3 e^2 / 8
+// (the binomial series of (1 - e)^(-1/2)), with e = 1 - x y the factor 1 + e + e^2.  Both remainders are
+// below 2^-56.
+__device__ __forceinline__ void fast_sqrt(double x, double& sq, double& rs) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y;
+  const double e = fma(-g, y, 1.0);
+  const double f = e * fma(0.375, e, 0.5);
+  sq = fma(g, f, g);
+  rs = fma(y, f, y);
 }
-__device__ __forceinline__ void ld_pair(const double* p, long long& hi, long long& lo) {
-  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(hi), "=l"(lo) : "l"(p) : "memory");
+__device__ __forceinline__ double fast_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double pair_value(long long hi, long long lo) {
-  return __longlong_as_double((hi & ~3LL) | (lo & 3LL));
+
+// Exchange between the blocks of the tridiagonalisation without barriers or flags: every step has its own
+// slots, filled with the sentinel (all bits set: a NaN that arithmetic only passes on from an operand, and
+// td_load() replaces it in the input) before the kernel starts; an owner writes each 8-byte word once, and a consumer polls the words it needs
+// until none is the sentinel.  Each word is written and read as one access.
+constexpr unsigned long long kSlotEmpty = ~0ULL;
+__device__ __forceinline__ void publish(double* p, double x) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(__double_as_longlong(x)) : "memory");
+}
+__device__ __forceinline__ double td_load(const double* p) {
+  const double x = *p;
+  return __isnan(x) ? __longlong_as_double(0x7FF8000000000000LL) : x;
+}
+__device__ __forceinline__ void ld_slot(const double* p, unsigned long long& s, unsigned long long& c) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(s), "=l"(c) : "l"(p) : "memory");
 }
 __device__ __forceinline__ int ld_relaxed_int(const int* p) {
   int v;
@@ -66,60 +79,225 @@ __device__ __forceinline__ int ld_relaxed_int(const int* p) {
 }
 constexpr long long kPollLimit = 4000000LL;
 
+// Power of two that brings a matrix of largest magnitude amax (its bit pattern) to about 1, and its inverse;
+// 1 for a zero, denormal or non-finite matrix.
+__device__ __forceinline__ void pow2_scale(unsigned long long amax, double& sc, double& inv) {
+  const long long ex = (long long)(amax >> 52) & 0x7FF;
+  if (ex == 0 || ex > 2045) { sc = inv = 1.0; return; }
+  sc = __longlong_as_double((2046 - ex) << 52);
+  inv = __longlong_as_double(ex << 52);
+}
+
+// *amax = largest magnitude of the N x N matrix, as a bit pattern (zero before the launch)
+__global__ void __launch_bounds__(256)
+k_absmax(const double* __restrict__ A, int lda, int N, unsigned long long* __restrict__ amax) {
+  unsigned long long m = 0;
+  for (int j = blockIdx.x; j < N; j += gridDim.x)
+    for (int t = threadIdx.x; t < N; t += blockDim.x) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(A[(size_t)j * lda + t]) & 0x7FFFFFFFFFFFFFFFULL;
+      m = b > m ? b : m;
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, m, o);
+    m = x > m ? x : m;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(amax, m);
+}
 
 // ---------------------------------------------------------------------------------- tridiagonal
-// Householder tridiagonalisation (lower), one exchange of epoch-tagged words per column.  Columns
-// of the trailing block are owned by (block, warp) round-robin and stay resident in shared memory.
-// At step k every block reads p_k = tau_k A22 v_k and the pre-update pivot column k+1 from double
-// buffers the owners published during step k-1, forms w_k = p_k - 1/2 tau_k (p_k . v_k) v_k, the
-// updated pivot column and from it v_{k+1}, tau_{k+1} (all redundantly, so nothing else has to be
-// exchanged); the owners then update their columns and, in the same pass, compute their entries of
-// p_{k+1} and publish the next pivot column.  Reflector v_k is stored in column k below the
-// subdiagonal (v_k[0] = 1).  Block reductions go through shared memory and one warp (the FP64 pipe
-// is narrow on this GPU, so a shuffle tree in every warp would cost more than the data it sums).
-constexpr int TD_THREADS = 160;      // warp 0: reductions and Householder scalars; warps 1-4: columns
-constexpr int TD_MAX_SLOTS = 64;     // owned columns per block
-constexpr int TD_BATCH = 5;     // exchange entries a thread polls with their loads in flight together
+// Householder tridiagonalisation (lower).  Columns of the trailing block are owned by blocks round-robin
+// (column j: block j % G, slot j / G) and stay in shared memory; vectors along the trailing rows are held
+// by every block.  With c the first column of the trailing block B_k (rows k..), x = c1^2 + sigma, sigma =
+// sum_{t>=2} c_t^2, s = sqrt(x) and gamma = c1 + sign(c1) s, the reflector is I - tau v v^T on rows k + 1..
+// with v = (gamma, c_2, c_3, ...), tau = 1 / (s |gamma|) -- unscaled, so that
+//   p = B v = S + gamma C,   S_j = sum_{t>=1} B_{tj} v_t,  C = column k + 1 of B (rows k + 1..),
+// where S depends on c but not on sigma.  Since C is also row k + 1, p_0 = C . v, so q = p . v =
+// sum_{t>=1} S_t v_t + gamma (S_0 + p_0) needs no p.  Step k:
+//   warps 0-3  poll S and C, with the partial sums of S_t v_t on the way                    -- barrier
+//   warp 4     their sum; warps 0-3 form p and C - gamma tau p                                -- barrier
+//   warps 0-3  next c = C - gamma tau p - e3 v, e3 = tau (p_0 - gamma tau q)                   -- barrier
+//   warps 0-3  owned columns: B_tj -= v_t a_j + p_t b_j  (a_j = tau (p_j - tau q v_j), b_j = tau v_j) and, in
+//              the same pass, the next S_j; publish S_j, and the next pivot column as it is formed
+//   warp 4     sigma and the scalars of the next reflector, which nobody waits for before the next
+//              exchange has arrived
+// What bounds it: an FP64 instruction holds its quarter of the SM (one warp here) for 64 cycles, 77 when all
+// four are busy, whatever its lanes or their predicates, and a shuffle level of an FP64 sum 126.  So warps
+// take whole columns, sums go through integers (warp_sum_int: 460 cycles instead of 690), loops have no padded
+// turns, and warp 4 takes what is not on the chain.  Per column at N = 576, about: column pass 2,700 cycles
+// (three FP64 instructions per 32 entries), its sum 460, exchange 1,800 (store to L2, load) plus the wait for
+// the slowest block, block sum 600, the next c 400.  The words go to REP replicas (a block polls one of
+// them): 152 blocks polling the same lines queue at their L2 slices (N = 576: 2.73 ms with one replica, 2.52
+// with 4, 2.66 with 16).  N = 576 takes 2.52 ms, N = 288 0.94 ms; 2.79 and 1.15 ms with scaled reflectors,
+// whose scalars stood between the column pass and the exchange, shuffle sums and pairs of 16 bytes a value.
+// The matrix is scaled by a power of two, which keeps the unscaled reflectors' products in range; a column
+// below 1e-140 of the matrix is left alone (tau = 0).  v and tau are kept for the back-transformation, v
+// below the subdiagonal of column k.
+constexpr int TD_VEC = 128;                  // threads of the vector work: 4 warps, the owner warps
+constexpr int TD_THREADS = TD_VEC + 32;      // warp 4: block reductions and scalars
+constexpr int TD_MAX_SLOTS = 64;             // owned columns per block
+// Replicas of the exchange slots (template parameter REP): 4 up to order 1,024, one above, where the slots
+// (8 N^2 bytes a replica) would begin to count among the workspace.
+inline int td_replicas(int N) { return N <= 1024 ? 4 : 1; }
+constexpr int TD_BATCH = 5;                  // exchange entries a thread polls with their loads in flight together
 
-// Householder scalars for x (x[0] = alpha, sum of the squares of x[1..] = sigma): H x = beta e_1,
-// H = I - tau v v^T with v[0] = 1 and v[t] = x[t] * scal.
-__device__ __forceinline__ void house_scalars(double alpha, double sigma, double& tau, double& beta, double& scal) {
-  if (sigma == 0.0) { tau = 0.0; beta = alpha; scal = 0.0; return; }
-  beta = -copysign(sqrt(alpha * alpha + sigma), alpha);
-  tau = (beta - alpha) * nr_rcp(beta);
-  scal = nr_rcp(alpha - beta);
+__host__ __device__ inline size_t td_slot_offset(int N, int k) {   // slots (S, C) of step k: N - 1 - k of them
+  return (size_t)k * (size_t)(N - 1) - (size_t)k * (size_t)(k - 1) / 2;
 }
 
-// Sum of red[0 .. blockDim.x) by warp 0 (called by warp 0 only); the result is in every lane.
-__device__ __forceinline__ double warp0_sum(const double* red) {
-  const int lane = threadIdx.x & 31;
+// Sum of NV doubles per lane over the warp, in every lane, in integer arithmetic.  A shuffle tree costs 126
+// cycles a level here (an FP64 operation holds its quarter of the SM for 64 cycles, however few lanes
+// take part), integer instructions about 4; so the mantissas are aligned to the largest exponent as three limbs
+// of LB bits (72 or 78 bits in all, 19 or more below the largest value's last place), the limbs are
+// summed by redux.sync, and the sum is rounded once: more accurate than the tree.  Non-finite or nearly
+// overflowing values take the tree.
+template <int NV>
+__device__ __forceinline__ double warp_sum_int(const double (&x)[NV]) {
+  static_assert(NV == 1 || NV == 4, "limbs of NV * 32 values must fit 31 bits");
+  constexpr int LB = NV == 1 ? 26 : 24, GUARD = 3 * LB - 53;
+  constexpr unsigned MASK = (1u << LB) - 1u;
+  unsigned long long m[NV];
+  int ex[NV], sg[NV];
+  unsigned emax = 0;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const long long b = __double_as_longlong(x[i]);
+    ex[i] = (int)((b >> 52) & 0x7FF);
+    sg[i] = (int)(b >> 63);
+    m[i] = ex[i] ? ((unsigned long long)b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL : 0ULL;
+    emax = max(emax, (unsigned)ex[i]);
+  }
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  if (emax > 2000u) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) t += x[i];
+    return warp_sum(t);
+  }
+  int hi = 0, mid = 0, lo = 0;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int d = min((int)emax - ex[i], 63);
+    const int h = (int)(m[i] >> min(53 - LB + d, 63));
+    const int md = (int)((unsigned)(m[i] >> min(53 - 2 * LB + d, 63)) & MASK);
+    const int l = (int)((unsigned)(d >= GUARD ? m[i] >> (d - GUARD) : m[i] << (GUARD - d)) & MASK);
+    hi += (h ^ sg[i]) - sg[i];
+    mid += (md ^ sg[i]) - sg[i];
+    lo += (l ^ sg[i]) - sg[i];
+  }
+  hi = __reduce_add_sync(0xffffffffu, hi);
+  mid = __reduce_add_sync(0xffffffffu, mid);
+  lo = __reduce_add_sync(0xffffffffu, lo);
+  // hi 2^(2 LB) + mid 2^LB + lo in units of 2^(emax - 1075 - GUARD), as a 64-bit integer times 2^sh
+  const long long T = ((long long)hi << LB) + mid;
+  const int sh = max(0, LB + 2 - __clzll(T < 0 ? -T : T));
+  const long long X = (T << (LB - sh)) + (lo >> sh);
+  const double r = __ll2double_rn(X);
+  const long long rb = __double_as_longlong(r);
+  const int er = (int)((rb >> 52) & 0x7FF) + (int)emax - 1075 - GUARD + sh;
+  if (X == 0 || er <= 0) return 0.0;
+  return __longlong_as_double((rb & ~(0x7FFLL << 52)) | ((long long)er << 52));
+}
+
+// Sum of red[0 .. TD_VEC) by one warp; the result is in every lane.
+__device__ __forceinline__ double td_sum(const double* red) {
+  const double2* r = reinterpret_cast<const double2*>(red) + 2 * (threadIdx.x & 31);
+  const double2 a = r[0], b = r[1];
+  const double x[4] = {a.x, a.y, b.x, b.y};
+  return warp_sum_int<4>(x);
+}
+__device__ __forceinline__ double td_warp_sum(double v) {
+  const double x[1] = {v};
+  return warp_sum_int<1>(x);
+}
+
+struct TdScalars { double gamma, gt, tau, beta; };   // gt = gamma tau; beta: the new subdiagonal entry
+__device__ __forceinline__ TdScalars td_scalars(double c1, double sigma) {
+  TdScalars r;
+  const double x = fma(c1, c1, sigma);
+  // (comparisons on the bit patterns: they stay off the FP64 pipe)
+  if (__double_as_longlong(sigma) == 0 || __double_as_longlong(x) < __double_as_longlong(1e-280)) {
+    r.gamma = 1.0; r.gt = r.tau = 0.0; r.beta = c1;
+    return r;
+  }
+  double sq, rs;
+  fast_sqrt(x, sq, rs);
+  const double ss = copysign(sq, c1);
+  r.gamma = c1 + ss;
+  r.beta = -ss;
+  r.gt = copysign(rs, c1);
+  r.tau = rs * fast_rcp(fabs(r.gamma));
+  return r;
+}
+
+// With q' = sum_{t>=1} S_t v_t, q = q' + gamma (2 S_0 + gamma C_0) and p_0 = S_0 + gamma C_0:
+//   e3 = tau (p_0 - gamma tau q) = (bc[3] S_0 + bc[4] C_0) - bc[5] q',   tau q = (2 bc[1] S_0 + bc[6] C_0) + tau q'
+__device__ __forceinline__ void td_coefficients(const TdScalars& h, double* bc) {
+  const double e2 = h.tau * h.gt, tg = h.gamma * h.gt;
+  bc[0] = h.gamma; bc[1] = h.gt; bc[2] = h.tau;
+  bc[3] = fma(-2.0 * e2, h.gamma, h.tau);
+  bc[4] = fma(-h.gt, tg, h.gt);
+  bc[5] = e2;
+  bc[6] = tg;
+}
+
+// Column pass of one owned column (col, v, p, cn from local row 0 = row k + 1): rows t >= 1 get the rank-2
+// update, and the sum over t >= 2 of the updated entries times cn is returned (the lane's part; cn[1] counts
+// as zero).  The next entry's operands are read while the current one's three dependent operations run (64
+// to 77 cycles each).  With out, entry t also goes to the next step's slots t - 1 (as its C).
+template <int REP>
+__device__ __forceinline__ double td_column(double* col, const double* v, const double* p, const double* cn, double aj,
+                                            double bj, int L, int lane, double* out, size_t rep) {
   double s = 0.0;
-  for (int i = lane; i < (int)blockDim.x; i += 32) s += red[i];
-  return warp_sum(s);
+  int t = 1 + lane, i = min(t, L - 1);
+  double xc = col[i], xv = v[i], xp = p[i], xn = i >= 2 && t < L ? cn[i] : 0.0;
+#pragma unroll 1
+  for (int b = 1; b < L; b += 32) {
+    double x = fma(-xp, bj, xc);
+    const int tn = t + 32;
+    i = min(tn, L - 1);
+    xc = col[i];
+    xp = p[i];
+    x = fma(-xv, aj, x);
+    const double cv = xn;
+    xv = v[i];
+    xn = tn < L ? cn[i] : 0.0;
+    if (t < L) {
+      col[t] = x;
+      if (out) {
+#pragma unroll
+        for (int r = 0; r < REP; ++r) publish(out + r * rep + 2 * (t - 1) + 1, x);
+      }
+    }
+    s = fma(x, cv, s);
+    t = tn;
+  }
+  return s;
 }
 
+template <int REP>
 __global__ void __launch_bounds__(TD_THREADS)
 k_tridiag(double* __restrict__ A, int lda, int N, double* __restrict__ d, double* __restrict__ e,
-          double* __restrict__ tau, double* __restrict__ Pbuf, double* __restrict__ Cbuf, int* err,
+          double* __restrict__ tau, double* __restrict__ slots, const unsigned long long* __restrict__ amax, int* err,
           long long poll_limit) {
-  extern __shared__ double sm[];
-  // sm[0, N) and sm[N, 2N): v_k and v_{k+1}, swapped every step
-  double* w = sm + 2 * N;           // w_k
-  double* c = sm + 3 * N;           // updated pivot column k+1
-  double* cols = sm + 4 * N;        // owned columns (full length N), resident for the whole reduction
-  __shared__ double red[TD_THREADS];
-  __shared__ double bc[4];          // broadcast scalars
-  __shared__ double colS[TD_MAX_SLOTS], colF[TD_MAX_SLOTS];   // owner warps' parts of p_{k+1}
-  const int G = gridDim.x, tid = threadIdx.x, TB = blockDim.x;
-  const int warp = tid >> 5, lane = tid & 31, nw = TB >> 5;
-  const int nslot = (N + G - 1) / G;   // column j lives in block j % G, slot j / G
-  // The block owning the last column writes the outputs (d, e, tau, reflectors): it publishes
-  // exchange words at every step.  Every other block leaves once it owns no column >= k + 2 (it
-  // would publish nothing more), so each block still reading step k's words publishes words for
-  // step k + 1 -- which is what keeps two exchange buffers safe: no block can publish step k + 2
-  // before every running block has consumed step k.
-  const int ob = (N - 1) % G;
+  extern __shared__ __align__(16) double sm[];
+  // c of three steps (a step's, the next one's, and the one that the words of the next exchange go to while
+  // slower warps still read this step's) and p of two; v of a step is its c from entry 1 on
+  double* cbuf = sm;
+  double* pbuf = sm + 3 * N;
+  double* cols = sm + 5 * N;        // owned columns (full length N)
+  __shared__ __align__(16) double red[TD_VEC];
+  // broadcast scalars: gamma, gamma tau, tau and the coefficients of (6) below, written by warp 4; q' (warp 4);
+  // S_0, C_0 (thread 0); e1, h1 (warp 3)
+  __shared__ double bc[12];
+  __shared__ double cS[TD_MAX_SLOTS], cB[TD_MAX_SLOTS], cT[TD_MAX_SLOTS];   // owned columns: S_j, tau v_j, tau p_j
+  const int G = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nslot = (N + G - 1) / G;
+  const int ob = (N - 1) % G;       // the block that owns the last column writes the outputs
   const int maxcol = (int)blockIdx.x + G * ((N - 1 - (int)blockIdx.x) / G);
+  const size_t rep = (size_t)N * (N + 1);     // words of a replica of the slots
+  double msc, minv;
+  pow2_scale(*amax, msc, minv);
   if (N <= 2) {
     if (blockIdx.x == 0 && tid == 0) {
       d[0] = A[0];
@@ -130,191 +308,183 @@ k_tridiag(double* __restrict__ A, int lda, int N, double* __restrict__ d, double
   for (int q = 0; q < nslot; ++q) {
     const int j = q * G + blockIdx.x;
     if (j >= N) break;
-    for (int t = tid; t < N; t += TB) cols[(size_t)q * N + t] = A[(size_t)j * lda + t];
+    for (int t = tid; t < N; t += TD_THREADS) cols[(size_t)q * N + t] = msc * td_load(A + (size_t)j * lda + t);
   }
-  // ---- prologue: v_0 from column 0; p_0; publish column 1
-  double tk, bk;
+  // ---- c_0 = column 0, its scalars; S and C of step 0
+  TdScalars h = {};                 // warp 4: the current reflector's scalars
   {
-    const int L = N - 1;
-    double part = 0.0;
-    for (int t = tid; t < L; t += TB) {
-      const double x = A[1 + t];
-      c[t] = x;
-      if (t >= 1) part = fma(x, x, part);
-    }
-    red[tid] = part;
+    for (int t = tid; t < N; t += TD_THREADS) cbuf[t] = msc * td_load(A + t);
     __syncthreads();
-    if (warp == 0) {
-      const double sigma = warp0_sum(red);
+    if (warp == 4) {
+      double part = 0.0;
+      for (int t = 2 + lane; t < N; t += 32) part = fma(cbuf[t], cbuf[t], part);
+      const double sigma = td_warp_sum(part);
+      h = td_scalars(cbuf[1], sigma);
+      __syncwarp();
       if (lane == 0) {
-        double ta, be, sc;
-        house_scalars(c[0], sigma, ta, be, sc);
-        bc[0] = ta; bc[1] = be; bc[2] = sc;
-      }
-    }
-    __syncthreads();
-    tk = bc[0]; bk = bc[1];
-    const double sc = bc[2];
-    double* v = sm;
-    for (int t = tid; t < L; t += TB) v[t] = (t == 0) ? 1.0 : c[t] * sc;
-    __syncthreads();
-    for (int q = warp; q < nslot; q += nw) {
-      const int j = q * G + blockIdx.x;
-      if (j < 1 || j >= N) continue;
-      const double* col = cols + (size_t)q * N + 1;
-      double acc = 0.0;
-      for (int t = lane; t < L; t += 32) acc = fma(col[t], v[t], acc);
-      acc = warp_sum(acc);
-      if (lane == 0) publish_pair(Pbuf + 2 * (j - 1), tk * acc, 0);
-      if (j == 1) for (int t = lane; t < L; t += 32) publish_pair(Cbuf + 2 * t, col[t], 0);
-    }
-    if (blockIdx.x == ob && tid == 0) d[0] = A[0];
-    __syncthreads();
-  }
-  for (int k = 0; k + 2 < N; ++k) {
-    if ((int)blockIdx.x != ob && maxcol < k + 2) return;
-    const int L = N - k - 1;
-    const double* Pk = Pbuf + (size_t)(k & 1) * 2 * N;
-    double* Pn = Pbuf + (size_t)((k + 1) & 1) * 2 * N;
-    const double* Ck = Cbuf + (size_t)(k & 1) * 2 * N;
-    double* Cn = Cbuf + (size_t)((k + 1) & 1) * 2 * N;
-    const double* v = sm + (size_t)(k & 1) * N;
-    double* v2 = sm + (size_t)((k + 1) & 1) * N;
-    const bool next = (k + 3 < N);      // a reflector for column k+1 exists
-    // (1) p_k . v_k; the pivot column C_k is fetched in the same pass (into c).  Each thread polls
-    // its entries of P_k and C_k, up to TD_BATCH of them with their loads in flight together, until
-    // all carry epoch k mod 4 (bounded; a timeout or another block's error ends the kernel).
-    const int ek = k & 3;
-    double part = 0.0;
-    bool ok = true;
-    for (int t0 = tid; t0 < L && ok; t0 += TB * TD_BATCH) {
-      long long ph[TD_BATCH], pl[TD_BATCH], ch[TD_BATCH], cl[TD_BATCH];
-      unsigned pend = 0;
-#pragma unroll
-      for (int u = 0; u < TD_BATCH; ++u)
-        if (t0 + u * TB < L) pend |= 1u << u;
-      long long spins = 0;
-      while (pend) {
-#pragma unroll
-        for (int u = 0; u < TD_BATCH; ++u)
-          if ((pend >> u) & 1u) {
-            const int t = t0 + u * TB;
-            ld_pair(Pk + 2 * t, ph[u], pl[u]);
-            ld_pair(Ck + 2 * t, ch[u], cl[u]);
-          }
-#pragma unroll
-        for (int u = 0; u < TD_BATCH; ++u)
-          if (((pend >> u) & 1u) && epoch_hi(ph[u]) == ek && epoch_lo(pl[u]) == ek && epoch_hi(ch[u]) == ek &&
-              epoch_lo(cl[u]) == ek)
-            pend &= ~(1u << u);
-        if (!pend) break;
-        if (++spins > poll_limit) { atomicExch(err, kErrTimeout); ok = false; break; }
-        if ((spins & 255) == 0 && ld_relaxed_int(err)) { ok = false; break; }
-      }
-      if (!ok) break;
-#pragma unroll
-      for (int u = 0; u < TD_BATCH; ++u) {
-        const int t = t0 + u * TB;
-        if (t < L) {
-          const double pt = pair_value(ph[u], pl[u]), ct = pair_value(ch[u], cl[u]);
-          c[t] = ct;
-          w[t] = pt;
-          part = fma(pt, v[t], part);
-        }
-      }
-    }
-    red[tid] = part;
-    if (!__syncthreads_and(ok)) return;
-    if (warp == 0) {
-      const double pv = warp0_sum(red);
-      if (lane == 0) {
-        const double kc = 0.5 * tk * pv;
-        bc[0] = kc;
-        bc[1] = w[0] - kc;               // w_k[0] (v_k[0] = 1)
-      }
-    }
-    __syncthreads();
-    const double kc = bc[0], w0 = bc[1];
-    // (2) w_k and the updated pivot column c = C_k - v w0 - w v0 (v0 = 1); sum of squares of c[2..]
-    part = 0.0;
-    for (int t = tid; t < L; t += TB) {
-      const double wt = fma(-kc, v[t], w[t]);
-      w[t] = wt;
-      const double ct = fma(-v[t], w0, c[t]) - wt;
-      c[t] = ct;
-      if (t >= 2) part = fma(ct, ct, part);
-    }
-    red[tid] = part;
-    __syncthreads();
-    // (3) warp 0 sums sigma and forms the Householder scalars of column k+1 while the owner warps
-    // update their columns, A22 -= v w^T + w v^T (rows k+1..), publish the next pivot column
-    // (column k+2) as it is formed, and sum their parts of p_{k+1} = tau_{k+1} A22 v_{k+1}:
-    // nv[1] + scn * sum_{t >= 2} nv[t] c[t]  (v_{k+1}[0] = 1, v_{k+1}[t-1] = c[t] scn), finished
-    // once scn is known.
-    if (warp == 0) {
-      const double sigma = warp0_sum(red);
-      if (lane == 0) {
-        double ta = 0.0, be = 0.0, sc = 0.0;
-        if (next) house_scalars(c[1], sigma, ta, be, sc);
-        bc[2] = ta; bc[3] = be; bc[0] = sc;
-        if (blockIdx.x == ob) {
-          d[k + 1] = c[0];
-          e[k] = bk;
-          tau[k] = tk;
-          if (!next) { e[k + 1] = c[1]; tau[k + 1] = 0.0; }
-        }
+        if (blockIdx.x == ob) d[0] = minv * cbuf[0];
+        td_coefficients(h, bc);
+        cbuf[1] = h.gamma;
       }
     } else {
-      for (int q = warp - 1; q < nslot; q += nw - 1) {
+      for (int q = warp; q < nslot; q += 4) {
         const int j = q * G + blockIdx.x;
-        if (j < k + 1 || j >= N) continue;
-        const int tj = j - (k + 1);
-        double* col = cols + (size_t)q * N + k + 1;
-        const double vj = v[tj], wj = w[tj];
-        const bool publish = next && tj == 1;       // column k+2 becomes the next pivot column
-        double a0 = 0.0, a1 = 0.0, first = 0.0;
-        for (int t = lane; t < L; t += 64) {
-          const double nv = fma(-v[t], wj, fma(-w[t], vj, col[t]));
-          col[t] = nv;
-          if (publish && t >= 1) publish_pair(Cn + 2 * (t - 1), nv, (k + 1) & 3);
-          if (t >= 2) a0 = fma(nv, c[t], a0);
-          else if (t == 1) first = nv;
-          const int t2 = t + 32;
-          if (t2 < L) {
-            const double nv2 = fma(-v[t2], wj, fma(-w[t2], vj, col[t2]));
-            col[t2] = nv2;
-            if (publish) publish_pair(Cn + 2 * (t2 - 1), nv2, (k + 1) & 3);
-            a1 = fma(nv2, c[t2], a1);
-          }
-        }
-        const double S = warp_sum(a0 + a1);
-        const double F = warp_sum(first);
-        if (lane == 0) { colS[q] = S; colF[q] = F; }
-        if (k + 3 == N && j == N - 1) {                  // last diagonal entry (written by lane L-1)
-          __syncwarp();
-          if (lane == 0) d[N - 1] = col[L - 1];
-        }
+        if (j < 1 || j >= N) continue;
+        const double* col = cols + (size_t)q * N;
+        double acc = 0.0;
+        for (int t = 2 + lane; t < N; t += 32) acc = fma(col[t], cbuf[t], acc);
+        acc = td_warp_sum(acc);
+        if (lane == 0) cS[q] = acc;
+        if (lane < REP) publish(slots + lane * rep + 2 * (j - 1), acc);
+        if (j == 1)
+          for (int t = 1 + lane; t < N; t += 32)
+            for (int r = 0; r < REP; ++r) publish(slots + r * rep + 2 * (t - 1) + 1, col[t]);
       }
     }
-    __syncthreads();
-    const double tn = bc[2], bn = bc[3], scn = bc[0];
-    // (4) the owners publish their entries of p_{k+1} (lane 0 reads back its own colS, colF);
-    // every thread writes v_{k+1}
-    if (warp > 0 && lane == 0 && next) {
-      for (int q = warp - 1; q < nslot; q += nw - 1) {
+  }
+  for (int k = 0; k + 2 < N; ++k) {
+    // a block with no column to publish for step k + 1 has nothing left to do
+    if ((int)blockIdx.x != ob && maxcol < k + 2) return;
+    const int L = N - k - 1;
+    const double* in = slots + (blockIdx.x % REP) * rep + 2 * td_slot_offset(N, k);
+    double* out = slots + 2 * td_slot_offset(N, k + 1);
+    double* c = cbuf + (size_t)(k % 3) * N;          // c_k, with gamma in entry 1
+    double* cn = cbuf + (size_t)((k + 1) % 3) * N;   // c_{k+1}
+    double* pv = pbuf + (size_t)(k & 1) * N;
+    const double* v = c + 1;
+    const bool next = (k + 3 < N);            // a reflector for column k + 1 exists
+    // (1) poll this step's S and C (into pv and cn), and the partial sums of S_t v_t, t >= 1
+    bool ok = true;
+    if (warp < 4) {
+      for (int t0 = tid; t0 < L && ok; t0 += TD_VEC * TD_BATCH) {
+        unsigned long long bs[TD_BATCH], bcl[TD_BATCH];
+        unsigned pend = 0;
+#pragma unroll
+        for (int u = 0; u < TD_BATCH; ++u)
+          if (t0 + u * TD_VEC < L) pend |= 1u << u;
+        long long spins = 0;
+        while (pend) {
+#pragma unroll
+          for (int u = 0; u < TD_BATCH; ++u)
+            if ((pend >> u) & 1u) ld_slot(in + 2 * (t0 + u * TD_VEC), bs[u], bcl[u]);
+#pragma unroll
+          for (int u = 0; u < TD_BATCH; ++u)
+            if (((pend >> u) & 1u) && bs[u] != kSlotEmpty && bcl[u] != kSlotEmpty) {
+              pend &= ~(1u << u);
+              pv[t0 + u * TD_VEC] = __longlong_as_double((long long)bs[u]);
+              cn[t0 + u * TD_VEC] = __longlong_as_double((long long)bcl[u]);
+            }
+          if (!pend) break;
+          if (++spins > poll_limit) { atomicExch(err, kErrTimeout); ok = false; break; }
+          if ((spins & 255) == 0 && ld_relaxed_int(err)) { ok = false; break; }
+        }
+      }
+      double q0 = 0.0;
+      if (ok) {
+        if (tid == 0) { bc[8] = pv[0]; bc[9] = cn[0]; }
+#pragma unroll 1
+        for (int t = tid ? tid : TD_VEC; t < L; t += TD_VEC) q0 = fma(pv[t], v[t], q0);
+      }
+      red[tid] = q0;
+    }
+    if (!__syncthreads_and(ok)) return;       // also: gamma, gamma tau, tau of this step are written
+    // (2) warp 4: q; the others: p and C - gamma tau p
+    const double gamma = bc[0], gt = bc[1], ta = bc[2];
+    if (warp == 4) {
+      const double q = td_sum(red);
+      if (lane == 0) bc[7] = q;
+    } else {
+      {
+        int t = tid;
+        double ct = cn[min(t, L - 1)], st = pv[min(t, L - 1)];
+#pragma unroll 1
+        for (; t < L; t += TD_VEC) {
+          const double c0 = ct, pt = fma(gamma, ct, st);
+          ct = cn[min(t + TD_VEC, L - 1)];
+          st = pv[min(t + TD_VEC, L - 1)];
+          pv[t] = pt;
+          cn[t] = fma(-gt, pt, c0);
+        }
+      }
+      if (warp == 3) {
+        const double S0 = bc[8], C0 = bc[9];
+        const double e1 = fma(bc[4], C0, bc[3] * S0), h1 = fma(bc[6], C0, 2.0 * gt * S0);
+        if (lane == 0) { bc[10] = e1; bc[11] = h1; }
+      }
+      // the owned columns' scalars that do not wait for q (p_j from the warp's own S_j and row k + 1)
+#pragma unroll 1
+      for (int q = warp; q < nslot; q += 4) {
         const int j = q * G + blockIdx.x;
         if (j < k + 2 || j >= N) continue;
-        publish_pair(Pn + 2 * (j - k - 2), tn * fma(scn, colS[q], colF[q]), (k + 1) & 3);
+        const double bj = ta * v[j - (k + 1)];
+        const double tp = ta * fma(gamma, cols[(size_t)q * N + k + 1], cS[q]);
+        if (lane == 0) { cB[q] = bj; cT[q] = tp; }
       }
     }
-    if (next)
-      for (int t = tid; t < L - 1; t += TB) v2[t] = (t == 0) ? 1.0 : c[t + 1] * scn;
-    // (5) store the reflector v_k below the subdiagonal of column k (for the back-transformation)
-    if (blockIdx.x == ob)
-      for (int t = tid; t < L; t += TB) A[(size_t)k * lda + k + 1 + t] = v[t];
-    tk = tn;
-    bk = bn;
     __syncthreads();
+    // (3) c_{k+1}
+    if (warp < 4) {
+      const double e3 = fma(-bc[5], bc[7], bc[10]);
+      int t = tid;
+      double gr = cn[min(t, L - 1)], vt = v[min(t, L - 1)];
+#pragma unroll 1
+      for (; t < L; t += TD_VEC) {
+        const double x = fma(-e3, vt, gr);
+        gr = cn[min(t + TD_VEC, L - 1)];
+        vt = v[min(t + TD_VEC, L - 1)];
+        cn[t] = x;
+      }
+    }
+    __syncthreads();
+    if (warp == 4) {
+      // (4) sigma and the scalars of column k + 1, beside the column passes
+      const double c0 = cn[0], c1 = cn[1], beta = h.beta;
+      if (next) {
+        double part = 0.0;
+        int t = 2 + lane;
+        double x = t < L ? cn[t] : 0.0;
+#pragma unroll 1
+        for (int b = 2; b < L; b += 32) {
+          const double y = x;
+          t += 32;
+          x = t < L ? cn[t] : 0.0;
+          part = fma(y, y, part);
+        }
+        h = td_scalars(c1, td_warp_sum(part));
+        __syncwarp();
+        if (lane == 0) {
+          td_coefficients(h, bc);
+          cn[1] = h.gamma;
+        }
+      }
+      if (blockIdx.x == ob && lane == 0) {
+        d[k + 1] = minv * c0;
+        e[k] = minv * beta;
+        tau[k] = ta;
+        if (!next) { e[k + 1] = minv * c1; tau[k + 1] = 0.0; }
+      }
+    } else {
+      const double hq = fma(ta, bc[7], bc[11]);
+#pragma unroll 1
+      for (int q = warp; q < nslot; q += 4) {
+        const int j = q * G + blockIdx.x;
+        if (j < k + 2 || j >= N) continue;
+        const int tj = j - (k + 1);
+        double* col = cols + (size_t)q * N + k + 1;
+        const double bj = cB[q], aj = fma(-bj, hq, cT[q]);
+        double S = td_column<REP>(col, v, pv, cn, aj, bj, L, lane, next && tj == 1 ? out : nullptr, rep);   // tj = 1: the next C
+        if (next) {
+          S = td_warp_sum(S);
+          if (lane == 0) cS[q] = S;
+          if (lane < REP) publish(out + lane * rep + 2 * (tj - 1), S);
+        } else if (lane == 0) {
+          d[N - 1] = minv * col[1];           // L = 2: the last diagonal entry
+        }
+      }
+    }
+    // (5) warp 4 stores the reflector below the subdiagonal of column k
+    if (blockIdx.x == ob && warp == 4)
+      for (int t = lane; t < L; t += 32) A[(size_t)k * lda + k + 1 + t] = v[t];
   }
 }
 
@@ -1052,11 +1222,20 @@ k_bt_tmat(const double* __restrict__ A, int lda, const double* __restrict__ tau,
   for (int e = threadIdx.x; e < RB * RB; e += blockDim.x) Tm[(size_t)g * RB * RB + e] = Ts[e / RB][e % RB];
   if (Vff) {
     // the group's reflectors (zero outside their support) and T as double-FP32 pairs, for
-    // k_backtransform_ff: converted once here instead of in every block of the back-transform
-    for (int e = threadIdx.x; e < RB * RB; e += blockDim.x) Tff[(size_t)g * RB * RB + e] = ff_from_double(Ts[e / RB][e % RB]);
+    // k_backtransform_ff: converted once here instead of in every block of the back-transform, and scaled to
+    // v_0 = 1 (T by v_0 on both sides), which keeps the pairs in FP32's range
+    __shared__ double v0[RB], r0[RB];
+    if (threadIdx.x < RB) {
+      const double x = threadIdx.x < nb ? A[(size_t)(k0 + threadIdx.x) * lda + k0 + threadIdx.x + 1] : 1.0;
+      v0[threadIdx.x] = x;
+      r0[threadIdx.x] = 1.0 / x;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < RB * RB; e += blockDim.x)
+      Tff[(size_t)g * RB * RB + e] = ff_from_double(Ts[e / RB][e % RB] * v0[e / RB] * v0[e % RB]);
     for (int e = threadIdx.x; e < RB * N; e += blockDim.x) {
       const int a = e / N, row = e - a * N;
-      const double x = (a < nb && row >= k0 + a + 1) ? A[(size_t)(k0 + a) * lda + row] : 0.0;
+      const double x = (a < nb && row >= k0 + a + 1) ? A[(size_t)(k0 + a) * lda + row] * r0[a] : 0.0;
       Vff[((size_t)g * RB + a) * N + row] = ff_from_double(x);
     }
   }
@@ -1396,8 +1575,8 @@ inline size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 size_t eig_workspace_bytes(int nmax) {
   size_t N = std::max(nmax, 1);
   size_t b = 0;
-  b += align_up(3 * N * sizeof(double));          // d, e, tau
-  b += 2 * align_up(4 * N * sizeof(double));      // P, C (double buffered (hi, lo) pairs)
+  b += align_up((3 * N + 1) * sizeof(double));    // d, e, tau, largest magnitude
+  b += align_up(td_replicas((int)N) * N * (N + 1) * sizeof(double));    // exchange slots of the tridiagonalisation, (S, C) per entry
   b += 3 * align_up(N * N * sizeof(double));      // Q, Qtmp, Delta
   b += 10 * align_up(N * sizeof(double));         // lam, lamk, lamtmp, Dw, Zw, Dk, Zk, Dd, rho, spare
   b += align_up(4 * N * sizeof(double));          // rot
@@ -1419,11 +1598,12 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   if (!pe) return 2;
   char* p = (char*)work;
   auto take = [&](size_t bytes) { void* q = p; p += align_up(bytes); return q; };
-  double* d = (double*)take(3 * N * sizeof(double));
+  double* d = (double*)take((3 * (size_t)N + 1) * sizeof(double));
   double* e = d + N;
   double* tau = e + N;
-  double* P = (double*)take(4 * N * sizeof(double));
-  double* Cb = (double*)take(4 * N * sizeof(double));
+  unsigned long long* amax = (unsigned long long*)(tau + N);
+  const size_t slot_bytes = td_replicas(N) * (size_t)N * (N + 1) * sizeof(double);
+  double* slots = (double*)take(slot_bytes);
   DcWork W;
   W.Q = (double*)take((size_t)N * N * sizeof(double));
   W.Qtmp = (double*)take((size_t)N * N * sizeof(double));
@@ -1451,35 +1631,34 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   W.gcnt = (int*)take(2 * N * sizeof(int));
   W.mergeof = nullptr;
 
-  // exchange buffers of the tridiagonalisation: every byte 0x0f, i.e. pairs whose both words carry
-  // epoch 3, which no consumer waits for before the buffer has been rewritten
-  cudaMemsetAsync(P, 0x0f, 4 * N * sizeof(double), st);
-  cudaMemsetAsync(Cb, 0x0f, 4 * N * sizeof(double), st);
+  cudaMemsetAsync(slots, 0xFF, slot_bytes, st);      // every slot empty
   cudaMemsetAsync(W.Q, 0, (size_t)N * N * sizeof(double), st);
-  cudaMemsetAsync(d, 0, 3 * N * sizeof(double), st);
+  cudaMemsetAsync(d, 0, (3 * (size_t)N + 1) * sizeof(double), st);
+  k_absmax<<<std::min(N, 304), 256, 0, st>>>(A, lda, N, amax); note_launch();
 
   // 1. tridiagonalisation (cooperative: all blocks co-resident)
   {
+    const void* fn = td_replicas(N) == 4 ? (const void*)k_tridiag<4> : (const void*)k_tridiag<1>;
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int G = N >= 3 ? std::max(1, std::min(nsm, (N + 3) / 4)) : 1;
-    cudaFuncSetAttribute(k_tridiag, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    int G = N >= 3 ? std::max(1, std::min(nsm, (N + 1) / 2)) : 1;
+    cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     size_t smem = 0;
     for (int attempt = 0; attempt < 8; ++attempt) {
       const int nslot = (N + G - 1) / G;
-      smem = (4 + (size_t)nslot) * N * sizeof(double);
-      cudaFuncSetAttribute(k_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
+      smem = (5 + (size_t)nslot) * N * sizeof(double);
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
       int occ = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tridiag, TD_THREADS, smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, TD_THREADS, smem);
       if ((long long)occ * nsm >= G) break;
       G = std::max(1, occ * nsm);     // fewer blocks own more columns each
       if (occ == 0) { cudaGetLastError(); return 1000 + (int)cudaErrorCooperativeLaunchTooLarge; }
     }
     if ((N + G - 1) / G > TD_MAX_SLOTS) return 1000 + (int)cudaErrorInvalidValue;
     long long poll_limit = wait_limit(kPollLimit);
-    void* args[] = {&A, &lda, &N, &d, &e, &tau, &P, &Cb, &err, &poll_limit};
-    cudaError_t ce = cudaLaunchCooperativeKernel((void*)k_tridiag, dim3(G), dim3(TD_THREADS), args, smem, st);
+    void* args[] = {&A, &lda, &N, &d, &e, &tau, &slots, &amax, &err, &poll_limit};
+    cudaError_t ce = cudaLaunchCooperativeKernel(fn, dim3(G), dim3(TD_THREADS), args, smem, st);
     note_launch();
     if (ce != cudaSuccess) return 1000 + (int)ce;
   }
