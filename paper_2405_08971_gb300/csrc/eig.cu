@@ -21,22 +21,6 @@ namespace {
 
 constexpr double kEps = 2.220446049250313e-16;
 
-// Reciprocal by Newton-Raphson: an FP32 seed (rcp.approx, ~2^-23 relative) refined by two FP64
-// Newton steps r <- r + r (1 - x r), which square the relative error each time (2^-46, 2^-92), so
-// the result is accurate to the last bit or two of FP64.  Falls back to division outside the FP32
-// exponent range.
-__device__ __forceinline__ double nr_rcp(double x) {
-  const float xf = (float)x;
-  const float ax = fabsf(xf);
-  if (!(ax > 1e-36f && ax < 1e36f)) return 1.0 / x;
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(xf));
-  double r = (double)rf;
-  r = fma(r, fma(-x, r, 1.0), r);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return r;
-}
-
 // sqrt(x) and 1 / sqrt(x), and 1 / x, for normal x > 0, from the hardware's approximations y (about 20 bits,
 // full FP64 exponent range) and one third-order step: with e = 1 - x y^2 the factor 1 + e / 2 + 3 e^2 / 8
 // (the binomial series of (1 - e)^(-1/2)), with e = 1 - x y the factor 1 + e + e^2.  Both remainders are
@@ -492,12 +476,14 @@ k_tridiag(double* __restrict__ A, int lda, int N, double* __restrict__ d, double
 struct MergeDesc { int lo, mid, hi; };
 
 struct DcWork {
-  double *lam, *lamk, *lamtmp, *Dw, *Zw, *Dk, *Zk, *Dd, *Q, *Qtmp, *Delta, *rho, *rot, *z2, *Tm;
-  int *colk, *cold, *perm, *Kp, *nrot, *mergeof, *gperm, *gcnt;
+  double *lam, *lamk, *Zw, *Dk, *Zk, *Dd, *Q, *Qtmp, *Delta, *rho, *rot, *z2, *Tm;
+  float2* Df;      // kept poles / rho as FP32 pairs, and the squared z components in FP32: for the secular guess
+  float* zf;
+  int *colk, *cold, *rank, *Kp, *nrot, *mergeof, *gperm, *gcnt;
 };
 
 __global__ void k_dc_init(const double* __restrict__ d, const double* __restrict__ e, int N, double* lam,
-                          double* Q) {
+                          double* Q, double* Qtmp) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= N) return;
   double v = d[j];
@@ -505,6 +491,7 @@ __global__ void k_dc_init(const double* __restrict__ d, const double* __restrict
   if (j + 1 < N) v -= fabs(e[j]);
   lam[j] = v;
   Q[(size_t)j * N + j] = 1.0;
+  Qtmp[(size_t)j * N + j] = 1.0;    // (a leaf without a merge at the deepest level is valid in both)
 }
 
 // Order-preserving integer key of a double (IEEE bit pattern; negative values mirrored), so the
@@ -512,22 +499,6 @@ __global__ void k_dc_init(const double* __restrict__ d, const double* __restrict
 __device__ __forceinline__ long long order_key(double x) {
   const long long b = __double_as_longlong(x);
   return b >= 0 ? b : (b ^ 0x7FFFFFFFFFFFFFFFLL);
-}
-
-// Block-wide maximum (every thread gets the result).
-__device__ double block_max(double v) {
-  __shared__ double red[32];
-  __syncthreads();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double t = (l < nw) ? red[l] : 0.0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
-  __syncthreads();
-  return t;
 }
 
 // Block-wide exclusive prefix sum of one int per thread (thread order); *total gets the sum.
@@ -562,7 +533,7 @@ __device__ int block_excl_scan(int v, int* total) {
 constexpr int DC_THREADS = 256;
 
 // Shared memory of k_dc_prep for a merge of order K: four FP64 arrays, one int64 key array, six int arrays.
-inline size_t prep_smem_bytes(int K) { return (size_t)K * (4 * sizeof(double) + sizeof(long long) + 6 * sizeof(int)); }
+__host__ __device__ inline size_t prep_smem_bytes(int K) { return (size_t)K * (4 * sizeof(double) + sizeof(long long) + 6 * sizeof(int)); }
 
 // Phase 1 of a merge: z vector, sorted poles, deflation.  One block per merge.
 //   1. The two ascending child spectra are merged by rank (each entry's position is its index
@@ -603,7 +574,8 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
     zz += z * z;
   }
   zz = block_sum(zz);
-  const double zn = sqrt(zz);
+  double zn, rzn;
+  fast_sqrt(fmax(zz, 1e-280), zn, rzn);
   const double rho = fabs(rho0) * zz;
   // 1. merge by rank (ties: child 1 first)
   for (int t = threadIdx.x; t < K; t += blockDim.x) {
@@ -620,14 +592,12 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
     }
     sPerm[pos] = t;
     sD[pos] = sLam[t];
-    sZ[pos] = sZr[t] / zn;
+    sZ[pos] = sZr[t] * rzn;
     sType[pos] = (t < n1) ? 1 : 3;
   }
   __syncthreads();
   // 2. tolerance and small-z deflation
-  double dm = 0.0;
-  for (int t = threadIdx.x; t < K; t += blockDim.x) dm = fmax(dm, fabs(sD[t]));
-  dm = block_max(dm);
+  const double dm = fmax(fabs(sD[0]), fabs(sD[K - 1]));   // sD ascends
   const double tol = 8.0 * kEps * fmax(dm, rho);
   for (int t = threadIdx.x; t < K; t += blockDim.x) sStat[t] = (rho * fabs(sZ[t]) <= tol) ? 1 : 0;
   __syncthreads();
@@ -723,11 +693,16 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
     __syncthreads();
     keep = sSort;
   }
+  const double irho = rho > 0.0 ? 1.0 / rho : 0.0;
   for (int q = threadIdx.x; q < kp; q += blockDim.x) {
     const int j = keep[q];
+    const double zj2 = sZ[j] * sZ[j], ds = sD[j] * irho;
+    const float dh = __double2float_rn(ds);
     W.Dk[lo + q] = sD[j];
     W.Zk[lo + q] = sZ[j];
-    W.z2[lo + q] = rho * sZ[j] * sZ[j];
+    W.z2[lo + q] = rho * zj2;
+    W.Df[lo + q] = make_float2(dh, __double2float_rn(ds - (double)dh));
+    W.zf[lo + q] = __double2float_rn(zj2);
     W.colk[lo + q] = lo + sPerm[j];
   }
   for (int q = threadIdx.x; q < K - kp; q += blockDim.x) {
@@ -810,109 +785,161 @@ k_dc_rot(const MergeDesc* __restrict__ merges, int N, DcWork W) {
   dc_rot_row(merges[blockIdx.y], N, W, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// Sum over the LANES lanes that share one root (LANES = 32: a warp; LANES = 1: one thread; in
-// between, an aligned group of lanes of a warp named by mask, which lets the groups of one warp
-// run different iteration counts).
+// Sum over the LANES lanes that share one root (LANES = 32: a warp; otherwise an aligned group of lanes of a
+// warp named by mask, which lets the groups of one warp run different iteration counts).
 template <int LANES> __device__ __forceinline__ double group_sum(double v, unsigned mask = 0xffffffffu) {
-  if constexpr (LANES == 32) return warp_sum(v);
-  else if constexpr (LANES == 1) return v;
-  else {
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-    return v;
-  }
+  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+// The same for four values at once, by a transposing butterfly: log2(LANES) + 1 additions per lane instead of
+// 4 log2(LANES) (each holds the FP64 pipe for 64 cycles); every lane gets all four sums.
+template <int LANES>
+__device__ __forceinline__ void group_sum4(double& a, double& b, double& c, double& d, int lane, unsigned mask) {
+  constexpr int H = LANES / 2, Q = LANES / 4;
+  const bool up = lane & H, up2 = lane & Q;
+  double x = up ? c : a, y = up ? d : b;
+  x += __shfl_xor_sync(mask, up ? a : c, H);
+  y += __shfl_xor_sync(mask, up ? b : d, H);
+  double v = up2 ? y : x;
+  v += __shfl_xor_sync(mask, up2 ? x : y, Q);
+#pragma unroll
+  for (int o = Q / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  a = __shfl_sync(mask, v, 0, LANES);
+  b = __shfl_sync(mask, v, Q, LANES);
+  c = __shfl_sync(mask, v, H, LANES);
+  d = __shfl_sync(mask, v, H + Q, LANES);
+}
+template <int LANES> __device__ __forceinline__ float group_sumf(float v, unsigned mask) {
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
 }
 
-// Phase 2: secular roots, LANES lanes per (merge, root) -- a warp for large merges, one thread for
-// small ones; the sums over poles are split across the lanes.
+__device__ __forceinline__ float rcp_r(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double rcp_r(double x) { return fast_rcp(x); }
+__device__ __forceinline__ float sqrt_r(float x) { return approx_sqrt(x); }
+__device__ __forceinline__ double sqrt_r(double x) {
+  if (!(x > 1e-280)) return 0.0;
+  double sq, rs;
+  fast_sqrt(x, sq, rs);
+  return sq;
+}
+// One step of the two-pole rational model of the secular function at tau (poles at distances Dl < 0 < Dr, in
+// the real type R): f ~ c + sl / (Dl - x) + sr / (Dr - x) with the parts' values and slopes matched.  Returns
+// the root inside (lo, hi), or NaN.
+template <class R>
+__device__ __forceinline__ R secular_step(R f, R dpsi, R dphi, R Dl, R Dr, bool inner, R tau, R lo, R hi) {
+  const R sl = Dl * Dl * dpsi;
+  R c1, c2;
+  if (inner) {
+    const R sr = Dr * Dr * dphi;
+    const R c = f - Dl * dpsi - Dr * dphi;
+    const R B2 = -(c * (Dl + Dr) + sl + sr), C2 = c * Dl * Dr + sl * Dr + sr * Dl;
+    R disc = B2 * B2 - R(4) * c * C2;
+    disc = disc > R(0) ? disc : R(0);
+    const R q = R(-0.5) * (B2 + copysign(sqrt_r(disc), B2));
+    c1 = q * rcp_r(c);
+    c2 = C2 * rcp_r(q);
+  } else {
+    const R c = f - Dl * dpsi;
+    c1 = c2 = Dl + sl * rcp_r(c);
+  }
+  const R t1 = tau + c1, t2 = tau + c2;
+  if (t1 > lo && t1 < hi) return t1;     // (false for NaN)
+  if (t2 > lo && t2 < hi) return t2;
+  return R(NAN);
+}
+
+// Phase 2: secular roots, LANES lanes per (merge, root); the sums over poles are split across the lanes.
 // delta column i: Delta[(lo+i)*N + lo + j] = Dk_j - lam_i, computed from the origin pole.
+// A guess is found in FP32 first (poles as FP32 pairs, so that their differences keep their leading digits;
+// about 30 times cheaper per evaluation than FP64); the FP64 iteration starts there, on the whole interval
+// between the poles as its bracket, and decides convergence alone: about 3 evaluations instead of 7.
 template <int LANES>
 __device__ void dc_secular_root(int lo, int i, int N, DcWork W, int* err, int lane, unsigned gmask) {
   const int Kp = W.Kp[lo];
   if (i >= Kp) return;
   const double* Dk = W.Dk + lo;
-  const double* Zk = W.Zk + lo;
   const double* z2 = W.z2 + lo;
   const double rho = W.rho[lo];
   double* delta = W.Delta + (size_t)(lo + i) * N + lo;
-  // For an inner root the sums are first evaluated at the midpoint of (D_i, D_{i+1}): the sign of f
-  // there picks the origin pole (the nearer end of the root's half interval), and the same sums give
-  // the first rational-model step from the midpoint.  The last root starts from its bracket midpoint.
-  int org;
-  double tlo, thi, tau;
-  double psi = 0.0, dpsi = 0.0, phi = 0.0, dphi = 0.0;
-  bool have = false;            // sums already evaluated at tau
-  if (i < Kp - 1) {
-    const double mid = 0.5 * (Dk[i] + Dk[i + 1]);
-    for (int j = lane; j < Kp; j += LANES) {
-      const double rinv = nr_rcp(Dk[j] - mid);
-      const double tv = z2[j] * rinv;
-      if (j <= i) { psi += tv; dpsi += tv * rinv; }
-      else { phi += tv; dphi += tv * rinv; }
+  const bool inner = i < Kp - 1;
+  // ---- FP32 guess, in units of rho
+  int org = i;
+  float tg;
+  {
+    const float2* Df = W.Df + lo;
+    const float* zf = W.zf + lo;
+    float2 o = Df[i];
+    const float gap = inner ? (Df[i + 1].x - o.x) + (Df[i + 1].y - o.y) : 1.0f;
+    float tl = 0.f, th = gap;
+    tg = 0.5f * gap;
+    for (int it = 0; it < 40; ++it) {
+      float psi = 0.f, dpsi = 0.f, phi = 0.f, dphi = 0.f;
+      for (int j = lane; j < Kp; j += LANES) {
+        const float2 dj = Df[j];
+        const float r = __fdividef(1.0f, ((dj.x - o.x) + (dj.y - o.y)) - tg);
+        const float tv = zf[j] * r;
+        if (j <= i) { psi += tv; dpsi = fmaf(tv, r, dpsi); }
+        else { phi += tv; dphi = fmaf(tv, r, dphi); }
+      }
+      psi = group_sumf<LANES>(psi, gmask); dpsi = group_sumf<LANES>(dpsi, gmask);
+      phi = group_sumf<LANES>(phi, gmask); dphi = group_sumf<LANES>(dphi, gmask);
+      const float f = 1.0f + psi + phi;
+      if (it == 0 && inner && f < 0.f) {     // the root is nearer to the right pole
+        org = i + 1;
+        o = Df[org];
+        tl = -gap; th = 0.f;
+        tg = -0.5f * gap;
+      }
+      if (!(fabsf(f) > 1e-6f * (1.0f - psi + phi))) break;
+      if (f > 0.f) th = tg; else tl = tg;
+      const float2 dl = Df[i], dr = inner ? Df[i + 1] : o;
+      const float Dl = ((dl.x - o.x) + (dl.y - o.y)) - tg, Dr = ((dr.x - o.x) + (dr.y - o.y)) - tg;
+      float nt = secular_step(f, dpsi, dphi, Dl, Dr, inner, tg, tl, th);
+      if (!(nt > tl && nt < th)) nt = 0.5f * (tl + th);
+      const bool done = fabsf(nt - tg) <= 1e-6f * fabsf(nt);
+      tg = nt;
+      if (done) break;
     }
-    psi = group_sum<LANES>(psi, gmask); dpsi = group_sum<LANES>(dpsi, gmask);
-    phi = group_sum<LANES>(phi, gmask); dphi = group_sum<LANES>(dphi, gmask);
-    if (1.0 + psi + phi >= 0.0) { org = i; tlo = 0.0; thi = mid - Dk[i]; tau = thi; }
-    else { org = i + 1; tlo = mid - Dk[i + 1]; thi = 0.0; tau = tlo; }
-    have = true;
-  } else {
-    org = i;
-    double zz = 0.0;
-    for (int j = lane; j < Kp; j += LANES) zz += Zk[j] * Zk[j];
-    tlo = 0.0;
-    thi = rho * group_sum<LANES>(zz, gmask);
-    tau = 0.5 * (tlo + thi);
   }
+  // ---- FP64
   const double Dorg = Dk[org];
+  double tlo, thi;
+  if (!inner) { tlo = 0.0; thi = rho * (1.0 + 1e-12); }      // |z| = 1
+  else if (org == i) { tlo = 0.0; thi = Dk[i + 1] - Dorg; }
+  else { tlo = Dk[i] - Dorg; thi = 0.0; }
+  double tau = (double)tg * rho;
+  if (!(tau > tlo && tau < thi)) tau = 0.5 * (tlo + thi);
   bool conv = false;
   for (int it = 0; it < 200 && !conv; ++it) {
-    if (!have) {
-      psi = 0.0; dpsi = 0.0; phi = 0.0; dphi = 0.0;
-      for (int j = lane; j < Kp; j += LANES) {
-        const double dl = (Dk[j] - Dorg) - tau;
-        const double rinv = nr_rcp(dl);
-        const double tv = z2[j] * rinv;
-        if (j <= i) { psi += tv; dpsi += tv * rinv; }
-        else { phi += tv; dphi += tv * rinv; }
-      }
-      psi = group_sum<LANES>(psi, gmask); dpsi = group_sum<LANES>(dpsi, gmask);
-      phi = group_sum<LANES>(phi, gmask); dphi = group_sum<LANES>(dphi, gmask);
+    double psi = 0.0, dpsi = 0.0, phi = 0.0, dphi = 0.0;
+    int j = lane;
+#pragma unroll 2
+    for (; j <= i; j += LANES) {
+      const double rinv = fast_rcp((Dk[j] - Dorg) - tau);
+      const double tv = z2[j] * rinv;
+      psi += tv;
+      dpsi = fma(tv, rinv, dpsi);
     }
-    have = false;
+#pragma unroll 2
+    for (; j < Kp; j += LANES) {
+      const double rinv = fast_rcp((Dk[j] - Dorg) - tau);
+      const double tv = z2[j] * rinv;
+      phi += tv;
+      dphi = fma(tv, rinv, dphi);
+    }
+    __syncwarp(gmask);
+    group_sum4<LANES>(psi, dpsi, phi, dphi, lane, gmask);
     const double f = 1.0 + psi + phi;
     if (f == 0.0) break;
     // residual test: f is as small as rounding of its terms allows (psi < 0 < phi term-wise)
     if (fabs(f) <= 8.0 * kEps * (1.0 - psi + phi)) break;
     if (f > 0.0) thi = tau; else tlo = tau;
-    // The model step is a guess (the bracket and the residual test decide convergence), so its
-    // quotients are taken as products with Newton reciprocals (about 1 ulp; an FP64 division has a
-    // much longer dependency chain on this GPU).
-    const double Dl = (Dk[i] - Dorg) - tau;
-    const double sl = Dl * Dl * dpsi;
-    double nt = NAN;
-    if (i < Kp - 1) {
-      const double Dr = (Dk[i + 1] - Dorg) - tau;
-      const double sr = Dr * Dr * dphi;
-      const double c = f - sl * nr_rcp(Dl) - sr * nr_rcp(Dr);
-      const double A2 = c, B2 = -(c * (Dl + Dr) + sl + sr), C2 = c * Dl * Dr + sl * Dr + sr * Dl;
-      double c1 = NAN, c2 = NAN;
-      if (A2 == 0.0) { if (B2 != 0.0) c1 = -C2 * nr_rcp(B2); }
-      else {
-        double disc = B2 * B2 - 4.0 * A2 * C2;
-        if (disc < 0.0) disc = 0.0;
-        const double q = -0.5 * (B2 + copysign(sqrt(disc), B2));
-        c1 = q * nr_rcp(A2);
-        if (q != 0.0) c2 = C2 * nr_rcp(q);
-      }
-      if (isfinite(c1) && tau + c1 > tlo && tau + c1 < thi) nt = tau + c1;
-      else if (isfinite(c2) && tau + c2 > tlo && tau + c2 < thi) nt = tau + c2;
-    } else {
-      const double c = f - sl * nr_rcp(Dl);
-      if (c != 0.0) {
-        const double t2 = tau + Dl + sl * nr_rcp(c);
-        if (isfinite(t2) && t2 > tlo && t2 < thi) nt = t2;
-      }
-    }
+    // the model step is a guess: the bracket and the residual test decide convergence
+    const double Dl = (Dk[i] - Dorg) - tau, Dr = inner ? (Dk[i + 1] - Dorg) - tau : 0.0;
+    double nt = secular_step(f, dpsi, dphi, Dl, Dr, inner, tau, tlo, thi);
     if (!isfinite(nt)) nt = 0.5 * (tlo + thi);
     conv = fabs(nt - tau) <= 2.0 * kEps * fmax(fabs(nt), fabs(tau)) ||
            (thi - tlo) <= 4.0 * kEps * fmax(fabs(tlo), fabs(thi));
@@ -934,9 +961,10 @@ __global__ void k_dc_secular(const MergeDesc* __restrict__ merges, const int* __
   dc_secular_root<LANES>(lo, p - lo, N, W, err, lane, 0xffffffffu);
 }
 
-// Phase 3: Loewner-corrected z (one warp per j):
+// Phase 3: Loewner-corrected z:
 //   zhat_j^2 = (lam_last - D_j)/rho * prod_{i<j} (lam_i - D_j)/(D_i - D_j) * prod_{i>j} (lam_{i-1} - D_j)/(D_i - D_j)
-// The product is formed as a sum of logarithms of the (positive) factors split across lanes.
+// Numerators and denominators are multiplied as mantissas in [1, 2) with their exponents summed in integers
+// (no division, logarithm or overflow per factor), rescaled every 512 factors of a lane.
 template <int LANES>
 __device__ void dc_zhat_one(int lo, int j, int N, DcWork W, int lane, unsigned gmask) {
   const int Kp = W.Kp[lo];
@@ -944,21 +972,55 @@ __device__ void dc_zhat_one(int lo, int j, int N, DcWork W, int lane, unsigned g
   const double* Dk = W.Dk + lo;
   const double rho = W.rho[lo];
   const double Dj = Dk[j];
-  // each lane multiplies its factors and takes one logarithm (more only if the product leaves
-  // [1e-150, 1e150]); the lanes' logarithms are summed
-  double lg = 0.0, prod = 1.0;
+  double pn = 1.0, pd = 1.0;
+  int ex = 0;
+  const long long kOne = 0x3FFLL << 52, kExp = 0x7FFLL << 52;
+  auto split = [&](double x, int sign) {      // mantissa of |x| in [1, 2); its exponent into ex
+    const long long b = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL;
+    ex += sign * ((int)(b >> 52) - 1023);
+    return __longlong_as_double((b & ~kExp) | kOne);
+  };
+  int cnt = 0;
   for (int i = lane; i < Kp; i += LANES) {
     if (i == j) continue;
     const int ii = (i < j) ? i : i - 1;                       // lam_i for i < j, lam_{i-1} for i > j
-    const double num = -W.Delta[(size_t)(lo + ii) * N + lo + j];
-    prod *= fabs(num / (Dk[i] - Dj));
-    if (!(prod > 1e-150 && prod < 1e150)) { lg += log(prod); prod = 1.0; }
+    pn *= split(W.Delta[(size_t)(lo + ii) * N + lo + j], 1);
+    pd *= split(Dk[i] - Dj, -1);
+    if (++cnt == 512) { pn = split(pn, 1); pd = split(pd, -1); cnt = 0; }
   }
-  lg += log(prod);
-  lg = group_sum<LANES>(lg, gmask);
+  pn = split(pn, 1);
+  pd = split(pd, -1);
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) {
+    pn *= __shfl_xor_sync(gmask, pn, o);
+    pd *= __shfl_xor_sync(gmask, pd, o);
+    ex += __shfl_xor_sync(gmask, ex, o);
+  }
   if (lane == 0) {
-    const double last = -W.Delta[(size_t)(lo + Kp - 1) * N + lo + j] / rho;
-    W.Zw[lo + j] = copysign(sqrt(fabs(last)) * exp(0.5 * lg), W.Zk[lo + j]);
+    // sqrt(last prod) with the exponent halved: an odd one leaves a factor 2 under the root
+    const double last = split(W.Delta[(size_t)(lo + Kp - 1) * N + lo + j], 1);
+    const double r = split(rho, -1);
+    double m = last * pn / (r * pd);
+    if (ex & 1) m *= 2.0;
+    W.Zw[lo + j] = copysign(ldexp(sqrt(m), ex >> 1), W.Zk[lo + j]);
+  }
+}
+// Position of item t (roots, then deflated poles) in the merged spectrum: its rank on (value key, item).
+template <int LANES>
+__device__ void dc_rank_one(const MergeDesc mg, int t, DcWork W, int lane, unsigned gmask) {
+  const int lo = mg.lo, K = mg.hi - mg.lo, Kp = W.Kp[lo];
+  const double v = (t < Kp) ? W.lamk[lo + t] : W.Dd[lo + t - Kp];
+  const long long kt = order_key(v);
+  int r = 0;
+  for (int u = lane; u < K; u += LANES) {
+    const long long ku = order_key((u < Kp) ? W.lamk[lo + u] : W.Dd[lo + u - Kp]);
+    r += (ku < kt) || (ku == kt && u < t);
+  }
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) r += __shfl_xor_sync(gmask, r, o);
+  if (lane == 0) {
+    W.lam[lo + r] = v;
+    W.rank[lo + t] = r;
   }
 }
 template <int LANES>
@@ -970,6 +1032,7 @@ __global__ void k_dc_zhat(const MergeDesc* __restrict__ merges, const int* __res
   if (mi < 0) return;
   const int lo = merges[mi].lo;
   dc_zhat_one<LANES>(lo, p - lo, N, W, lane, 0xffffffffu);
+  dc_rank_one<LANES>(merges[mi], p - lo, W, lane, 0xffffffffu);
 }
 
 // Phase 4: eigenvector columns u_i = zhat / delta_i, normalised, written over Delta (one warp per i).
@@ -979,9 +1042,10 @@ __device__ void dc_vecs_one(int lo, int i, int N, DcWork W, int lane, unsigned g
   if (i >= Kp) return;
   double* col = W.Delta + (size_t)(lo + i) * N + lo;
   double nrm = 0.0;
-  for (int j = lane; j < Kp; j += LANES) { double u = W.Zw[lo + j] * nr_rcp(col[j]); col[j] = u; nrm += u * u; }
+  for (int j = lane; j < Kp; j += LANES) { double u = W.Zw[lo + j] * fast_rcp(col[j]); col[j] = u; nrm = fma(u, u, nrm); }
   nrm = group_sum<LANES>(nrm, gmask);
-  const double inv = 1.0 / sqrt(nrm);
+  double nv, inv;
+  fast_sqrt(nrm, nv, inv);
   for (int j = lane; j < Kp; j += LANES) col[j] *= inv;
 }
 template <int LANES>
@@ -995,22 +1059,37 @@ __global__ void k_dc_vecs(const MergeDesc* __restrict__ merges, const int* __res
   dc_vecs_one<LANES>(lo, p - lo, N, W, lane, 0xffffffffu);
 }
 
-// Phase 5: Qtmp[lo:hi, lo+i] = Q[lo:hi, colk] U[:, i] (i < Kp); deflated columns copied after them.
-// The sum over kept poles runs in the support order of phase 1 (gperm): a row tile inside child 1
-// skips the columns supported on child 2 only and vice versa, about half of the products.
+// Phase 5: Qtmp[lo:hi, lo + rank] = Q[lo:hi, colk] U[:, i] (i < Kp), and the deflated columns copied; the columns
+// land in ascending order of the merged spectrum, and Q and Qtmp change places for the next level.  Columns
+// of rank below cmin (the final merge's, where the caller keeps only the top) are left out.  The sum over kept
+// poles runs in the support order of phase 1 (gperm): a row tile inside child 1 skips the columns supported
+// on child 2 only and vice versa, about half of the products.  FP64-bound, so nothing is computed for
+// padding: the last stage has its own length and halves of a tile beyond the merge are skipped.
 constexpr int DG_T = 32;
-// (device function: every thread of a 256-thread block calls it with the same tile)
-__device__ void dc_gemm_tile(const MergeDesc mg, int N, DcWork W, int r0, int c0) {
+__global__ void __launch_bounds__(256)
+k_dc_gemm(const MergeDesc* __restrict__ merges, int N, DcWork W, int cmin) {
+  const MergeDesc mg = merges[blockIdx.z];
+  const int r0 = blockIdx.x * DG_T, c0 = blockIdx.y * DG_T;
   const int lo = mg.lo, K = mg.hi - mg.lo, n1 = mg.mid - mg.lo;
   const int Kp = W.Kp[lo];
   if (r0 >= K || c0 >= K) return;
   __shared__ double As[DG_T][DG_T + 1], Bs[DG_T][DG_T + 1];
+  __shared__ int srank[DG_T];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  int want = 0;
+  if (threadIdx.x < DG_T) {
+    const int c = c0 + threadIdx.x;
+    const int r = c < K ? W.rank[lo + c] : -1;
+    srank[threadIdx.x] = r >= cmin ? r : -1;
+    want = r >= cmin;
+  }
+  if (!__syncthreads_or(want)) return;
   const int g1 = W.gcnt[2 * lo], g2 = W.gcnt[2 * lo + 1];
   int kb = 0, ke = Kp;
   if (r0 + DG_T <= n1) ke = g1 + g2;        // rows of child 1 only
   else if (r0 >= n1) kb = g1;               // rows of child 2 only
   const int* gp = W.gperm + lo;
+  const bool a2 = r0 + 16 < K, b2 = c0 + 16 < Kp;
   double acc[2][2] = {{0, 0}, {0, 0}};
   if (c0 < Kp) {
     for (int k0 = kb; k0 < ke; k0 += DG_T) {
@@ -1028,115 +1107,110 @@ __device__ void dc_gemm_tile(const MergeDesc mg, int N, DcWork W, int r0, int c0
         }
       }
       __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < DG_T; ++kk)
+      const int kn = min(DG_T, ke - k0);
+      if (a2 && b2) {
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk)
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+          for (int a = 0; a < 2; ++a)
 #pragma unroll
-          for (int b = 0; b < 2; ++b) acc[a][b] = fma(As[kk][ty + 16 * a], Bs[kk][tx + 16 * b], acc[a][b]);
+            for (int b = 0; b < 2; ++b) acc[a][b] = fma(As[kk][ty + 16 * a], Bs[kk][tx + 16 * b], acc[a][b]);
+      } else if (a2) {
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk)
+#pragma unroll
+          for (int a = 0; a < 2; ++a) acc[a][0] = fma(As[kk][ty + 16 * a], Bs[kk][tx], acc[a][0]);
+      } else if (b2) {
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk)
+#pragma unroll
+          for (int b = 0; b < 2; ++b) acc[0][b] = fma(As[kk][ty], Bs[kk][tx + 16 * b], acc[0][b]);
+      } else {
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk) acc[0][0] = fma(As[kk][ty], Bs[kk][tx], acc[0][0]);
+      }
       __syncthreads();
     }
   }
+  // through shared memory, so that consecutive threads store consecutive rows
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      int row = r0 + ty + 16 * a, c = c0 + tx + 16 * b;
-      if (row >= K || c >= K) continue;
-      double val;
-      if (c < Kp) val = acc[a][b];
-      else val = W.Q[(size_t)W.cold[lo + (c - Kp)] * N + lo + row];
-      W.Qtmp[(size_t)(lo + c) * N + lo + row] = val;
-    }
-}
-__global__ void __launch_bounds__(256)
-k_dc_gemm(const MergeDesc* __restrict__ merges, int N, DcWork W) {
-  dc_gemm_tile(merges[blockIdx.z], N, W, blockIdx.x * DG_T, blockIdx.y * DG_T);
-}
-
-// Phase 6a: order the merged spectrum ascending (one block per merge): W.lam and the column
-// permutation W.perm (relative to lo) for phase 6b.  Rank sort on (value key, position): the kept
-// roots come before deflated poles of equal value.
-__device__ void dc_finish(const MergeDesc mg, int N, DcWork W, double* fsm) {
-  const int lo = mg.lo, K = mg.hi - mg.lo;
-  const int Kp = W.Kp[lo];
-  double* sl = fsm;                                          // K merged eigenvalues (kept roots, deflated poles)
-  long long* key = reinterpret_cast<long long*>(fsm + K);
-  for (int t = threadIdx.x; t < K; t += blockDim.x) {
-    const double v = (t < Kp) ? W.lamk[lo + t] : W.Dd[lo + t - Kp];
-    sl[t] = v;
-    key[t] = order_key(v);
-  }
+    for (int b = 0; b < 2; ++b) As[tx + 16 * b][ty + 16 * a] = acc[a][b];
   __syncthreads();
-  for (int t = threadIdx.x; t < K; t += blockDim.x) {
-    const long long kt = key[t];
-    int rank = 0;
-    for (int u = 0; u < K; ++u) {
-      const long long ku = key[u];
-      rank += (ku < kt) || (ku == kt && u < t);
-    }
-    W.lam[lo + rank] = sl[t];
-    W.perm[lo + rank] = t;
+  for (int e2 = threadIdx.x; e2 < DG_T * DG_T; e2 += 256) {
+    const int rr = e2 % DG_T, cc = e2 / DG_T, row = r0 + rr, c = c0 + cc, r = srank[cc];
+    if (row >= K || r < 0) continue;
+    W.Qtmp[(size_t)(lo + r) * N + lo + row] =
+        c < Kp ? As[cc][rr] : W.Q[(size_t)W.cold[lo + (c - Kp)] * N + lo + row];
   }
-}
-__global__ void __launch_bounds__(256)
-k_dc_finish(const MergeDesc* __restrict__ merges, int N, DcWork W) {
-  extern __shared__ double fsm[];
-  dc_finish(merges[blockIdx.x], N, W, fsm);
-}
-
-// Phase 6b: move the merged eigenvector columns back into Q in ascending order
-// (grid: column groups of 8 x merges).
-__device__ void dc_copy_cols(const MergeDesc mg, int N, DcWork W, int c0) {
-  const int lo = mg.lo, K = mg.hi - mg.lo;
-  if (c0 >= K) return;
-  const int c1 = min(K, c0 + 8);
-  for (int c = c0; c < c1; ++c) {
-    const double* src = W.Qtmp + (size_t)(lo + W.perm[lo + c]) * N + lo;
-    double* dst = W.Q + (size_t)(lo + c) * N + lo;
-    for (int row = threadIdx.x; row < K; row += blockDim.x) dst[row] = src[row];
-  }
-}
-__global__ void __launch_bounds__(256)
-k_dc_copy(const MergeDesc* __restrict__ merges, int N, DcWork W) {
-  dc_copy_cols(merges[blockIdx.y], N, W, blockIdx.x * 8);
 }
 
 // All phases of a merge of order at most DC_SMALL_K in one block (one block per merge of the level):
-// the levels near the leaves have many small merges, where eight launches per level cost more than
-// the work.  The phases run in the order of the per-phase kernels, separated by block barriers;
-// every phase touches only the merge's own rows and columns.  Roots, z entries and eigenvector
-// columns are taken by groups of DC_SMALL_LANES lanes.
+// the levels near the leaves have many small merges, where six launches per level cost more than the
+// work.  The phases run in the order of the per-phase kernels, separated by block barriers; every phase
+// touches only the merge's own rows and columns.  Roots, z entries and eigenvector columns are taken by
+// groups of L lanes; the child eigenvectors and U are multiplied out of shared memory.  Blocks beyond the
+// merges (the first level's launch has them) run the back-transformation's bt_tmat, which depends on the
+// tridiagonalisation alone.
 constexpr int DC_SMALL_K = 40;
-constexpr int DC_SMALL_LANES = 8;
-inline size_t small_smem_bytes(int K) {
-  return std::max(prep_smem_bytes(K), (size_t)K * (sizeof(double) + sizeof(long long)));
+inline size_t small_smem_bytes(int K) { return prep_smem_bytes(K) + (size_t)2 * K * (K + 1) * sizeof(double); }
+__device__ void bt_tmat(const double* A, int lda, const double* tau, int N, int g, double* Tm, float2* Vff, float2* Tff);
+struct TmatArgs { const double* A; int lda; const double* tau; double* Tm; float2 *Vff, *Tff; };
+
+template <int L>
+__device__ __forceinline__ void dc_small_roots(int lo, int K, int N, DcWork W, const MergeDesc mg, int* err) {
+  const int grp = threadIdx.x / L, lane = threadIdx.x % L, ngrp = blockDim.x / L;
+  const unsigned gmask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u)) << ((threadIdx.x & 31) & ~(L - 1));
+  const int Kp = W.Kp[lo];
+  for (int i = grp; i < Kp; i += ngrp) dc_secular_root<L>(lo, i, N, W, err, lane, gmask);
+  __syncthreads();
+  for (int j = grp; j < K; j += ngrp) {
+    dc_zhat_one<L>(lo, j, N, W, lane, gmask);
+    dc_rank_one<L>(mg, j, W, lane, gmask);
+  }
+  __syncthreads();
+  for (int i = grp; i < Kp; i += ngrp) dc_vecs_one<L>(lo, i, N, W, lane, gmask);
+  __syncthreads();
 }
 __global__ void __launch_bounds__(DC_THREADS)
-k_dc_small(const MergeDesc* __restrict__ merges, const double* __restrict__ e, int N, DcWork W, int* err) {
+k_dc_small(const MergeDesc* __restrict__ merges, int nm, const double* __restrict__ e, int N, DcWork W, int* err,
+           TmatArgs ta) {
   extern __shared__ double ssm[];
-  constexpr int L = DC_SMALL_LANES;
+  if ((int)blockIdx.x >= nm) {
+    bt_tmat(ta.A, ta.lda, ta.tau, N, blockIdx.x - nm, ta.Tm, ta.Vff, ta.Tff);
+    return;
+  }
   const MergeDesc mg = merges[blockIdx.x];
-  const int lo = mg.lo, K = mg.hi - mg.lo;
+  const int lo = mg.lo, K = mg.hi - mg.lo, n1 = mg.mid - mg.lo;
   dc_prep(mg, e, N, W, ssm);
   __syncthreads();
   for (int row = threadIdx.x; row < K; row += blockDim.x) dc_rot_row(mg, N, W, row);
   __syncthreads();
-  const int Kp = W.Kp[lo];
-  const int grp = threadIdx.x / L, lane = threadIdx.x % L, ngrp = blockDim.x / L;
-  const unsigned gmask = ((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
-  for (int i = grp; i < Kp; i += ngrp) dc_secular_root<L>(lo, i, N, W, err, lane, gmask);
+  if (K <= DC_THREADS / 8) dc_small_roots<8>(lo, K, N, W, mg, err);
+  else dc_small_roots<4>(lo, K, N, W, mg, err);
+  const int Kp = W.Kp[lo], g1 = W.gcnt[2 * lo], g2 = W.gcnt[2 * lo + 1], ld = K + 1;
+  double* Qs = ssm + prep_smem_bytes(K) / sizeof(double);
+  double* Us = Qs + (size_t)K * ld;
+  const int* gp = W.gperm + lo;
+  for (int x = threadIdx.x; x < Kp * K; x += blockDim.x) {     // kept columns and U in support order
+    const int row = x % K, q = x / K, g = gp[q];
+    Qs[q * ld + row] = W.Q[(size_t)W.colk[lo + g] * N + lo + row];
+    if (row < Kp) Us[row * ld + q] = W.Delta[(size_t)(lo + row) * N + lo + g];
+  }
   __syncthreads();
-  for (int j = grp; j < Kp; j += ngrp) dc_zhat_one<L>(lo, j, N, W, lane, gmask);
-  __syncthreads();
-  for (int i = grp; i < Kp; i += ngrp) dc_vecs_one<L>(lo, i, N, W, lane, gmask);
-  __syncthreads();
-  const int nt = (K + DG_T - 1) / DG_T;
-  for (int t = 0; t < nt * nt; ++t) dc_gemm_tile(mg, N, W, (t / nt) * DG_T, (t % nt) * DG_T);
-  __syncthreads();
-  dc_finish(mg, N, W, ssm);
-  __syncthreads();
-  for (int c0 = 0; c0 < K; c0 += 8) dc_copy_cols(mg, N, W, c0);
+  for (int x = threadIdx.x; x < K * K; x += blockDim.x) {
+    const int row = x % K, c = x / K;
+    double v;
+    if (c < Kp) {
+      const int kb = row < n1 ? 0 : g1, ke = row < n1 ? g1 + g2 : Kp;
+      v = 0.0;
+      for (int q = kb; q < ke; ++q) v = fma(Qs[q * ld + row], Us[c * ld + q], v);
+    } else {
+      v = W.Q[(size_t)W.cold[lo + (c - Kp)] * N + lo + row];
+    }
+    W.Qtmp[(size_t)(lo + W.rank[lo + c]) * N + lo + row] = v;
+  }
 }
 
 // ---- double-FP32 arithmetic (pairs hi + lo of FP32 numbers).  The _rn intrinsics keep the compiler
@@ -1185,10 +1259,9 @@ constexpr int CB = 4;
 
 // T of every group (one block per group): T_ii = tau_i, T[0:i, i] = -tau_i T[0:i, 0:i] V[:, 0:i]^T v_i.
 // The RB (RB - 1) / 2 reflector dots are spread over the warps.
-__global__ void __launch_bounds__(256)
-k_bt_tmat(const double* __restrict__ A, int lda, const double* __restrict__ tau, int N,
-          double* __restrict__ Tm, float2* __restrict__ Vff, float2* __restrict__ Tff) {
-  const int g = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+__device__ void bt_tmat(const double* __restrict__ A, int lda, const double* __restrict__ tau, int N, int g,
+                        double* __restrict__ Tm, float2* __restrict__ Vff, float2* __restrict__ Tff) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int nref = N - 2;
   const int k0 = g * RB, nb = min(RB, nref - k0);
   __shared__ double vv[RB][RB];
@@ -1610,8 +1683,8 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   W.Delta = (double*)take((size_t)N * N * sizeof(double));
   W.lam = (double*)take(N * sizeof(double));
   W.lamk = (double*)take(N * sizeof(double));
-  W.lamtmp = (double*)take(N * sizeof(double));
-  W.Dw = (double*)take(N * sizeof(double));
+  W.Df = (float2*)take(N * sizeof(float2));
+  W.zf = (float*)take(N * sizeof(double));
   W.Zw = (double*)take(N * sizeof(double));
   W.Dk = (double*)take(N * sizeof(double));
   W.Zk = (double*)take(N * sizeof(double));
@@ -1624,7 +1697,7 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   float2* Vff = (float2*)take(((size_t)N / RB + 2) * RB * (size_t)N * sizeof(float2));
   W.colk = (int*)take(N * sizeof(int));
   W.cold = (int*)take(N * sizeof(int));
-  W.perm = (int*)take(N * sizeof(int));
+  W.rank = (int*)take(N * sizeof(int));
   W.Kp = (int*)take(N * sizeof(int));
   W.nrot = (int*)take(N * sizeof(int));
   W.gperm = (int*)take(N * sizeof(int));
@@ -1632,7 +1705,8 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   W.mergeof = nullptr;
 
   cudaMemsetAsync(slots, 0xFF, slot_bytes, st);      // every slot empty
-  cudaMemsetAsync(W.Q, 0, (size_t)N * N * sizeof(double), st);
+  // Q and Qtmp (adjacent): a merge's row tiles that straddle its children read zeros outside them
+  cudaMemsetAsync(W.Q, 0, (size_t)((char*)W.Qtmp - (char*)W.Q) + (size_t)N * N * sizeof(double), st);
   cudaMemsetAsync(d, 0, (3 * (size_t)N + 1) * sizeof(double), st);
   k_absmax<<<std::min(N, 304), 256, 0, st>>>(A, lda, N, amax); note_launch();
 
@@ -1663,8 +1737,12 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
     if (ce != cudaSuccess) return 1000 + (int)ce;
   }
   if (marks) cudaEventRecord(marks[0], st);
-  // 2. divide and conquer
-  k_dc_init<<<(N + 255) / 256, 256, 0, st>>>(d, e, N, W.lam, W.Q); note_launch();
+  // 2. divide and conquer; the T matrices of the back-transformation ride on the first launch of small merges
+  const bool ff = sizeof(T) == sizeof(double) && assembly == kAssemblyFF && N >= 3 &&
+                  (size_t)(2 * RB + CB) * N * sizeof(float2) <= 227 * 1024;   // (the double-buffered staging fits)
+  const TmatArgs ta{A, lda, tau, W.Tm, ff ? Vff : nullptr, ff ? Tff : nullptr};
+  int tmat_blocks = N >= 3 ? (N - 2 + RB - 1) / RB : 0;
+  k_dc_init<<<(N + 255) / 256, 256, 0, st>>>(d, e, N, W.lam, W.Q, W.Qtmp); note_launch();
   const Plan& pl = pe->plan;
   const int nlev = (int)pl.level_off.size() - 1;
   for (int lv = 0; lv < nlev; ++lv) {
@@ -1676,43 +1754,32 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
     int kmax = 0;
     for (int q = m0; q < m1; ++q) kmax = std::max(kmax, pl.merges[q].hi - pl.merges[q].lo);
     if (kmax <= DC_SMALL_K) {
-      k_dc_small<<<nm, DC_THREADS, small_smem_bytes(kmax), st>>>(dm, e, N, W, err); note_launch();
+      k_dc_small<<<nm + tmat_blocks, DC_THREADS, small_smem_bytes(kmax), st>>>(dm, nm, e, N, W, err, ta); note_launch();
+      tmat_blocks = 0;
+      std::swap(W.Q, W.Qtmp);
       continue;
     }
     const size_t psmem = prep_smem_bytes(kmax);
     if (psmem > 40 * 1024) cudaFuncSetAttribute(k_dc_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem);
     k_dc_prep<<<nm, DC_THREADS, psmem, st>>>(dm, e, N, W); note_launch();
     k_dc_rot<<<dim3((kmax + 127) / 128, nm), 128, 0, st>>>(dm, N, W); note_launch();
-    // The per-root work is FP64-bound (2 FMA/clk/SM), so the grids use two-warp blocks (one warp per
-    // root) to spread the roots over all SMs.  (One thread per root for the small merges measured
-    // 3x slower: one warp per SM leaves its FP64 dependency chains uncovered.)
+    // The per-root work is FP64-bound, so the grids use two-warp blocks (one warp per root) to spread the
+    // roots over all SMs.  (One thread per root for the small merges measured 3x slower: one warp per SM
+    // leaves its FP64 dependency chains uncovered.)
     k_dc_secular<32><<<(N + 1) / 2, 64, 0, st>>>(dm, dmo, N, W, err); note_launch();
     k_dc_zhat<32><<<(N + 1) / 2, 64, 0, st>>>(dm, dmo, N, W); note_launch();
     k_dc_vecs<32><<<(N + 1) / 2, 64, 0, st>>>(dm, dmo, N, W); note_launch();
     dim3 gg((kmax + DG_T - 1) / DG_T, (kmax + DG_T - 1) / DG_T, nm);
-    k_dc_gemm<<<gg, 256, 0, st>>>(dm, N, W); note_launch();
-    const size_t fsmem = (size_t)kmax * (sizeof(double) + sizeof(long long));
-    if (fsmem > 40 * 1024) cudaFuncSetAttribute(k_dc_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
-    k_dc_finish<<<nm, 256, fsmem, st>>>(dm, N, W); note_launch();
-    k_dc_copy<<<dim3((kmax + 7) / 8, nm), 256, 0, st>>>(dm, N, W); note_launch();
+    k_dc_gemm<<<gg, 256, 0, st>>>(dm, N, W, lv == nlev - 1 ? N - nkeep : 0); note_launch();
+    std::swap(W.Q, W.Qtmp);
   }
   if (marks) cudaEventRecord(marks[1], st);
   // 3. back-transformation of the top nkeep columns (descending eigenvalues)
-  {
-    const int ng = std::max(1, (N - 2 + RB - 1) / RB);
-    if constexpr (sizeof(T) == sizeof(double)) {
-      // (larger orders than the double-buffered staging fits in shared memory take the FP64 kernel)
-      if (assembly == kAssemblyFF && N >= 3 && (size_t)(2 * RB + CB) * N * sizeof(float2) <= 227 * 1024) {
-        k_bt_tmat<<<ng, 256, 0, st>>>(A, lda, tau, N, W.Tm, Vff, Tff); note_launch();
-        const size_t smem = (size_t)(2 * RB + CB) * N * sizeof(float2);
-        if (smem > 40 * 1024) cudaFuncSetAttribute(k_backtransform_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_backtransform_ff<<<(nkeep + CB - 1) / CB, 256, smem, st>>>(Vff, Tff, N, W.Q, W.lam, nkeep, w, U, ldu); note_launch();
-        return cudaGetLastError() == cudaSuccess ? 0 : 4;
-      }
-    }
-    if (N >= 3) {
-      k_bt_tmat<<<ng, 256, 0, st>>>(A, lda, tau, N, W.Tm, nullptr, nullptr); note_launch();
-    }
+  if (ff) {
+    const size_t smem = (size_t)(2 * RB + CB) * N * sizeof(float2);
+    if (smem > 40 * 1024) cudaFuncSetAttribute(k_backtransform_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_backtransform_ff<<<(nkeep + CB - 1) / CB, 256, smem, st>>>(Vff, Tff, N, W.Q, W.lam, nkeep, w, (double*)U, ldu); note_launch();
+  } else {
     const size_t smem = (size_t)(RB + CB) * N * sizeof(double);
     if (smem > 40 * 1024) cudaFuncSetAttribute(k_backtransform<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_backtransform<T><<<(nkeep + CB - 1) / CB, 256, smem, st>>>(A, lda, W.Tm, N, W.Q, W.lam, nkeep, w, U, ldu); note_launch();
