@@ -57,8 +57,7 @@ template <int MD> struct Mode {
   static constexpr int BK = ROWB / ES;                // kernel columns per pipeline stage
   static constexpr int NPART = SPLIT ? 2 : 1;         // operand parts (hi, lo)
   static constexpr int A_TILE = BM * ROWB;            // bytes per A part
-  static constexpr int C_STAGE = BK * 16;             // column coordinates, pair layout
-  static constexpr int W_STAGE = BK * 4;              // mean column
+  static constexpr int C_STAGE = BK * 16;             // column coordinates and mean column, pair layout
   static constexpr int CPT = BK / 8;                  // columns per producer thread and slice
   static constexpr uint32_t SBO = 8 * ROWB;           // 8-row group stride
   static constexpr uint64_t LAYOUT = SPLIT ? 4 : 2;   // descriptor swizzle: 64-byte / 128-byte
@@ -74,6 +73,37 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Shared-memory accesses by 32-bit address.  (The stages' base is rounded up to 1,024 bytes, after which the
+// compiler no longer knows the address space and emits generic loads and stores, which go the way of
+// global ones.)
+__device__ __forceinline__ ulonglong2 lds128(uint32_t a) {
+  ulonglong2 v;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float lds32f(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int lds32(uint32_t a) {
+  int v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts32f(uint32_t a, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -85,7 +115,7 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 }
 // Bounded wait for the completion of the phase with the given parity.  Returns false on timeout
 // or when another role of this CTA already aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_flag, long long limit) {
   for (long long it = 0; it < limit; ++it) {
     uint32_t ok;
     asm volatile(
@@ -94,11 +124,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (*abort_flag) return false;
+    if (lds32(abort_flag)) return false;
   }
-  *abort_flag = 1;
+  sts32(abort_flag, 1);
   return false;
 }
+
+// Position in a ring of S stages: the stage and the parity of its current use.  (Counted up: a modulo of the
+// slice number by the runtime stage count costs about as many instructions as a slice's own work.)
+struct Ring {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int S) {
+    if (++s == S) { s = 0; ph ^= 1; }
+  }
+};
 
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -200,7 +240,6 @@ struct TcParams {
   const C4<float>* Xr;
   int nr;
   const C4<float>* Xc;     // nk * BK columns in pair layout (see k_pad_coords), sentinels beyond nc
-  const float* wcol;       // padded mean column (zeros beyond nc), FP32
   const float* binv;       // FP16 x3: per-column factor undoing the operand scaling (else null)
   int nk;                  // number of K slices per row tile
   int ntiles;              // row tiles of BM rows
@@ -257,9 +296,8 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
   // per stage: A parts (NPART x A_TILE), then B parts (NPART x npad rows x ROWB bytes)
   uint8_t* A_base = smem;
   uint8_t* B_base = A_base + (size_t)S * M::NPART * M::A_TILE;
-  uint8_t* C_base = B_base + (size_t)S * P.b_stage_bytes;            // coordinates
-  uint8_t* W_base = C_base + (size_t)S * M::C_STAGE;                 // mean column
-  uint64_t* bars = reinterpret_cast<uint64_t*>(W_base + (size_t)S * M::W_STAGE);
+  uint8_t* C_base = B_base + (size_t)S * P.b_stage_bytes;            // coordinates and mean column
+  uint64_t* bars = reinterpret_cast<uint64_t*>(C_base + (size_t)S * M::C_STAGE);
   uint64_t* fullA = bars;
   uint64_t* fullB = bars + S;
   uint64_t* fullC = bars + 2 * S;
@@ -268,7 +306,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
   uint64_t* tfree = bars + 4 * S + 1;      // epilogue -> MMA: the accumulator has been read out
   uint64_t* fin = bars + 4 * S + 2;        // MMA issuer: all its MMAs have completed (exit)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 4 * S + 3);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  uint32_t abort_flag = smem_u32(tmem_holder + 1);
   float* mean_part = reinterpret_cast<float*>(tmem_holder + 4);     // [2][8][BM]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -286,7 +324,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     mbar_init(smem_u32(done), 1);
     mbar_init(smem_u32(tfree), NPROD_WARPS);
     mbar_init(smem_u32(fin), 1);
-    *abort_flag = 0;
+    sts32(abort_flag, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -313,6 +351,12 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     long long u = u0;
     int tcount = 0;
     bool ok = true;
+    Ring ring;
+    const uint32_t fullC0 = smem_u32(fullC), fullA0 = smem_u32(fullA);
+    // this thread's parts of a stage: coordinates and mean column of its column group, its two operand rows
+    constexpr int NPAIR = M::CPT / 2;
+    const uint32_t cp0 = smem_u32(C_base) + cg * NPAIR * 32, a0 = smem_u32(A_base), mp0 = smem_u32(mean_part);
+    const uint32_t o0 = sw_off<MD>(pr0, cg * M::CPT * M::ES), o1 = sw_off<MD>(pr1, cg * M::CPT * M::ES);
     while (u < u1) {
       const int tile = (int)(u / P.nk);
       const long long tbeg = (long long)tile * P.nk, tend = tbeg + P.nk;
@@ -329,25 +373,20 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
         rx1 = f2_make(x1.x, x1.x); ry1 = f2_make(x1.y, x1.y); rz1 = f2_make(x1.z, x1.z);
       }
       uint64_t macc0 = 0ull, macc1 = 0ull;          // (even, odd column) partial means, FP32 pairs
-      for (; u < uend; ++u) {
-        const long long it = u - u0;
-        const int s = (int)(it % S);
-        const uint32_t n = (uint32_t)(it / S);
+      for (int left = (int)(uend - u); left > 0; --left, ++u, ring.next(S)) {
+        const int s = ring.s;
         // fullC completes only after the TMA warp saw empty[s] (the MMAs of this stage's previous
         // use are done) and its copies landed, so it also releases the A stage to the producers.
-        ok = mbar_wait(smem_u32(&fullC[s]), n & 1, abort_flag, P.wait_limit);
+        ok = mbar_wait(fullC0 + 8 * s, ring.ph, abort_flag, P.wait_limit);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        constexpr int NPAIR = M::CPT / 2;
-        const uint8_t* cp = C_base + (size_t)s * M::C_STAGE + (size_t)cg * NPAIR * 32;
-        const float* wc = reinterpret_cast<const float*>(W_base + (size_t)s * M::W_STAGE) + cg * M::CPT;
+        const uint32_t cp = cp0 + s * M::C_STAGE;
         // 16-bit modes: one packed word per column pair and part; TF32 modes: one word per column
         uint32_t pk0[2 * NPAIR], pk1[2 * NPAIR], pl0[2 * NPAIR], pl1[2 * NPAIR];
 #pragma unroll
         for (int q = 0; q < NPAIR; ++q) {
-          const ulonglong2 xy = *reinterpret_cast<const ulonglong2*>(cp + q * 32);
-          const uint64_t cz = *reinterpret_cast<const uint64_t*>(cp + q * 32 + 16);
-          const uint64_t w2 = *reinterpret_cast<const uint64_t*>(wc + 2 * q);
+          const ulonglong2 xy = lds128(cp + q * 32), zw = lds128(cp + q * 32 + 16);
+          const uint64_t cz = zw.x, w2 = zw.y;
           const uint64_t k0 = kpair<KER>(rx0, ry0, rz0, xy.x, xy.y, cz);
           const uint64_t k1 = kpair<KER>(rx1, ry1, rz1, xy.x, xy.y, cz);
           macc0 = f2_fma(k0, w2, macc0);
@@ -374,32 +413,30 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
             pk1[q] = f2_bf16(k1);
           }
         }
-        uint8_t* ast = A_base + (size_t)s * M::NPART * M::A_TILE;
-        const int b0 = cg * M::CPT * M::ES;             // byte of this column group within a row
-        const uint32_t o0 = sw_off<MD>(pr0, b0), o1 = sw_off<MD>(pr1, b0);
+        const uint32_t ast = a0 + s * (M::NPART * M::A_TILE);
         if constexpr (M::SPLIT) {   // 8 bytes per row and part (4 fp16 or 2 tf32 values)
-          *reinterpret_cast<uint2*>(ast + o0) = make_uint2(pk0[0], pk0[1]);
-          *reinterpret_cast<uint2*>(ast + o1) = make_uint2(pk1[0], pk1[1]);
-          *reinterpret_cast<uint2*>(ast + M::A_TILE + o0) = make_uint2(pl0[0], pl0[1]);
-          *reinterpret_cast<uint2*>(ast + M::A_TILE + o1) = make_uint2(pl1[0], pl1[1]);
+          sts64(ast + o0, pk0[0], pk0[1]);
+          sts64(ast + o1, pk1[0], pk1[1]);
+          sts64(ast + M::A_TILE + o0, pl0[0], pl0[1]);
+          sts64(ast + M::A_TILE + o1, pl1[0], pl1[1]);
         } else {                    // 16 bytes per row (8 bf16 or 4 tf32 values)
-          *reinterpret_cast<uint4*>(ast + o0) = make_uint4(pk0[0], pk0[1], pk0[2], pk0[3]);
-          *reinterpret_cast<uint4*>(ast + o1) = make_uint4(pk1[0], pk1[1], pk1[2], pk1[3]);
+          sts128(ast + o0, pk0[0], pk0[1], pk0[2], pk0[3]);
+          sts128(ast + o1, pk1[0], pk1[1], pk1[2], pk1[3]);
         }
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&fullA[s]));
+        if (lane == 0) mbar_arrive(fullA0 + 8 * s);
       }
       // ---- end of this CTA's part of the tile: every producer warp arrives here, also on abort
-      float* mp = mean_part + (tcount & 1) * (8 * BM);
-      mp[cg * BM + pr0] = f2_sum(macc0);
-      mp[cg * BM + pr1] = f2_sum(macc1);
-      ok = producers_all(ok && !*abort_flag);
+      const uint32_t mp = mp0 + (tcount & 1) * (8 * BM * 4);
+      sts32f(mp + (cg * BM + pr0) * 4, f2_sum(macc0));
+      sts32f(mp + (cg * BM + pr1) * 4, f2_sum(macc1));
+      ok = producers_all(ok && !lds32(abort_flag));
       if (!ok) break;
       if (qt == 0 && row < P.nr) {
-        float m = mp[rl];
+        float m = lds32f(mp + rl * 4);
 #pragma unroll
-        for (int j = 1; j < 8; ++j) m += mp[j * BM + rl];
+        for (int j = 1; j < 8; ++j) m += lds32f(mp + (j * BM + rl) * 4);
         m *= P.sf2;
         float* dst = P.Out + (size_t)P.wtc * P.ldo + row;
         if (split) atomicAdd(dst, m);
@@ -449,16 +486,14 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     // ------------------------------------------------------------ TMA / bulk-copy producer
     if (lane == 0) {
       long long issued = 0;
-      for (long long u = u0; u < u1; ++u) {
-        const long long it = u - u0;
-        const int s = (int)(it % S);
-        const uint32_t n = (uint32_t)(it / S);
-        const int kt = (int)(u % P.nk);
-        if (!mbar_wait(smem_u32(&empty[s]), (n & 1) ^ 1, abort_flag, P.wait_limit)) break;
+      Ring ring;
+      int kt = (int)(u0 % P.nk);
+      for (long long u = u0; u < u1; ++u, ring.next(S)) {
+        const int s = ring.s;
+        if (!mbar_wait(smem_u32(&empty[s]), ring.ph ^ 1, abort_flag, P.wait_limit)) break;
         const uint32_t cb = smem_u32(&fullC[s]);
-        mbar_expect_tx(cb, M::C_STAGE + M::W_STAGE);
+        mbar_expect_tx(cb, M::C_STAGE);
         bulk_load(smem_u32(C_base + (size_t)s * M::C_STAGE), P.Xc + (size_t)kt * M::BK, M::C_STAGE, cb);
-        bulk_load(smem_u32(W_base + (size_t)s * M::W_STAGE), P.wcol + (size_t)kt * M::BK, M::W_STAGE, cb);
         const uint32_t bb = smem_u32(&fullB[s]);
         mbar_expect_tx(bb, P.b_stage_bytes);
         // B rows (operand columns) 0..npad-1 hold the hi part, npad..2 npad-1 the lo part
@@ -468,9 +503,10 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
                                  ((size_t)part * P.npad + (size_t)b * P.boxh) * M::ROWB),
                         &tmapB, kt * M::BK, part * P.npad + b * P.boxh, bb);
         ++issued;
+        if (++kt == P.nk) kt = 0;
       }
       // on abort, let the copies possibly still in flight (the last S issued) land before exit
-      if (*abort_flag) {
+      if (lds32(abort_flag)) {
         for (long long it = issued > S ? issued - S : 0; it < issued; ++it) {
           const int s = (int)(it % S);
           const uint32_t par = (uint32_t)(it / S) & 1;
@@ -485,6 +521,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
       bool ok = true;
       long long u = u0;
       int tcount = 0;
+      Ring ring;
       while (u < u1 && ok) {
         const long long tend = (u / P.nk + 1) * P.nk;
         const long long uend = u1 < tend ? u1 : tend;
@@ -494,11 +531,10 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         bool first = true;
-        for (; u < uend; ++u) {
-          const long long it = u - u0;
-          const int s = (int)(it % S);
-          const uint32_t n = (uint32_t)(it / S);
-          ok = mbar_wait(smem_u32(&fullA[s]), n & 1, abort_flag, P.wait_limit) && mbar_wait(smem_u32(&fullB[s]), n & 1, abort_flag, P.wait_limit);
+        for (int left = (int)(uend - u); left > 0; --left, ++u, ring.next(S)) {
+          const int s = ring.s;
+          ok = mbar_wait(smem_u32(&fullA[s]), ring.ph, abort_flag, P.wait_limit) &&
+               mbar_wait(smem_u32(&fullB[s]), ring.ph, abort_flag, P.wait_limit);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a0 = smem_u32(A_base + (size_t)s * M::NPART * M::A_TILE);
@@ -533,7 +569,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicExch(P.err, kErrTimeout);
+  if (lds32(abort_flag) && threadIdx.x == 0) atomicExch(P.err, kErrTimeout);
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.tmem_cols) : "memory");
@@ -579,45 +615,25 @@ constexpr int GEMM_BROWS = 2;
 constexpr int GEMM_PF = 3;   // slices of A in flight per producer thread
 constexpr int GEMM_MAX_CHUNK = 128 * GEMM_BROWS;
 
-// Global loads of one 16-wide K slice: A (128 rows) and B (npad operand rows) for this thread,
-// zero outside the matrices.  Thread mapping: A of a TN product and B as (row tid / 4, quad tid % 4
-// of 4 consecutive K values, one 16-byte load when aligned); A of an NN product as (row tid % 128,
-// quad tid / 128), the lanes of a warp on consecutive rows.
-__device__ __forceinline__ void load_slice(const GemmParams& P, int ks, int row0, int col0, int tid, float av[4],
-                                           float bv[GEMM_BROWS][4], bool with_b, bool with_a = true) {
-  const int k0 = ks * 16;
-  if (!with_a) {
-  } else if (P.transA) {
-    const int r = tid >> 2, kq = tid & 3;
-    const int row = row0 + r, k = k0 + kq * 4;
-    const float* src = P.A + (size_t)row * P.lda + k;
-    if (row < P.M && P.vecA && k + 3 < P.K) {
-      const float4 q = *reinterpret_cast<const float4*>(src);
-      av[0] = q.x; av[1] = q.y; av[2] = q.z; av[3] = q.w;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) av[e] = (row < P.M && k + e < P.K) ? src[e] : 0.f;
-    }
+// Global loads of this thread's 4 consecutive K values k .. k + 3 of one operand row.  Rows beyond the matrix
+// are read as its last row (their accumulators are never stored); K values beyond K read as zero.  src
+// points at (row, k).  Thread mapping: A of a TN product and B as (row tid / 4, quad tid % 4), one 16-byte load when
+// aligned; A of an NN product as (row tid % 128, quad tid / 128), the lanes of a warp on consecutive rows.
+__device__ __forceinline__ void load_contig(const float* src, int k, int K, int vec, float v[4]) {
+  if (vec && k + 3 < K) {
+    const float4 q = *reinterpret_cast<const float4*>(src);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   } else {
-    const int r = tid & 127, kq = tid >> 7;
-    const int row = row0 + r, k = k0 + kq * 4;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) av[e] = (row < P.M && k + e < P.K) ? P.A[(size_t)(k + e) * P.lda + row] : 0.f;
+    for (int e = 0; e < 4; ++e) v[e] = k + e < K ? src[e] : 0.f;
   }
-  if (!with_b) return;
+}
+__device__ __forceinline__ void load_strided(const float* src, size_t ld, int k, int K, float v[4]) {
+  if (k + 3 < K) {
+    v[0] = src[0]; v[1] = src[ld]; v[2] = src[2 * ld]; v[3] = src[3 * ld];
+  } else {
 #pragma unroll
-  for (int b = 0; b < GEMM_BROWS; ++b) {
-    const int jr = (tid >> 2) + 128 * b, kq = tid & 3, k = k0 + kq * 4;
-    const int col = col0 + jr;
-    const bool valid = jr < P.cw && col < P.N;
-    const float* src = P.B + (size_t)col * P.ldb + k;
-    if (valid && P.vecB && k + 3 < P.K) {
-      const float4 q = *reinterpret_cast<const float4*>(src);
-      bv[b][0] = q.x; bv[b][1] = q.y; bv[b][2] = q.z; bv[b][3] = q.w;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) bv[b][e] = (valid && k + e < P.K) ? src[e] : 0.f;
-    }
+    for (int e = 0; e < 4; ++e) v[e] = k + e < K ? src[e * ld] : 0.f;
   }
 }
 
@@ -638,7 +654,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
   uint64_t* fin = bars + 2 * S + 2;        // MMA issuer: all its MMAs have completed (exit)
   uint64_t* fullB = bars + 2 * S + 3;      // bulk copy -> MMA: the stage's pre-split B slice landed
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 3 * S + 3);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  uint32_t abort_flag = smem_u32(tmem_holder + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int units = P.ntiles * P.nchunks * P.kchunks;
@@ -652,7 +668,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
     mbar_init(smem_u32(done), 1);
     mbar_init(smem_u32(tfree), NPROD_WARPS);
     mbar_init(smem_u32(fin), 1);
-    *abort_flag = 0;
+    sts32(abort_flag, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -672,7 +688,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
     const int tid = threadIdx.x;                    // 0 .. 511
     long long issued = 0;                           // B copies issued by thread 0
     const int lg = warp & 3, qt = warp >> 2;        // epilogue: TMEM lane group, column-chunk phase
-    long long it = 0;                               // slices produced so far (stage counter)
+    Ring ring;
+    const uint32_t empty0 = smem_u32(empty), fullA0 = smem_u32(fullA), a0 = smem_u32(A_base), b0 = smem_u32(B_base);
+    const int ar_row = P.transA ? (tid >> 2) : (tid & 127), ar_kq = P.transA ? (tid & 3) : (tid >> 7);
+    const uint32_t ao = sw_off<MD>(ar_row, ar_kq * 16);
+    const uint32_t bo = sw_off<MD>(tid >> 2, (tid & 3) * 16);   // (+ 128 rows: a multiple of the swizzle period)
+    const size_t astep = P.transA ? 16 : (size_t)16 * P.lda;
     int tcount = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
@@ -684,67 +705,76 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
       // A is loaded GEMM_PF slices ahead (a ring of registers indexed statically: the loop over
       // the slices is unrolled GEMM_PF times), B one slice ahead when the producers split it, so
       // that the loads' latency overlaps the conversion, the stores and the waits for free stages
-      float ar[GEMM_PF][4], bv[GEMM_BROWS][4];
-      load_slice(P, ks0, row0, col0, tid, ar[0], bv, !preB);
+      int ak = ks0 * 16 + ar_kq * 4, bk = ks0 * 16 + (tid & 3) * 4;      // K of the next loads
+      const size_t arow = min(row0 + ar_row, P.M - 1);
+      const float* ap = P.transA ? P.A + arow * P.lda + ak : P.A + (size_t)ak * P.lda + arow;
+      const float* bp[GEMM_BROWS];
 #pragma unroll
-      for (int q = 1; q < GEMM_PF; ++q)
-        if (ks0 + q < ks1) load_slice(P, ks0 + q, row0, col0, tid, ar[q], bv, false);
+      for (int b = 0; b < GEMM_BROWS; ++b)
+        bp[b] = P.B + (size_t)min(col0 + min((tid >> 2) + 128 * b, P.cw - 1), P.N - 1) * P.ldb + bk;
+      float ar[GEMM_PF][4], bv[GEMM_BROWS][4];
+      auto load_a = [&](float v[4]) {
+        if (P.transA) load_contig(ap, ak, P.K, P.vecA, v);
+        else load_strided(ap, P.lda, ak, P.K, v);
+        ap += astep;
+        ak += 16;
+      };
+      auto load_b = [&](float v[GEMM_BROWS][4]) {
+#pragma unroll
+        for (int b = 0; b < GEMM_BROWS; ++b) {
+          if ((tid >> 2) + 128 * b < P.npad) load_contig(bp[b], bk, P.K, P.vecB, v[b]);
+          bp[b] += 16;
+        }
+        bk += 16;
+      };
+      if (!preB) load_b(bv);
+#pragma unroll
+      for (int q = 0; q < GEMM_PF; ++q)
+        if (ks0 + q < ks1) load_a(ar[q]);
       for (int kb = ks0; kb < ks1 && ok; kb += GEMM_PF) {
 #pragma unroll
         for (int j = 0; j < GEMM_PF; ++j) {
           const int ks = kb + j;
           if (ks >= ks1) break;
-          const int s = (int)(it % S);
-          const uint32_t n = (uint32_t)(it / S);
-          float bn[GEMM_BROWS][4];
-          if (!preB && ks + 1 < ks1) load_slice(P, ks + 1, row0, col0, tid, ar[j], bn, true, false);
-          ok = mbar_wait(smem_u32(&empty[s]), (n & 1) ^ 1, abort_flag, P.wait_limit);
+          const int s = ring.s;
+          ok = mbar_wait(empty0 + 8 * s, ring.ph ^ 1, abort_flag, P.wait_limit);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          uint8_t* ast = A_base + (size_t)s * M::NPART * M::A_TILE;
-          uint8_t* bst = B_base + (size_t)s * P.b_stage_bytes;
+          const uint32_t ast = a0 + s * (M::NPART * M::A_TILE), bst = b0 + s * P.b_stage_bytes;
           if (preB && tid == 0) {
             mbar_expect_tx(smem_u32(&fullB[s]), P.b_stage_bytes);
-            bulk_load(smem_u32(bst), P.Bpre + ((size_t)nc * P.nk + ks) * P.b_stage_bytes, P.b_stage_bytes,
+            bulk_load(bst, P.Bpre + ((size_t)nc * P.nk + ks) * P.b_stage_bytes, P.b_stage_bytes,
                       smem_u32(&fullB[s]));
             ++issued;
           }
           {
-            const int r = P.transA ? (tid >> 2) : (tid & 127);
-            const int kq = P.transA ? (tid & 3) : (tid >> 7);
             uint32_t h[4], l[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(ar[j][e]); l[e] = tf32_rna(ar[j][e] - __uint_as_float(h[e])); }
-            const uint32_t o = sw_off<MD>(r, kq * 16);
-            *reinterpret_cast<uint4*>(ast + o) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(ast + M::A_TILE + o) = make_uint4(l[0], l[1], l[2], l[3]);
+            sts128(ast + ao, h[0], h[1], h[2], h[3]);
+            sts128(ast + M::A_TILE + ao, l[0], l[1], l[2], l[3]);
           }
-          if (ks + GEMM_PF < ks1) load_slice(P, ks + GEMM_PF, row0, col0, tid, ar[j], bn, false);
-#pragma unroll
-          for (int b = 0; b < GEMM_BROWS; ++b) {
-            const int jr = (tid >> 2) + 128 * b;
-            if (preB || jr >= P.npad) break;
-            const int kq = tid & 3;
-            uint32_t h[4], l[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(bv[b][e]); l[e] = tf32_rna(bv[b][e] - __uint_as_float(h[e])); }
-            const uint32_t o = sw_off<MD>(jr, kq * 16);
-            *reinterpret_cast<uint4*>(bst + o) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(bst + (size_t)P.npad * M::ROWB + o) = make_uint4(l[0], l[1], l[2], l[3]);
-          }
+          if (ks + GEMM_PF < ks1) load_a(ar[j]);
           if (!preB) {
 #pragma unroll
-            for (int b = 0; b < GEMM_BROWS; ++b)
+            for (int b = 0; b < GEMM_BROWS; ++b) {
+              if ((tid >> 2) + 128 * b >= P.npad) break;
+              uint32_t h[4], l[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) bv[b][e] = bn[b][e];
+              for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(bv[b][e]); l[e] = tf32_rna(bv[b][e] - __uint_as_float(h[e])); }
+              const uint32_t o = bst + bo + b * 128 * M::ROWB;
+              sts128(o, h[0], h[1], h[2], h[3]);
+              sts128(o + P.npad * M::ROWB, l[0], l[1], l[2], l[3]);
+            }
+            if (ks + 1 < ks1) load_b(bv);
           }
           fence_proxy_async();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&fullA[s]));
-          ++it;
+          if (lane == 0) mbar_arrive(fullA0 + 8 * s);
+          ring.next(S);
         }
       }
-      ok = producers_all(ok && !*abort_flag);
+      ok = producers_all(ok && !lds32(abort_flag));
       if (!ok) break;
       // ---- epilogue of the unit
       ok = mbar_wait(smem_u32(done), tcount & 1, abort_flag, P.wait_limit);
@@ -809,7 +839,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       bool ok = true;
-      long long it = 0;
+      Ring ring;
       int tcount = 0;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const int kc = u / (P.ntiles * P.nchunks);
@@ -819,11 +849,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
-        for (int ks = ks0; ks < ks1; ++ks, ++it) {
-          const int s = (int)(it % S);
-          const uint32_t n = (uint32_t)(it / S);
-          ok = mbar_wait(smem_u32(&fullA[s]), n & 1, abort_flag, P.wait_limit);
-          if (ok && preB) ok = mbar_wait(smem_u32(&fullB[s]), n & 1, abort_flag, P.wait_limit);
+        for (int ks = ks0; ks < ks1; ++ks, ring.next(S)) {
+          const int s = ring.s;
+          ok = mbar_wait(smem_u32(&fullA[s]), ring.ph, abort_flag, P.wait_limit);
+          if (ok && preB) ok = mbar_wait(smem_u32(&fullB[s]), ring.ph, abort_flag, P.wait_limit);
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a0 = smem_u32(A_base + (size_t)s * M::NPART * M::A_TILE);
@@ -855,7 +884,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicExch(P.err, kErrTimeout);
+  if (lds32(abort_flag) && threadIdx.x == 0) atomicExch(P.err, kErrTimeout);
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.tmem_cols) : "memory");
@@ -955,9 +984,10 @@ __global__ void k_pack_b(const float* __restrict__ B, int ldb, int rows, int wtc
   }
 }
 
-// Xp holds the columns' coordinates in pairs: for columns 2p, 2p + 1 the 8 floats
-// {x0, x1, y0, y1, z0, z1, 0, 0} (32 bytes), the layout the producers read as f32x2 operands.
-__global__ void k_pad_coords(const C4<float>* __restrict__ X, int n, int ldp, float* __restrict__ Xp) {
+// Xp holds the columns' coordinates and mean weights in pairs: for columns 2p, 2p + 1 the 8 floats
+// {x0, x1, y0, y1, z0, z1, w0, w1} (32 bytes), the layout the producers read as f32x2 operands.
+__global__ void k_pad_coords(const C4<float>* __restrict__ X, int n, int ldp, const float* __restrict__ wp,
+                             float* __restrict__ Xp) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ldp) return;
   C4<float> c;
@@ -967,7 +997,7 @@ __global__ void k_pad_coords(const C4<float>* __restrict__ X, int n, int ldp, fl
   o[0] = c.x;
   o[2] = c.y;
   o[4] = c.z;
-  o[6] = 0.f;
+  o[6] = wp[i];
 }
 
 // ---------------------------------------------------------------------------- host side
@@ -1014,7 +1044,7 @@ Layout plan_layout(int wtc) {
   L.nbox = (L.npad + 255) / 256;           // npad <= 512: one or two boxes per part
   L.boxh = L.npad / L.nbox;                // a multiple of 8: boxes start on swizzle-atom boundaries
   L.b_stage_bytes = (uint32_t)(M::NPART * L.npad * M::ROWB);
-  const size_t per_stage = (size_t)M::NPART * M::A_TILE + L.b_stage_bytes + M::C_STAGE + M::W_STAGE;
+  const size_t per_stage = (size_t)M::NPART * M::A_TILE + L.b_stage_bytes + M::C_STAGE;
   const size_t fixed = 1024 /*alignment slack*/ + 64 * 8 + 64 + 2 * 8 * BM * 4;
   const size_t budget = 220 * 1024;
   L.stages = (int)std::min<size_t>(8, (budget - fixed) / per_stage);
@@ -1083,7 +1113,6 @@ int launch(int ker, const C4<float>* Xr, int nr, int nc, const void* Bp, int ldp
 
   TcParams P;
   P.Xr = Xr; P.nr = nr; P.Xc = reinterpret_cast<const C4<float>*>(base + g.xc);
-  P.wcol = reinterpret_cast<const float*>(base + g.wp);
   P.binv = M::SCALED ? reinterpret_cast<const float*>(base + g.sc) + L.npad : nullptr;
   P.nk = ldp / M::BK; P.ntiles = (nr + BM - 1) / BM; P.npad = L.npad;
   P.nbox = L.nbox; P.boxh = L.boxh; P.wtc = wtc; P.sf2 = sf2; P.Out = Out; P.ldo = ldo; P.err = err;
@@ -1277,7 +1306,7 @@ int gram_block_tc(int ker, int kind, const C4<float>* Xr, int nr, const C4<float
   if (ldp % BK_MAX != 0 || ldp < nc) return 4;
   const Staging g = staging_layout(nc, width, kind);
   float* xcp = reinterpret_cast<float*>(reinterpret_cast<char*>(const_cast<void*>(Bp)) + g.xc);
-  k_pad_coords<<<(ldp + 255) / 256, 256, 0, st>>>(Xc, nc, ldp, xcp);
+  k_pad_coords<<<(ldp + 255) / 256, 256, 0, st>>>(Xc, nc, ldp, reinterpret_cast<const float*>(reinterpret_cast<const char*>(Bp) + g.wp), xcp);
   note_launch();
   switch (kind) {
     case MD_F16X3: return launch<MD_F16X3>(ker, Xr, nr, nc, Bp, ldp, width, sf2, Out, ldo, err, st);
