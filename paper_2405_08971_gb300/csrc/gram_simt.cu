@@ -58,6 +58,69 @@ template <int CPT, int RPT> struct F32Tile {
   }
 };
 
+// One stage's products: acc += (RPT rows at ty RPT) x (CPT columns F32Tile::col(tx, .)), 16 terms each.
+template <int CPT, int RPT>
+__device__ __forceinline__ void stage_fma(const float* Ks, const float* Bs, int tx, int ty,
+                                          uint64_t (&acc)[CPT][RPT / 2]) {
+  using F = F32Tile<CPT, RPT>;
+#pragma unroll 4
+  for (int kk = 0; kk < GS_KS; ++kk) {
+    const float* kp = Ks + (size_t)kk * F::LDK + ty * RPT;
+    uint64_t kr[RPT / 2];
+    if constexpr (RPT % 4 == 0) {
+#pragma unroll
+      for (int q = 0; q < RPT / 4; ++q) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(kp + 4 * q);
+        kr[2 * q] = v.x;
+        kr[2 * q + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < RPT / 2; ++q) kr[q] = *reinterpret_cast<const uint64_t*>(kp + 2 * q);
+    }
+    const float* bp = Bs + kk * F::LDB;
+    float b[CPT];
+#pragma unroll
+    for (int q = 0; q < F::N4; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(bp + q * 32 + tx * 4);
+      b[4 * q] = v.x; b[4 * q + 1] = v.y; b[4 * q + 2] = v.z; b[4 * q + 3] = v.w;
+    }
+    if constexpr (F::N2) {
+      const float2 v = *reinterpret_cast<const float2*>(bp + F::N4 * 32 + tx * 2);
+      b[4 * F::N4] = v.x; b[4 * F::N4 + 1] = v.y;
+    }
+    if constexpr (CPT % 2) b[CPT - 1] = bp[F::N4 * 32 + F::N2 * 16 + tx];
+#pragma unroll
+    for (int u = 0; u < CPT; ++u) {
+      const uint64_t bb = f2_make(b[u], b[u]);
+#pragma unroll
+      for (int p = 0; p < RPT / 2; ++p) acc[u][p] = f2_fma(kr[p], bb, acc[u][p]);
+    }
+  }
+}
+// The block's tile into Rs (column-major, LDR apart): group 1's part, then group 0's on top of it.
+template <int CPT, int RPT>
+__device__ __forceinline__ void reduce_groups(float* Rs, int g, int tx, int ty, const uint64_t (&acc)[CPT][RPT / 2]) {
+  using F = F32Tile<CPT, RPT>;
+  __syncthreads();
+  for (int half = 1; half >= 0; --half) {
+    if (g == half) {
+#pragma unroll
+      for (int u = 0; u < CPT; ++u)
+#pragma unroll
+        for (int p = 0; p < RPT / 2; ++p) {
+          float lo, hi;
+          f2_split(acc[u][p], lo, hi);
+          float* o = Rs + (size_t)F::col(tx, u) * F::LDR + ty * RPT + 2 * p;
+          if (half == 0) { lo += o[0]; hi += o[1]; }
+          o[0] = lo;
+          o[1] = hi;
+        }
+    }
+    __syncthreads();
+  }
+}
+
 template <int CPT, int RPT>
 __global__ void __launch_bounds__(GS_THREADS, 2)
 k_gram_block_f32(int fn, const C4<float>* __restrict__ Xr, int nr, const C4<float>* __restrict__ Xc, int nc,
@@ -148,40 +211,7 @@ k_gram_block_f32(int fn, const C4<float>* __restrict__ Xr, int nr, const C4<floa
     bar();
     int buf = 0;
     for (int st = first; st < nst; st += step, buf ^= 1) {
-#pragma unroll 4
-      for (int kk = 0; kk < GS_KS; ++kk) {
-        const float* kp = Ks + (size_t)(buf * GS_KS + kk) * F::LDK + ty * RPT;
-        uint64_t kr[RPT / 2];
-        if constexpr (RPT % 4 == 0) {
-#pragma unroll
-          for (int q = 0; q < RPT / 4; ++q) {
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(kp + 4 * q);
-            kr[2 * q] = v.x;
-            kr[2 * q + 1] = v.y;
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < RPT / 2; ++q) kr[q] = *reinterpret_cast<const uint64_t*>(kp + 2 * q);
-        }
-        const float* bp = Bs + (buf * GS_KS + kk) * F::LDB;
-        float b[CPT];
-#pragma unroll
-        for (int q = 0; q < F::N4; ++q) {
-          const float4 v = *reinterpret_cast<const float4*>(bp + q * 32 + tx * 4);
-          b[4 * q] = v.x; b[4 * q + 1] = v.y; b[4 * q + 2] = v.z; b[4 * q + 3] = v.w;
-        }
-        if constexpr (F::N2) {
-          const float2 v = *reinterpret_cast<const float2*>(bp + F::N4 * 32 + tx * 2);
-          b[4 * F::N4] = v.x; b[4 * F::N4 + 1] = v.y;
-        }
-        if constexpr (CPT % 2) b[CPT - 1] = bp[F::N4 * 32 + F::N2 * 16 + tx];
-#pragma unroll
-        for (int u = 0; u < CPT; ++u) {
-          const uint64_t bb = f2_make(b[u], b[u]);
-#pragma unroll
-          for (int p = 0; p < RPT / 2; ++p) acc[u][p] = f2_fma(kr[p], bb, acc[u][p]);
-        }
-      }
+      stage_fma<CPT, RPT>(Ks + (size_t)buf * GS_KS * F::LDK, Bs + buf * GS_KS * F::LDB, tx, ty, acc);
       if (st + step < nst) {
         eval(buf ^ 1);
         store_b(buf ^ 1);
@@ -191,25 +221,9 @@ k_gram_block_f32(int fn, const C4<float>* __restrict__ Xr, int nr, const C4<floa
       bar();
     }
   }
-  // ---- partial tiles: group 1 into shared memory, group 0 on top of it, then the cluster's blocks
+  // ---- partial tiles: the groups' in shared memory, then the cluster's blocks
   float* Rs = reinterpret_cast<float*>(gsm);
-  __syncthreads();
-  for (int half = 1; half >= 0; --half) {
-    if (g == half) {
-#pragma unroll
-      for (int u = 0; u < CPT; ++u)
-#pragma unroll
-        for (int p = 0; p < RPT / 2; ++p) {
-          float lo, hi;
-          f2_split(acc[u][p], lo, hi);
-          float* o = Rs + (size_t)F::col(tx, u) * F::LDR + ty * RPT + 2 * p;
-          if (half == 0) { lo += o[0]; hi += o[1]; }
-          o[0] = lo;
-          o[1] = hi;
-        }
-    }
-    __syncthreads();
-  }
+  reduce_groups<CPT, RPT>(Rs, g, tx, ty, acc);
   cl.sync();
   const int share = (ncol + Z - 1) / Z, c0 = rank * share, c1 = min(ncol, c0 + share);
   for (int e = threadIdx.x; e < (c1 - c0) * BM; e += GS_THREADS) {
@@ -220,6 +234,88 @@ k_gram_block_f32(int fn, const C4<float>* __restrict__ Xr, int nr, const C4<floa
     Out[(size_t)(col0 + c) * ldo + row0 + r] = sf2 * v;
   }
   cl.sync();                                            // no block leaves while its tile is being read
+}
+
+// The plain FP32 factor product C (M x N) = alpha A (M x K) B (K x N) + beta C on the same tiles: a stage's
+// 16 columns of A take the place of the kernel values (the next stage's A and B are in registers while the
+// current one is multiplied), and the K range is split over the cluster in the same way.  B may be FP64
+// (small coefficient blocks), converted when staged.
+// 5,000 x 33 x 257 takes 17.9 us; a cakf_factor_gemm call of that size 49 us, against 84 us with 64 x 64 tiles (79
+// blocks, 64 columns computed).
+template <int CPT, int RPT, class TB>
+__global__ void __launch_bounds__(GS_THREADS, 2)
+k_gemm_nn_f32(int M, int N, int K, float alpha, const float* __restrict__ A, int lda, const TB* __restrict__ B, int ldb,
+              int cw, float beta, float* __restrict__ C, int ldc) {
+  using F = F32Tile<CPT, RPT>;
+  constexpr int BM = F::BM, NA = BM * GS_KS / 128;
+  extern __shared__ __align__(16) unsigned char gsm[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int Z = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int g = threadIdx.x >> 7, t = threadIdx.x & 127, tx = t & 7, ty = t >> 3;
+  float* Ks = reinterpret_cast<float*>(gsm + (size_t)g * F::GROUP);
+  float* Bs = reinterpret_cast<float*>(gsm + (size_t)g * F::GROUP + F::K_BYTES);
+  const int row0 = (int)(blockIdx.x / Z) * BM, col0 = blockIdx.y * cw, ncol = min(cw, N - col0);
+  const int nst = (K + GS_KS - 1) / GS_KS;
+  const int first = rank * 2 + g, step = 2 * Z;
+  auto bar = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); };
+  float ar[NA], br[CPT];
+  auto load = [&](int st) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int e = t + 128 * i, r = e % BM, k = st * GS_KS + e / BM;
+      ar[i] = (row0 + r < M && k < K) ? A[(size_t)k * lda + row0 + r] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < CPT; ++i) {
+      const int e = t + 128 * i, k = st * GS_KS + (e & (GS_KS - 1)), c = e / GS_KS;
+      br[i] = (k < K && c < ncol) ? float(B[(size_t)(col0 + c) * ldb + k]) : 0.f;
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int e = t + 128 * i;
+      Ks[(size_t)(buf * GS_KS + e / BM) * F::LDK + e % BM] = ar[i];
+    }
+#pragma unroll
+    for (int i = 0; i < CPT; ++i) {
+      const int e = t + 128 * i;
+      Bs[(buf * GS_KS + (e & (GS_KS - 1))) * F::LDB + e / GS_KS] = br[i];
+    }
+  };
+  uint64_t acc[CPT][RPT / 2];
+#pragma unroll
+  for (int u = 0; u < CPT; ++u)
+#pragma unroll
+    for (int p = 0; p < RPT / 2; ++p) acc[u][p] = 0ull;
+  if (first < nst) {
+    load(first);
+    store(0);
+    if (first + step < nst) load(first + step);
+    bar();
+    int buf = 0;
+    for (int st = first; st < nst; st += step, buf ^= 1) {
+      stage_fma<CPT, RPT>(Ks + (size_t)buf * GS_KS * F::LDK, Bs + buf * GS_KS * F::LDB, tx, ty, acc);
+      if (st + step < nst) {
+        store(buf ^ 1);
+        if (st + 2 * step < nst) load(st + 2 * step);
+      }
+      bar();
+    }
+  }
+  float* Rs = reinterpret_cast<float*>(gsm);
+  reduce_groups<CPT, RPT>(Rs, g, tx, ty, acc);
+  cl.sync();
+  const int share = (ncol + Z - 1) / Z, c0 = rank * share, c1 = min(ncol, c0 + share);
+  for (int e = threadIdx.x; e < (c1 - c0) * BM; e += GS_THREADS) {
+    const int c = c0 + e / BM, r = e % BM;
+    if (row0 + r >= M) continue;
+    float v = 0.f;
+    for (int q = 0; q < Z; ++q) v += cl.map_shared_rank(Rs, q)[(size_t)c * F::LDR + r];
+    float* o = C + (size_t)(col0 + c) * ldc + row0 + r;
+    *o = beta == 0.f ? alpha * v : fmaf(alpha, v, beta * *o);
+  }
+  cl.sync();
 }
 
 // FP64.  A block owns 32 rows (one per lane) and up to 72 columns, column w + 8 u with warp w.  What
@@ -348,6 +444,22 @@ int pick_cluster(long long tiles, int units, int slots, double fixed, double* co
   return best;
 }
 
+template <int CPT, class TB>
+void launch_nn(int M, int N, int K, float alpha, const float* A, int lda, const TB* B, int ldb, int cw, int nchunk,
+               float beta, float* C, int ldc, cudaStream_t st) {
+  const int units = ((K + GS_KS - 1) / GS_KS + 1) / 2, slots = 2 * 152;
+  double c8, c2;
+  const int t8 = (M + 127) / 128, t2 = (M + 31) / 32;
+  const int z8 = pick_cluster((long long)t8 * nchunk, units, slots, 4.0, &c8);
+  const int z2 = pick_cluster((long long)t2 * nchunk, units, slots, 4.0, &c2);
+  if (2.5 * c8 <= c2)
+    launch_clustered(k_gemm_nn_f32<CPT, 8, TB>, dim3(t8, nchunk), z8, F32Tile<CPT, 8>::SMEM, st, M, N, K, alpha, A, lda,
+                     B, ldb, cw, beta, C, ldc);
+  else
+    launch_clustered(k_gemm_nn_f32<CPT, 2, TB>, dim3(t2, nchunk), z2, F32Tile<CPT, 2>::SMEM, st, M, N, K, alpha, A, lda,
+                     B, ldb, cw, beta, C, ldc);
+}
+
 template <int CPT>
 void launch_f32(int fn, const C4<float>* Xr, int nr, const C4<float>* Xc, int nc, const float* B, int ldb, int width,
                 int cw, int nchunk, float sf2, float* Out, int ldo, cudaStream_t st) {
@@ -395,6 +507,21 @@ void gram_block_fn(int fn, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, con
 }
 
 }  // namespace
+
+template <class TB>
+void gemm_nn_f32(int M, int N, int K, float alpha, const float* A, int lda, const TB* B, int ldb, float beta, float* C,
+                 int ldc, cudaStream_t st) {
+  constexpr int kMaxCols = 64;                          // (72 would spill: A's stage is in registers too)
+  const int nchunk = (N + kMaxCols - 1) / kMaxCols, cw = (N + nchunk - 1) / nchunk, per = (cw + 7) / 8;
+  if (per <= 1) launch_nn<1, TB>(M, N, K, alpha, A, lda, B, ldb, cw, nchunk, beta, C, ldc, st);
+  else if (per <= 3) launch_nn<3, TB>(M, N, K, alpha, A, lda, B, ldb, cw, nchunk, beta, C, ldc, st);
+  else if (per <= 5) launch_nn<5, TB>(M, N, K, alpha, A, lda, B, ldb, cw, nchunk, beta, C, ldc, st);
+  else launch_nn<8, TB>(M, N, K, alpha, A, lda, B, ldb, cw, nchunk, beta, C, ldc, st);
+}
+template void gemm_nn_f32<float>(int, int, int, float, const float*, int, const float*, int, float, float*, int,
+                                 cudaStream_t);
+template void gemm_nn_f32<double>(int, int, int, float, const float*, int, const double*, int, float, float*, int,
+                                  cudaStream_t);
 
 template <class T>
 void gram_block_simt(int ker, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, const T* B, int ldb, int width,

@@ -32,7 +32,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// plain FP32 factor product (gram_simt.cu): C = alpha A B + beta C, B FP32 or FP64
+template <class TB>
+void gemm_nn_f32(int M, int N, int K, float alpha, const float* A, int lda, const TB* B, int ldb, float beta, float* C,
+                 int ldc, cudaStream_t st);
 template <class T> void prep_coords(const double* X, int n, int dim, double scale, C4<T>* out, cudaStream_t st);
+template <class T>
+void prep_coords2(const double* Xr, int nr, const double* Xc, int nc, int dim, double scale, C4<T>* out, cudaStream_t st);
 template <class T> void gather_coords(const C4<T>* X, const int* idx, int m, C4<T>* out, cudaStream_t st);
 template <class T>
 // K(X_o, X_o) s into gram_matvec_slots(m) partial rows of part; with rp > 0 the same launch forms the

@@ -44,6 +44,21 @@ __global__ void k_prep_coords(const double* __restrict__ X, int n, int dim, doub
   out[i] = c;
 }
 
+// The same for the rows and columns of a Gram x block product, into one array (rows first): one launch.
+template <class T>
+__global__ void k_prep_coords2(const double* __restrict__ Xr, int nr, const double* __restrict__ Xc, int nc, int dim,
+                               double scale, C4<T>* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nr + nc) return;
+  const double* x = i < nr ? Xr + (size_t)i * dim : Xc + (size_t)(i - nr) * dim;
+  C4<T> c;
+  c.x = T(scale * x[0]);
+  c.y = dim > 1 ? T(scale * x[1]) : T(0);
+  c.z = dim > 2 ? T(scale * x[2]) : T(0);
+  c.w = T(0);
+  out[i] = c;
+}
+
 template <class T>
 __global__ void k_gather_coords(const C4<T>* __restrict__ X, const int* __restrict__ idx, int m,
                                 C4<T>* __restrict__ out) {
@@ -954,60 +969,6 @@ __global__ void k_reduce_splits(const double* __restrict__ part, int nsplit, int
 }
 
 // ------------------------------------------------------------------------------------------
-// Tiled NN product for tall A: C[M x N] = alpha * A[M x K] * B[K x N] + beta * C (column-major).
-// B may be double (small coefficient matrices); it is converted to T when staged.
-constexpr int NN_BM = 64, NN_BN = 64, NN_BK = 16;
-template <class T, class TB>
-__global__ void __launch_bounds__(256)
-k_gemm_nn(int M, int N, int K, T alpha, const T* __restrict__ A, int lda, const TB* __restrict__ B, int ldb,
-          T beta, T* __restrict__ C, int ldc) {
-  __shared__ T As[NN_BK][NN_BM + 1];
-  __shared__ T Bs[NN_BK][NN_BN + 1];
-  const int m0 = blockIdx.x * NN_BM, n0 = blockIdx.y * NN_BN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  for (int k0 = 0; k0 < K; k0 += NN_BK) {
-    for (int e = threadIdx.x; e < NN_BM * NN_BK; e += 256) {
-      int rr = e % NN_BM, kk = e / NN_BM;
-      As[kk][rr] = (m0 + rr < M && k0 + kk < K) ? A[(size_t)(k0 + kk) * lda + m0 + rr] : T(0);
-    }
-    for (int e = threadIdx.x; e < NN_BK * NN_BN; e += 256) {
-      int kk = e % NN_BK, cc = e / NN_BK;
-      Bs[kk][cc] = (k0 + kk < K && n0 + cc < N) ? T(B[(size_t)(n0 + cc) * ldb + k0 + kk]) : T(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < NN_BK; ++kk) {
-      T aa[4], bb[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) aa[a] = As[kk][ty + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bb[b] = Bs[kk][tx + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(aa[a], bb[b], acc[a][b]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    int rr = m0 + ty + 16 * a;
-    if (rr >= M) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      int c = n0 + tx + 16 * b;
-      if (c >= N) continue;
-      T* p = C + (size_t)c * ldc + rr;
-      *p = (beta == T(0)) ? alpha * acc[a][b] : fma(alpha, acc[a][b], beta * *p);
-    }
-  }
-}
-
 // Small FP64 product with transposes: C = alpha op(A) op(B) + beta C  (sizes up to a few hundred)
 __global__ void k_gemm_small_f64(int ta, int tb, int M, int N, int K, double alpha, const double* __restrict__ A,
                                  int lda, const double* __restrict__ B, int ldb, double beta, double* __restrict__ C,
@@ -1574,6 +1535,11 @@ void prep_coords(const double* X, int n, int dim, double scale, C4<T>* out, cuda
   k_prep_coords<T><<<cdiv(n, 256), 256, 0, st>>>(X, n, dim, scale, out); note_launch();
 }
 template <class T>
+void prep_coords2(const double* Xr, int nr, const double* Xc, int nc, int dim, double scale, C4<T>* out,
+                  cudaStream_t st) {
+  k_prep_coords2<T><<<cdiv((size_t)nr + nc, 256), 256, 0, st>>>(Xr, nr, Xc, nc, dim, scale, out); note_launch();
+}
+template <class T>
 void gather_coords(const C4<T>* X, const int* idx, int m, C4<T>* out, cudaStream_t st) {
   if (m <= 0) return;
   k_gather_coords<T><<<cdiv(m, 256), 256, 0, st>>>(X, idx, m, out); note_launch();
@@ -1827,7 +1793,7 @@ void gemm_nn(int M, int N, int K, T alpha, const T* A, int lda, const TB* B, int
     }
     note_launch();
   } else {
-    k_gemm_nn<T, TB><<<dim3(cdiv(M, NN_BM), cdiv(N, NN_BN)), 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc); note_launch();
+    gemm_nn_f32<TB>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st);
   }
 }
 
@@ -2216,6 +2182,7 @@ void check_finite(const double* x, size_t n, int* err, cudaStream_t st) {
 
 #define INST(T)                                                                                                  \
   template void prep_coords<T>(const double*, int, int, double, C4<T>*, cudaStream_t);                           \
+  template void prep_coords2<T>(const double*, int, const double*, int, int, double, C4<T>*, cudaStream_t);      \
   template void gather_coords<T>(const C4<T>*, const int*, int, C4<T>*, cudaStream_t);                          \
   template void gram_matvec<T>(int, const C4<T>*, const T*, int, T, T*, const T*, int, int, T*, const int*,     \
                                cudaStream_t);                                                                   \
