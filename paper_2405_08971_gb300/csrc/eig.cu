@@ -1314,8 +1314,10 @@ __device__ void bt_tmat(const double* __restrict__ A, int lda, const double* __r
   }
 }
 
-// One block per CB output columns (descending eigenvalue order: column c holds Q[:, N-1-c]).
-template <class T>
+// One block per CB output columns (descending eigenvalue order: column c holds Q[:, N-1-c]); 4, or 2 where 4
+// leave SMs without a block: the columns' FP64 work is what a group costs (N = 288, 256 columns: 64 blocks of
+// 4 took 245 us, 128 blocks of 2 take 200 us).
+template <class T, int CB>
 __global__ void __launch_bounds__(256)
 k_backtransform(const double* __restrict__ A, int lda, const double* __restrict__ Tm, int N,
                 const double* __restrict__ Q, const double* __restrict__ lam, int nkeep,
@@ -1344,11 +1346,11 @@ k_backtransform(const double* __restrict__ A, int lda, const double* __restrict_
     // per lane, summed over the warp by a transposing butterfly (each exchange halves the values a
     // lane holds; 9 adds per lane instead of 5 per dot)
     {
-      static_assert(RB == 16 && CB == 4, "the butterfly assumes 16 reflectors over 8 warps and 4 columns");
+      static_assert(RB == 16 && (CB == 4 || CB == 2), "the butterfly assumes 16 reflectors over 8 warps");
       const int a0 = 2 * warp;
-      double acc[8];
+      double acc[2 * CB];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc[u] = 0.0;
+      for (int u = 0; u < 2 * CB; ++u) acc[u] = 0.0;
       const double* va0 = Vs + (size_t)a0 * N;
       const double* va1 = va0 + N;
       for (int row = r0 + lane; row < N; row += 32) {
@@ -1360,30 +1362,22 @@ k_backtransform(const double* __restrict__ A, int lda, const double* __restrict_
           acc[CB + c] = fma(x1, z, acc[CB + c]);
         }
       }
-      const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+      int idx = 0, o = 16;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const double send = b16 ? acc[u] : acc[u + 4];
-        const double keep = b16 ? acc[u + 4] : acc[u];
-        acc[u] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-      }
+      for (int nv = 2 * CB; nv > 1; nv >>= 1, o >>= 1) {
+        const bool up = lane & o;
+        idx = 2 * idx + up;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const double send = b8 ? acc[u] : acc[u + 2];
-        const double keep = b8 ? acc[u + 2] : acc[u];
-        acc[u] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+        for (int u = 0; u < nv / 2; ++u) {
+          const double send = up ? acc[u] : acc[u + nv / 2];
+          const double keep = up ? acc[u + nv / 2] : acc[u];
+          acc[u] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
       }
-      {
-        const double send = b4 ? acc[0] : acc[1];
-        const double keep = b4 ? acc[1] : acc[0];
-        acc[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-      }
-      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
-      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-      if ((lane & 3) == 0) {
-        const int idx = (b16 ? 4 : 0) + (b8 ? 2 : 0) + (b4 ? 1 : 0);   // = 4 * (a - a0) + c
-        Y[a0 + (idx >> 2)][idx & 3] = acc[0];
-      }
+      const int last = o;                     // lanes that differ below here hold parts of the same dot
+#pragma unroll
+      for (; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+      if ((lane & (2 * last - 1)) == 0) Y[a0 + idx / CB][idx % CB] = acc[0];   // idx = CB (a - a0) + c
     }
     __syncthreads();
     // Yt = T Y (T upper triangular), then Z -= V Yt
@@ -1780,9 +1774,11 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
     if (smem > 40 * 1024) cudaFuncSetAttribute(k_backtransform_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_backtransform_ff<<<(nkeep + CB - 1) / CB, 256, smem, st>>>(Vff, Tff, N, W.Q, W.lam, nkeep, w, (double*)U, ldu); note_launch();
   } else {
-    const size_t smem = (size_t)(RB + CB) * N * sizeof(double);
-    if (smem > 40 * 1024) cudaFuncSetAttribute(k_backtransform<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_backtransform<T><<<(nkeep + CB - 1) / CB, 256, smem, st>>>(A, lda, W.Tm, N, W.Q, W.lam, nkeep, w, U, ldu); note_launch();
+    const int cb = (nkeep + 3) / 4 < 128 ? 2 : 4;
+    auto fn = cb == 2 ? k_backtransform<T, 2> : k_backtransform<T, 4>;
+    const size_t smem = (size_t)(RB + cb) * N * sizeof(double);
+    if (smem > 40 * 1024) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    fn<<<(nkeep + cb - 1) / cb, 256, smem, st>>>(A, lda, W.Tm, N, W.Q, W.lam, nkeep, w, U, ldu); note_launch();
   }
   return cudaGetLastError() == cudaSuccess ? 0 : 4;
 }
