@@ -2191,18 +2191,16 @@ extern "C" int cakf_gram_matmul(int32_t kernel, double log_lx, double log_sf2, i
   if (!g_gs.err) {
     if (cudaMalloc(&g_gs.err, sizeof(int)) != cudaSuccess) return fail(CAKF_ERR_OOM, "scratch allocation failed");
   }
-  cudaMemsetAsync(g_gs.err, 0, sizeof(int), st);
+  if (tcp) cudaMemsetAsync(g_gs.err, 0, sizeof(int), st);   // (only the tensor-core kernels raise it)
   if (precision == CAKF_FP64) {
     C4<double>* xr = (C4<double>*)g_gs.coords;
     C4<double>* xc = xr + nr;
-    prep_coords<double>(Xr, nr, dim, scale, xr, st);
-    prep_coords<double>(Xc, nc, dim, scale, xc, st);
+    prep_coords2<double>(Xr, nr, Xc, nc, dim, scale, xr, st);
     gram_block_simt<double>(kernel, xr, nr, xc, nc, (const double*)B, ldb, width, sf2, (double*)Out, ldo, st);
   } else {
     C4<float>* xr = (C4<float>*)g_gs.coords;
     C4<float>* xc = xr + nr;
-    prep_coords<float>(Xr, nr, dim, scale, xr, st);
-    prep_coords<float>(Xc, nc, dim, scale, xc, st);
+    prep_coords2<float>(Xr, nr, Xc, nc, dim, scale, xr, st);
     if (precision == CAKF_FP32) {
       gram_block_simt<float>(kernel, xr, nr, xc, nc, (const float*)B, ldb, width, (float)sf2, (float*)Out, ldo, st);
     } else {
@@ -2215,10 +2213,10 @@ extern "C" int cakf_gram_matmul(int32_t kernel, double log_lx, double log_sf2, i
       if (r2) return fail(CAKF_ERR_CUDA, "tensor-core Gram x block launch failed (code " + std::to_string(r2) + ")");
     }
   }
+  int e = 0;
+  if (tcp) cudaMemcpyAsync(&e, g_gs.err, sizeof(int), cudaMemcpyDeviceToHost, st);
   cudaError_t ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) return fail(CAKF_ERR_CUDA, std::string("cakf_gram_matmul: ") + cudaGetErrorString(ce));
-  int e = 0;
-  cudaMemcpy(&e, g_gs.err, sizeof(int), cudaMemcpyDeviceToHost);
   if (e == kErrTimeout) return fail(CAKF_ERR_TIMEOUT, "cakf_gram_matmul: a device-side wait exceeded its limit");
   if (e) return fail(CAKF_ERR_NUMERIC, "cakf_gram_matmul: numeric error");
   (void)es;
@@ -2250,22 +2248,22 @@ extern "C" int cakf_factor_gemm(int32_t trans_a, int32_t M, int32_t N, int32_t K
   double* part = reinterpret_cast<double*>(ws.stage);
   double* c64 = part + part_elems;
   int* err = ws.err;
-  cudaMemsetAsync(err, 0, sizeof(int), st);
+  if (mode == 2) cudaMemsetAsync(err, 0, sizeof(int), st);   // (only the tensor-core kernels raise it)
   const int saved = gemm_mode();
   set_gemm_mode(mode);
   set_gemm_err(err);
   if (trans_a) {
     // C = alpha A^T B + beta C through the FP64-output product, converted back to FP32
-    convert_to_f64(C, ldc, M, N, c64, M, st);
+    if (beta != 0.0) convert_to_f64(C, ldc, M, N, c64, M, st);
     gemm_tn<float>(A, lda, M, B, ldb, N, K, alpha, beta, c64, M, part, part_elems, st);
     convert_from_f64<float>(c64, M, M, N, C, ldc, st);
   } else {
     gemm_nn<float, float>(M, N, K, (float)alpha, A, lda, B, ldb, (float)beta, C, ldc, st);
   }
   set_gemm_mode(saved);
-  cudaError_t ce = cudaStreamSynchronize(st);
   int e = 0;
-  if (ce == cudaSuccess) cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost);
+  if (mode == 2) cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  cudaError_t ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) return fail(CAKF_ERR_CUDA, std::string("cakf_factor_gemm: ") + cudaGetErrorString(ce));
   if (e == kErrTimeout) return fail(CAKF_ERR_TIMEOUT, "cakf_factor_gemm: a device-side wait exceeded its limit");
   if (e) return fail(CAKF_ERR_NUMERIC, "cakf_factor_gemm: numeric error");
@@ -2278,24 +2276,46 @@ static int eig_topk_entry(const double* A, int32_t N, int32_t keep, double* w_ou
   if (!is_device_ptr(A) || !is_device_ptr(w_out) || !is_device_ptr(U_out))
     return fail(CAKF_ERR_ARG, "cakf_eig_topk: all arrays must be device arrays of the current device");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  const size_t wb = eig_workspace_bytes(N);
-  double* Aw = nullptr;
-  void* work = nullptr;
-  int* err = nullptr;
-  auto release = [&]() { if (Aw) cudaFree(Aw); if (work) cudaFree(work); if (err) cudaFree(err); };
-  if (cudaMalloc(&Aw, (size_t)N * N * sizeof(double)) != cudaSuccess || cudaMalloc(&work, wb) != cudaSuccess ||
-      cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
-    cudaGetLastError();
-    release();
-    return fail(CAKF_ERR_OOM, "cakf_eig_topk: workspace allocation failed");
+  const size_t wb = (eig_workspace_bytes(N) + 255) & ~size_t(255), ab = ((size_t)N * N * sizeof(double) + 255) & ~size_t(255);
+  // one block of workspace, copy of A and error flag; a block of at most kEigKeepBytes (N = 576 needs 23 MB) is
+  // kept per thread and device for the next call -- allocating and freeing cost 0.25 ms a call, 6 to 10 % of
+  // it -- and given back when the thread ends, changes its device or needs another size
+  constexpr size_t kEigKeepBytes = size_t(64) << 20;
+  struct Kept {
+    void* p = nullptr;
+    size_t bytes = 0;
+    int dev = -1;
+    void drop() { if (p) cudaFree(p); p = nullptr; bytes = 0; }
+    ~Kept() { drop(); }
+  };
+  static thread_local Kept kept;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return fail(CAKF_ERR_CUDA, "cakf_eig_topk: cudaGetDevice"); }
+  const size_t need = wb + ab + 256;
+  void* own = nullptr;
+  char* base;
+  if (kept.p && kept.dev == dev && kept.bytes >= need) {
+    base = (char*)kept.p;
+  } else {
+    kept.drop();
+    void* p = nullptr;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(CAKF_ERR_OOM, "cakf_eig_topk: workspace allocation failed");
+    }
+    if (need <= kEigKeepBytes) { kept.p = p; kept.bytes = need; kept.dev = dev; }
+    else own = p;
+    base = (char*)p;
   }
+  double* Aw = (double*)(base + wb);
+  int* err = (int*)(base + wb + ab);
   cudaMemsetAsync(err, 0, sizeof(int), st);
   cudaMemcpyAsync(Aw, A, (size_t)N * N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-  int rc = eig_sym_topk<double>(Aw, N, N, keep, w_out, U_out, N, work, wb, err, st, nullptr, assembly);
-  cudaError_t ce = cudaStreamSynchronize(st);
+  int rc = eig_sym_topk<double>(Aw, N, N, keep, w_out, U_out, N, base, wb, err, st, nullptr, assembly);
   int e = 0;
-  if (ce == cudaSuccess) cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost);
-  release();
+  cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  cudaError_t ce = cudaStreamSynchronize(st);
+  if (own) cudaFree(own);
   if (rc) return fail(CAKF_ERR_CUDA, "cakf_eig_topk: eigensolver launch failed (code " + std::to_string(rc) + ")");
   if (ce != cudaSuccess) return fail(CAKF_ERR_CUDA, std::string("cakf_eig_topk: ") + cudaGetErrorString(ce));
   if (e == kErrTimeout) return fail(CAKF_ERR_TIMEOUT, "cakf_eig_topk: a device-side wait exceeded its limit");

@@ -108,19 +108,18 @@ extern "C" int cakf_gram_matmul_noalloc(int32_t kernel, double log_lx, double lo
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const double scale = nu_scale_of(kernel) / std::exp(log_lx);
   const double sf2 = std::exp(log_sf2);
-  cudaError_t ce = cudaMemsetAsync(dflag, 0, sizeof(int), st);
+  // (only the tensor-core kernels, with their bounded waits, raise the flag)
+  cudaError_t ce = tcp ? cudaMemsetAsync(dflag, 0, sizeof(int), st) : cudaSuccess;
   if (ce != cudaSuccess) return err(CAKF_ERR_CUDA, std::string("cakf_gram_matmul_noalloc: ") + cudaGetErrorString(ce));
   if (precision == CAKF_FP64) {
     C4<double>* xr = reinterpret_cast<C4<double>*>(s + off_coords);
     C4<double>* xc = xr + nr;
-    prep_coords<double>(Xr, nr, dim, scale, xr, st);
-    prep_coords<double>(Xc, nc, dim, scale, xc, st);
+    prep_coords2<double>(Xr, nr, Xc, nc, dim, scale, xr, st);
     gram_block_simt<double>(kernel, xr, nr, xc, nc, (const double*)B, ldb, width, sf2, (double*)Out, ldo, st);
   } else {
     C4<float>* xr = reinterpret_cast<C4<float>*>(s + off_coords);
     C4<float>* xc = xr + nr;
-    prep_coords<float>(Xr, nr, dim, scale, xr, st);
-    prep_coords<float>(Xc, nc, dim, scale, xc, st);
+    prep_coords2<float>(Xr, nr, Xc, nc, dim, scale, xr, st);
     if (precision == CAKF_FP32) {
       gram_block_simt<float>(kernel, xr, nr, xc, nc, (const float*)B, ldb, width, (float)sf2, (float*)Out, ldo, st);
     } else {
@@ -133,10 +132,10 @@ extern "C" int cakf_gram_matmul_noalloc(int32_t kernel, double log_lx, double lo
                                       std::to_string(r2) + ")");
     }
   }
-  ce = cudaStreamSynchronize(st);
-  if (ce != cudaSuccess) return err(CAKF_ERR_CUDA, std::string("cakf_gram_matmul_noalloc: ") + cudaGetErrorString(ce));
   int e = 0;
-  ce = cudaMemcpy(&e, dflag, sizeof(int), cudaMemcpyDeviceToHost);
+  if (tcp) ce = cudaMemcpyAsync(&e, dflag, sizeof(int), cudaMemcpyDeviceToHost, st);
+  const cudaError_t cs = cudaStreamSynchronize(st);
+  if (ce == cudaSuccess) ce = cs;
   if (ce != cudaSuccess) return err(CAKF_ERR_CUDA, std::string("cakf_gram_matmul_noalloc: ") + cudaGetErrorString(ce));
   if (e == kErrTimeout) return err(CAKF_ERR_TIMEOUT, "cakf_gram_matmul_noalloc: a device-side wait exceeded its limit");
   if (e) return err(CAKF_ERR_NUMERIC, "cakf_gram_matmul_noalloc: numeric error");
