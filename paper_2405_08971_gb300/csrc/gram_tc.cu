@@ -596,6 +596,7 @@ struct GemmParams {
   int M, N, K;
   int ntiles, nchunks, cw, npad;   // row tiles, N chunks of cw columns (npad = cw rounded to 16)
   int nk, kslices, kchunks;        // K slices in all, per chunk, chunks
+  int kfull, ktail;                // chunks kfull .. have ktail slices each
   int vecA, vecB;                  // 16-byte loads allowed along K
   float* C;
   int ldc;
@@ -609,10 +610,17 @@ struct GemmParams {
   const uint8_t* Bpre;             // non-null: B already split and swizzled per (N chunk, K slice)
 };
 
+// K slices [ks0, ks1) of chunk kc
+__device__ __forceinline__ void chunk_range(const GemmParams& P, int kc, int& ks0, int& ks1) {
+  const bool full = kc < P.kfull;
+  ks0 = full ? kc * P.kslices : P.kfull * P.kslices + (kc - P.kfull) * P.ktail;
+  ks1 = min(P.nk, ks0 + (full ? P.kslices : P.ktail));
+}
+
 // Operand rows of B per producer thread and slice: a chunk has at most 256 columns (npad <= 256),
 // 128 rows per pass of the 512 producer threads.
 constexpr int GEMM_BROWS = 2;
-constexpr int GEMM_PF = 3;   // slices of A in flight per producer thread
+constexpr int GEMM_PF = 3;   // slices of A (and of B, when the producers split it) in flight per producer thread
 constexpr int GEMM_MAX_CHUNK = 128 * GEMM_BROWS;
 
 // Global loads of this thread's 4 consecutive K values k .. k + 3 of one operand row.  Rows beyond the matrix
@@ -701,10 +709,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
       const int nc = (u / P.ntiles) % P.nchunks;
       const int kc = u / (P.ntiles * P.nchunks);
       const int row0 = t * BM, col0 = nc * P.cw;
-      const int ks0 = kc * P.kslices, ks1 = min(P.nk, ks0 + P.kslices);
-      // A is loaded GEMM_PF slices ahead (a ring of registers indexed statically: the loop over
-      // the slices is unrolled GEMM_PF times), B one slice ahead when the producers split it, so
-      // that the loads' latency overlaps the conversion, the stores and the waits for free stages
+      int ks0, ks1;
+      chunk_range(P, kc, ks0, ks1);
+      // A, and B when the producers split it, are loaded GEMM_PF slices ahead (a ring of registers indexed
+      // statically: the loop over the slices is unrolled GEMM_PF times), so that the loads' latency
+      // overlaps the conversion, the stores and the waits for free stages
       int ak = ks0 * 16 + ar_kq * 4, bk = ks0 * 16 + (tid & 3) * 4;      // K of the next loads
       const size_t arow = min(row0 + ar_row, P.M - 1);
       const float* ap = P.transA ? P.A + arow * P.lda + ak : P.A + (size_t)ak * P.lda + arow;
@@ -712,7 +721,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
 #pragma unroll
       for (int b = 0; b < GEMM_BROWS; ++b)
         bp[b] = P.B + (size_t)min(col0 + min((tid >> 2) + 128 * b, P.cw - 1), P.N - 1) * P.ldb + bk;
-      float ar[GEMM_PF][4], bv[GEMM_BROWS][4];
+      float ar[GEMM_PF][4], br[GEMM_PF][GEMM_BROWS][4];
       auto load_a = [&](float v[4]) {
         if (P.transA) load_contig(ap, ak, P.K, P.vecA, v);
         else load_strided(ap, P.lda, ak, P.K, v);
@@ -727,10 +736,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
         }
         bk += 16;
       };
-      if (!preB) load_b(bv);
 #pragma unroll
       for (int q = 0; q < GEMM_PF; ++q)
-        if (ks0 + q < ks1) load_a(ar[q]);
+        if (ks0 + q < ks1) {
+          load_a(ar[q]);
+          if (!preB) load_b(br[q]);
+        }
       for (int kb = ks0; kb < ks1 && ok; kb += GEMM_PF) {
 #pragma unroll
         for (int j = 0; j < GEMM_PF; ++j) {
@@ -761,12 +772,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
               if ((tid >> 2) + 128 * b >= P.npad) break;
               uint32_t h[4], l[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(bv[b][e]); l[e] = tf32_rna(bv[b][e] - __uint_as_float(h[e])); }
+              for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(br[j][b][e]); l[e] = tf32_rna(br[j][b][e] - __uint_as_float(h[e])); }
               const uint32_t o = bst + bo + b * 128 * M::ROWB;
               sts128(o, h[0], h[1], h[2], h[3]);
               sts128(o + P.npad * M::ROWB, l[0], l[1], l[2], l[3]);
             }
-            if (ks + 1 < ks1) load_b(bv);
+            if (ks + GEMM_PF < ks1) load_b(br[j]);
           }
           fence_proxy_async();
           __syncwarp();
@@ -843,7 +854,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
       int tcount = 0;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const int kc = u / (P.ntiles * P.nchunks);
-        const int ks0 = kc * P.kslices, ks1 = min(P.nk, ks0 + P.kslices);
+        int ks0, ks1;
+        chunk_range(P, kc, ks0, ks1);
         if (tcount > 0) {
           ok = mbar_wait(smem_u32(tfree), (tcount - 1) & 1, abort_flag, P.wait_limit);
           if (!ok) break;
@@ -925,7 +937,17 @@ __global__ void k_gemm_reduce(const float* __restrict__ part, int kchunks, int M
   const int col = blockIdx.y;
   if (row >= M || col >= N) return;
   double acc = 0.0;
-  for (int kc = 0; kc < kchunks; ++kc) acc += (double)part[((size_t)kc * N + col) * Mpad + row];
+  const float* p = part + (size_t)col * Mpad + row;
+  const size_t step = (size_t)N * Mpad;
+  int kc = 0;
+  for (; kc + 8 <= kchunks; kc += 8) {      // (8 loads in flight, summed in order)
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = p[(size_t)(kc + u) * step];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc += (double)x[u];
+  }
+  for (; kc < kchunks; ++kc) acc += (double)p[(size_t)kc * step];
   OutT* c = C + (size_t)col * ldc + row;
   *c = OutT(alpha * acc + (beta != 0.0 ? beta * (double)*c : 0.0));
 }
@@ -1226,6 +1248,22 @@ int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A
   P.kslices = (P.nk + kchunks - 1) / kchunks;
   P.kchunks = (P.nk + P.kslices - 1) / P.kslices;
   const bool split = force_split || P.kchunks > 1;
+  P.kfull = P.kchunks;
+  P.ktail = P.kslices;
+  // a last round of units with few of them would leave most SMs idle for a whole unit's time: the chunks those
+  // units belong to are cut finer instead, one round of short units (512 x 577 x 65,536: 768 units of 64 slices
+  // are 5.05 rounds of 152 CTAs; 756 of them and 144 of 6 slices are 5.1)
+  const int left = (base_units * P.kchunks) % slots, drop = (left + base_units - 1) / base_units;
+  if (split && left > 0 && left <= slots / 4 && drop < P.kchunks) {
+    const int kfull = P.kchunks - drop, tail = P.nk - kfull * P.kslices;
+    const int ktail = std::max(1, (tail + slots / base_units - 1) / (slots / base_units));
+    const int total = kfull + (tail + ktail - 1) / ktail;
+    if (ktail < P.kslices && (size_t)total * N * P.Mpad <= part_floats) {
+      P.kfull = kfull;
+      P.ktail = ktail;
+      P.kchunks = total;
+    }
+  }
   if (split && !part) return 11;
   P.vecA = transA && lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   P.vecB = ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
