@@ -621,7 +621,6 @@ __device__ __forceinline__ void chunk_range(const GemmParams& P, int kc, int& ks
 // Operand rows of B per producer thread and slice: a chunk has at most 256 columns (npad <= 256),
 // 128 rows per pass of the 512 producer threads.
 constexpr int GEMM_BROWS = 2;
-constexpr int GEMM_PF = 3;   // slices of A (and of B, when the producers split it) in flight per producer thread
 constexpr int GEMM_MAX_CHUNK = 128 * GEMM_BROWS;
 
 // Global loads of this thread's 4 consecutive K values k .. k + 3 of one operand row.  Rows beyond the matrix
@@ -646,7 +645,7 @@ __device__ __forceinline__ void load_strided(const float* src, size_t ld, int k,
   }
 }
 
-template <int MD>
+template <int MD, bool PREB>
 __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
   using M = Mode<MD>;
   static_assert(M::BK == 16 && M::SPLIT && M::TF32, "the GEMM loaders assume 16-wide split-TF32 slices");
@@ -667,7 +666,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int units = P.ntiles * P.nchunks * P.kchunks;
-  const bool preB = P.Bpre != nullptr;
+  constexpr bool preB = PREB;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(smem_u32(&fullA[s]), NPROD_WARPS);
@@ -712,9 +711,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
       const int row0 = t * BM, col0 = nc * P.cw;
       int ks0, ks1;
       chunk_range(P, kc, ks0, ks1);
-      // A, and B when the producers split it, are loaded GEMM_PF slices ahead (a ring of registers indexed
-      // statically: the loop over the slices is unrolled GEMM_PF times), so that the loads' latency
-      // overlaps the conversion, the stores and the waits for free stages
+      // Two slices per turn (one proxy fence and vote for both).  A, and B when the producers split it, are
+      // loaded PF slices ahead (a ring of registers indexed statically: the loop over the slices is unrolled
+      // PF times), so that the loads' latency overlaps the conversion, the stores and the waits for free
+      // stages.  One slice per turn and PF = 3: 512 x 577 x 65,536 306 us, 65,536 x 512 x 576 200 us; this way
+      // 255 and 187 us.
+      constexpr int PF = PREB ? 4 : 2;
       int ak = ks0 * 16 + ar_kq * 4, bk = ks0 * 16 + (tid & 3) * 4;      // K of the next loads
       const size_t arow = min(row0 + ar_row, P.M - 1);
       const float* ap = P.transA ? P.A + arow * P.lda + ak : P.A + (size_t)ak * P.lda + arow;
@@ -722,9 +724,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
 #pragma unroll
       for (int b = 0; b < GEMM_BROWS; ++b)
         bp[b] = P.B + (size_t)min(col0 + min((tid >> 2) + 128 * b, P.cw - 1), P.N - 1) * P.ldb + bk;
-      float ar[GEMM_PF][4], br[GEMM_PF][GEMM_BROWS][4];
+      float ar[PF][4], br[PREB ? 1 : PF][GEMM_BROWS][4];
       auto load_a = [&](float v[4]) {
-        if (P.transA) load_contig(ap, ak, P.K, P.vecA, v);
+        if (!PREB && P.transA) load_contig(ap, ak, P.K, P.vecA, v);
         else load_strided(ap, P.lda, ak, P.K, v);
         ap += astep;
         ak += 16;
@@ -737,53 +739,69 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
         }
         bk += 16;
       };
-#pragma unroll
-      for (int q = 0; q < GEMM_PF; ++q)
-        if (ks0 + q < ks1) {
-          load_a(ar[q]);
-          if (!preB) load_b(br[q]);
+      auto load = [&](int q) {
+        load_a(ar[q]);
+        if constexpr (!PREB) load_b(br[q]);
+      };
+      // slice j of the register ring into stage s (which is free)
+      auto produce = [&](int j, int s, int ks) {
+        const uint32_t ast = a0 + s * (M::NPART * M::A_TILE), bst = b0 + s * P.b_stage_bytes;
+        if (preB && tid == 0) {
+          mbar_expect_tx(smem_u32(&fullB[s]), P.b_stage_bytes);
+          bulk_load(bst, P.Bpre + ((size_t)nc * P.nk + ks) * P.b_stage_bytes, P.b_stage_bytes, smem_u32(&fullB[s]));
+          ++issued;
         }
-      for (int kb = ks0; kb < ks1 && ok; kb += GEMM_PF) {
+        {
+          uint32_t h[4], l[4];
 #pragma unroll
-        for (int j = 0; j < GEMM_PF; ++j) {
-          const int ks = kb + j;
-          if (ks >= ks1) break;
-          const int s = ring.s;
-          ok = mbar_wait(empty0 + 8 * s, ring.ph ^ 1, abort_flag, P.wait_limit);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          const uint32_t ast = a0 + s * (M::NPART * M::A_TILE), bst = b0 + s * P.b_stage_bytes;
-          if (preB && tid == 0) {
-            mbar_expect_tx(smem_u32(&fullB[s]), P.b_stage_bytes);
-            bulk_load(bst, P.Bpre + ((size_t)nc * P.nk + ks) * P.b_stage_bytes, P.b_stage_bytes,
-                      smem_u32(&fullB[s]));
-            ++issued;
-          }
-          {
+          for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(ar[j][e]); l[e] = tf32_rna(ar[j][e] - __uint_as_float(h[e])); }
+          sts128(ast + ao, h[0], h[1], h[2], h[3]);
+          sts128(ast + M::A_TILE + ao, l[0], l[1], l[2], l[3]);
+        }
+        if constexpr (!PREB) {
+#pragma unroll
+          for (int b = 0; b < GEMM_BROWS; ++b) {
+            if ((tid >> 2) + 128 * b >= P.npad) break;
             uint32_t h[4], l[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(ar[j][e]); l[e] = tf32_rna(ar[j][e] - __uint_as_float(h[e])); }
-            sts128(ast + ao, h[0], h[1], h[2], h[3]);
-            sts128(ast + M::A_TILE + ao, l[0], l[1], l[2], l[3]);
+            for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(br[j][b][e]); l[e] = tf32_rna(br[j][b][e] - __uint_as_float(h[e])); }
+            const uint32_t o = bst + bo + b * 128 * M::ROWB;
+            sts128(o, h[0], h[1], h[2], h[3]);
+            sts128(o + P.npad * M::ROWB, l[0], l[1], l[2], l[3]);
           }
-          if (ks + GEMM_PF < ks1) load_a(ar[j]);
-          if (!preB) {
+        }
+      };
 #pragma unroll
-            for (int b = 0; b < GEMM_BROWS; ++b) {
-              if ((tid >> 2) + 128 * b >= P.npad) break;
-              uint32_t h[4], l[4];
+      for (int q = 0; q < PF; ++q)
+        if (ks0 + q < ks1) load(q);
+      for (int kb = ks0; kb < ks1 && ok; kb += PF) {
 #pragma unroll
-              for (int e = 0; e < 4; ++e) { h[e] = tf32_rna(br[j][b][e]); l[e] = tf32_rna(br[j][b][e] - __uint_as_float(h[e])); }
-              const uint32_t o = bst + bo + b * 128 * M::ROWB;
-              sts128(o, h[0], h[1], h[2], h[3]);
-              sts128(o + P.npad * M::ROWB, l[0], l[1], l[2], l[3]);
-            }
-            if (ks + GEMM_PF < ks1) load_b(br[j]);
+        for (int j = 0; j < PF; j += 2) {
+          const int ks = kb + j;
+          if (ks >= ks1) break;
+          const bool two = ks + 1 < ks1;
+          const int s0 = ring.s;
+          ok = mbar_wait(empty0 + 8 * s0, ring.ph ^ 1, abort_flag, P.wait_limit);
+          ring.next(S);
+          const int s1 = ring.s;
+          if (two) {
+            ok = ok && mbar_wait(empty0 + 8 * s1, ring.ph ^ 1, abort_flag, P.wait_limit);
+            ring.next(S);
+          }
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          produce(j, s0, ks);
+          if (ks + PF < ks1) load(j);
+          if (two) {
+            produce(j + 1, s1, ks + 1);
+            if (ks + 1 + PF < ks1) load(j + 1);
           }
           fence_proxy_async();
           __syncwarp();
-          if (lane == 0) mbar_arrive(fullA0 + 8 * s);
-          ring.next(S);
+          if (lane == 0) {
+            mbar_arrive(fullA0 + 8 * s0);
+            if (two) mbar_arrive(fullA0 + 8 * s1);
+          }
         }
       }
       ok = producers_all(ok && !lds32(abort_flag));
@@ -1240,7 +1258,9 @@ int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A
   P.nk = (K + M::BK - 1) / M::BK;
   P.Mpad = P.ntiles * BM;
   const GemmLayout L = gemm_layout(P.npad);
-  const void* fn = (const void*)k_gemm_tc<MD_TF32X3>;
+  const bool pre = !transA && P.ntiles >= 64;   // B (K x N, small) is read by every row tile: split once, copied per stage
+  uint8_t* bp = pre ? bpre_scratch((size_t)P.nchunks * P.nk * L.b_stage_bytes) : nullptr;
+  const void* fn = bp ? (const void*)k_gemm_tc<MD_TF32X3, true> : (const void*)k_gemm_tc<MD_TF32X3, false>;
   cudaError_t ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
   if (ce != cudaSuccess) return 8;
   int per_sm = 0;
@@ -1288,14 +1308,10 @@ int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A
   P.stages = L.stages; P.tmem_cols = L.tmem_cols; P.b_stage_bytes = L.b_stage_bytes;
   P.wait_limit = wait_limit(WAIT_LIMIT);
   P.Bpre = nullptr;
-  if (!transA && P.ntiles >= 64) {
-    // B (K x N, small) is read by every row tile: split it once and copy it per stage in bulk
-    const size_t bytes = (size_t)P.nchunks * P.nk * P.b_stage_bytes;
-    if (uint8_t* bp = bpre_scratch(bytes)) {
-      k_gemm_prep_b<<<P.nchunks * P.nk, 256, 0, st>>>(B, ldb, K, N, P.cw, P.npad, P.nk, P.b_stage_bytes, bp);
-      note_launch();
-      P.Bpre = bp;
-    }
+  if (bp) {
+    k_gemm_prep_b<<<P.nchunks * P.nk, 256, 0, st>>>(B, ldb, K, N, P.cw, P.npad, P.nk, P.b_stage_bytes, bp);
+    note_launch();
+    P.Bpre = bp;
   }
   const int units = P.ntiles * P.nchunks * P.kchunks;
   const int grid = std::min(units, slots);
