@@ -735,15 +735,14 @@ struct Runner {
       // the later residuals, at FP32 rounding level, are no longer independent of the earlier ones.
       // (a recomputed step takes every action from its stored column: no selection, no reorth)
       const bool reorth = !rep && !recompute && (sizeof(T) == 8 || 4 * ic >= m);
-      // CG policy without re-orthogonalisation: k_cg_upd2 writes the next action (the updated
-      // residual) itself, so the selection runs only for the first action
-      const bool fused_select = !rep && !reorth && !recompute;
+      // Without re-orthogonalisation k_cg_upd2 writes the next action (the updated residual, the replayed
+      // or the stored one) itself, so the selection runs only for the first action
       T* dpart1 = (T*)c->dpart;
-      T* dpart2 = dpart1 + (size_t)(B + 4) * ((m + 31) / 32);
+      T* dpart2 = dpart1 + cg_dpart2_offset(m, B, sizeof(T));
       for (int j = 0; j < ic; ++j) {
         T* g = GSk + (size_t)j * m;
-        if (recompute) cg_select<T>(j, Sk(k) + (size_t)j * m, nullptr, m, s, Sk(k), m, c->active, st);
-        else if (!fused_select || j == 0) cg_select<T>(j, r, rep, m, s, Sk(k), m, c->active, st);
+        if (j == 0 || reorth)
+          cg_select<T>(j, recompute ? Sk(k) + (size_t)j * m : r, rep, m, s, Sk(k), m, c->active, st);
         if (reorth) cg_reorth<T>(Qa, m, j, s, m, c->dots2, Sk(k), m, c->active, st);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         bool prof = c->profiling && !recompute && (j % 8 == 0);
@@ -757,9 +756,10 @@ struct Runner {
         cg_combine<T>((const T*)c->part, nsplit, s, T(c->sn2), Mo, m, rp, (const T*)c->tv, T(a2), m, g, V, m, j,
                       (const T*)c->r0v, vcol, dpart1, c->active, st);
         cg_upd1<T>(j, dpart1, c->dots, V, GV, m, s, g, m, dpart2, c->active, st);
-        T* snext = (fused_select && j + 1 < ic) ? Sk(k) + (size_t)(j + 1) * m : nullptr;
+        T* scol = (!reorth && j + 1 < ic) ? Sk(k) + (size_t)(j + 1) * m : nullptr;
         cg_upd2<T>(j, c->dots, dpart2, V, GV, m, r, vcol, s, reorth ? Qa : nullptr, m, bd_tol, rtol2, use_rtol,
-                   c->active, c->eta + (size_t)k * B, c->alpha + (size_t)k * B, c->count + k, snext, st);
+                   c->active, c->eta + (size_t)k * B, c->alpha + (size_t)k * B, c->count + k, recompute ? nullptr : scol,
+                   rep && scol ? rep + (size_t)(j + 1) * m : nullptr, recompute ? scol : nullptr, st);
       }
       sqnorm_acc<T>(r, m, c->rfin + k, st);   // the final (updated) residual
       }

@@ -58,20 +58,22 @@ void gram_block_dlogl_simt(int ker, const C4<T>* Xr, int nr, const C4<T>* Xc, in
 // CG iteration j (non-FP64 modes skip cg_reorth; see the loop in cakf.cu):
 //   cg_combine: g = K s + sn2 s - a2 Mo t, and per-block partials of the first-pass dots (dpart1)
 //   cg_upd1:    first G-orthogonalisation pass, per-block partials of the second-pass dots (dpart2)
-//   cg_upd2:    second pass, scalars, V/GV/v/r update; with Snext the next action s = r
+//   cg_upd2:    second pass, scalars, V/GV/v/r update; the next action s: snext_rep, snext_col or (Snext) r
 template <class T>
 void cg_combine(const T* part, int nsplit, const T* s, T sn2, const T* Mo, int ldm, int r, const T* t, T a2, int m,
                 T* g, const T* V, int ldv, int j, const T* r0, const T* v, T* dpart1, const int* active,
                 cudaStream_t st);
-// elements needed for dpart1 followed by dpart2 at m observations and an action budget
-size_t cg_dpart_elems(int m, int budget);
+// elements needed for dpart1 followed by dpart2 at up to mmax observations and an action budget
+size_t cg_dpart_elems(int mmax, int budget);
+// where dpart2 begins at m observations
+size_t cg_dpart2_offset(int m, int budget, size_t elem_size);
 template <class T>
 void cg_upd1(int j, const T* dpart1, double* dots1, T* V, T* GV, int ldv, const T* s, const T* g, int m,
              T* dpart2, const int* active, cudaStream_t st);
 template <class T>
 void cg_upd2(int j, const double* dots1, const T* dpart2, T* V, T* GV, int ldv, T* r, T* v, T* s, T* Q,
              int m, double bd_tol, double rtol2_r0sq, int use_rtol, int* active, double* eta, double* alpha,
-             int* count, T* Snext, cudaStream_t st);
+             int* count, T* Snext, const double* snext_rep, const T* snext_col, cudaStream_t st);
 template <class T>
 void cg_reorth(const T* Q, int ldq, int j, T* s, int m, double* qd, T* S, int lds, const int* active, cudaStream_t st);
 template <class T>

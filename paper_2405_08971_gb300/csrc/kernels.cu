@@ -321,131 +321,236 @@ k_gram_matvec_f2(const C4<float>* __restrict__ Xo, const float* __restrict__ s, 
   }
 }
 
+// ---- the CG iteration's vector kernels: k_cg_combine, k_cg_upd1, k_cg_upd2.  Each moves a few MB at most, so
+// a chain of L2 round trips and barriers bounds them, and in FP64 the FP64 pipe of the few SMs a small step
+// occupies.  Hence:
+//  - Everything a kernel reads that was written two launches earlier or before (the factor rows, the previous
+//    directions, s, r, v) is loaded before pdl_wait(), while the kernel in front is still running: that kernel
+//    began its own work only after its pdl_wait(), that is after the one before it had completed, and this one
+//    was launched only after that.  These loads bypass L1 (ldcg): the launch in front may be writing a
+//    neighbouring column whose first rows share a cache line with them.
+//  - Sums over the lanes are taken several at a time (warp_sum_t: half the lanes go on with half the values),
+//    which for 8 FP64 sums takes 9 additions per lane instead of 40.
+//  - FP64 with up to CG64_SMALL_MAX observations takes small row blocks (8 rows by 4 columns per warp), which
+//    put the products on four times as many SMs.
+//  - The update kernel also writes the next action where it is known (residual, replayed or stored one).
+// Every FP32 sum keeps its order whatever is loaded ahead.  One iteration with its matvec, before and after:
+// 128 observations, 256 columns, 32 directions (FP64) 32.0 -> 20.0 us; 8,192 x 512 x 64 (FP32) 40.6 -> 32.2 us.
+constexpr int CG64_SMALL_MAX = 2048;
+__device__ __forceinline__ float ldcg_if(bool p, const float* a) {
+  float x;
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n mov.b32 %0, 0;\n @q ld.global.cg.f32 %0, [%1];\n}\n"
+               : "=f"(x) : "l"(a), "r"((int)p) : "memory");
+  return x;
+}
+__device__ __forceinline__ double ldcg_if(bool p, const double* a) {
+  double x;
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n mov.b64 %0, 0;\n @q ld.global.cg.f64 %0, [%1];\n}\n"
+               : "=d"(x) : "l"(a), "r"((int)p) : "memory");
+  return x;
+}
+__device__ __forceinline__ int ldcg_i(const int* a) {
+  int x;
+  asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(x) : "l"(a) : "memory");
+  return x;
+}
+
+// Sums of NV values (a power of two, <= 32) over the lanes of a warp; lane l gets the total of value
+// warp_sum_idx<NV>(l).  Pairs lanes in warp_sum's order, so the totals equal its bit for bit.
+template <int NV> __device__ __forceinline__ int warp_sum_idx(int lane) {
+  int k = 0;
+#pragma unroll
+  for (int h = NV / 2, o = 16; h >= 1; h >>= 1, o >>= 1) k += (lane & o) ? h : 0;
+  return k;
+}
+template <int NV, class T> __device__ __forceinline__ T warp_sum_t(T (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const bool up = lane & o;
+      const T send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  T t = v[0];
+#pragma unroll
+  for (; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
 // g = sum_p part[p] + sn2 * s - a2 * Mo t     (Mo: m x r col-major, ld = ldm).  t is summed from
 // the row-chunk partials of the matvec launch's Mo^T s blocks (tz chunks) into shared memory
-// first.  A block owns CB_ROWS rows: lane = row, each of the CB_WARPS warps takes every
-// CB_WARPS-th column of Mo (coalesced
-// 128-byte column segments, CB_UNROLL independent accumulators), and the warps' sums are added
+// first.  A block owns ROWS rows; a warp takes CC = 32 / ROWS columns of Mo at a time, every CB_WARPS-th
+// group of them (CB_UNROLL independent accumulators), and the warps' sums are added
 // in shared memory.  The block then forms its rows' share of the first dot pass of CG iteration j
 //   q < j: V[:, q] . g ;  j: s . g ;  j+1: s . r0 ;  j+2: g . v ;  j+3: s . s
 // into dpart[q * gridDim.x + block] (summed by k_cg_upd1 in a fixed order, in the working precision:
 // FP64 adds would cost more than the data they sum on this GPU).
-constexpr int CB_ROWS = 32, CB_WARPS = 8, CB_UNROLL = 8;
-template <class T>
+constexpr int CB_ROWS = 32, CB_ROWS_SMALL = 8, CB_WARPS = 8, CB_UNROLL = 8;
+template <class T, int ROWS>
 __global__ void __launch_bounds__(CB_WARPS * 32)
 k_cg_combine(const T* __restrict__ part, int nsplit, const T* __restrict__ s, T sn2,
              const T* __restrict__ Mo, int ldm, int r, const T* __restrict__ tpart, int tz, T a2,
              int m, T* __restrict__ g, const T* __restrict__ V, int ldv, int j, const T* __restrict__ r0,
              const T* __restrict__ v, T* __restrict__ dpart, const int* __restrict__ active) {
+  constexpr int CC = 32 / ROWS;
+  constexpr int PRE = sizeof(T) == 4 ? 64 : (CC > 1 ? 16 : 32);   // columns per thread loaded ahead
+  constexpr int QB = CC > 1 ? 2 : 8;                              // dots per thread whose loads are in flight together
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rl = lane % ROWS, cl = lane / ROWS;
+  const int i = blockIdx.x * ROWS + rl;
+  const bool valid = i < m;
+  const int rv = (r + CC - 1) / CC;                    // groups of CC columns
+  T x0[PRE], xq[QB];
+#pragma unroll
+  for (int e = 0; e < PRE; ++e) {
+    const int col = (warp + e * CB_WARPS) * CC + cl;
+    x0[e] = ldcg_if(valid && col < r, Mo + (size_t)col * ldm + i);
+  }
+#pragma unroll
+  for (int u = 0; u < QB; ++u) {
+    const int q = (warp + u * CB_WARPS) * CC + cl;
+    xq[u] = ldcg_if(valid && q < j, V + (size_t)q * ldv + i);
+  }
+  const T si = ldcg_if(valid, s + i), r0i = ldcg_if(valid, r0 + i), vi = ldcg_if(valid, v + i);
+  const int act = ldcg_i(active);
   pdl_wait();
   pdl_trigger();
-  if (!*active) return;
+  if (!act) return;
   extern __shared__ unsigned char sm_raw[];
-  T* t = reinterpret_cast<T*>(sm_raw);                 // r coefficients
-  __shared__ T red[CB_WARPS][CB_ROWS], redk[CB_WARPS][CB_ROWS];
-  __shared__ T gsh[CB_ROWS];
-  // Every loop below loads a batch of independent values before it uses any of them, so a thread
-  // waits for one L2 round trip per batch rather than one per value (the summation order is the
-  // same as one value at a time).
-  for (int l = threadIdx.x; l < r; l += blockDim.x) {
-    T acc = T(0);
-    int z = 0;
-    for (; z + 8 <= tz; z += 8) {
+  T* t = reinterpret_cast<T*>(sm_raw);                 // r coefficients, zeros up to rv * CC
+  __shared__ T red[CB_WARPS][ROWS], redk[CB_WARPS][ROWS];
+  __shared__ T gsh[ROWS];
+  // the Gram partials: warp w sums slots w, w + CB_WARPS, ... (with CC > 1 CC of them at a time).  Every loop
+  // below loads a batch of independent values before it uses any of them, so a thread waits for one L2 round
+  // trip per batch rather than one per value (the summation order is the same as one value at a time).
+  T kw = T(0);
+  if (valid) {
+    constexpr int ST = CB_WARPS * CC;
+    int p = warp * CC + cl;
+    for (; p + 7 * ST < nsplit; p += 8 * ST) {
       T x[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = tpart[(size_t)(z + u) * r + l];
+      for (int u = 0; u < 8; ++u) x[u] = part[(size_t)(p + u * ST) * m + i];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc += x[u];
+      for (int u = 0; u < 8; ++u) kw += x[u];
     }
-    for (; z < tz; ++z) acc += tpart[(size_t)z * r + l];
+    for (; p < nsplit; p += ST) kw += part[(size_t)p * m + i];
+  }
+  for (int l = threadIdx.x; l < rv * CC; l += blockDim.x) {
+    T acc = T(0);
+    if (l < r) {
+      int z = 0;
+      for (; z + 8 <= tz; z += 8) {
+        T x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = tpart[(size_t)(z + u) * r + l];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += x[u];
+      }
+      for (; z < tz; ++z) acc += tpart[(size_t)z * r + l];
+    }
     t[l] = acc;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * CB_ROWS + lane;
-  const bool valid = i < m;
   T acc[CB_UNROLL];
 #pragma unroll
   for (int u = 0; u < CB_UNROLL; ++u) acc[u] = T(0);
-  if (valid) {
-    int l = warp;
-    constexpr int CB_BATCH = 4;   // groups of CB_UNROLL columns loaded together
-    for (; l + (CB_BATCH * CB_UNROLL - 1) * CB_WARPS < r; l += CB_BATCH * CB_UNROLL * CB_WARPS) {
-      T x[CB_BATCH][CB_UNROLL];
 #pragma unroll
-      for (int b = 0; b < CB_BATCH; ++b)
+  for (int e0 = 0; e0 < PRE; e0 += CB_UNROLL) {
+    const int l = warp + e0 * CB_WARPS;
+    if (l >= rv) break;
+    if (l + (CB_UNROLL - 1) * CB_WARPS < rv) {
 #pragma unroll
-        for (int u = 0; u < CB_UNROLL; ++u) x[b][u] = Mo[(size_t)(l + (b * CB_UNROLL + u) * CB_WARPS) * ldm + i];
-#pragma unroll
-      for (int b = 0; b < CB_BATCH; ++b)
-#pragma unroll
-        for (int u = 0; u < CB_UNROLL; ++u) acc[u] = fma(x[b][u], t[l + (b * CB_UNROLL + u) * CB_WARPS], acc[u]);
-    }
-    for (; l + (CB_UNROLL - 1) * CB_WARPS < r; l += CB_UNROLL * CB_WARPS) {
+      for (int u = 0; u < CB_UNROLL; ++u) acc[u] = fma(x0[e0 + u], t[(l + u * CB_WARPS) * CC + cl], acc[u]);
+    } else {
 #pragma unroll
       for (int u = 0; u < CB_UNROLL; ++u) {
-        const int lu = l + u * CB_WARPS;
-        acc[u] = fma(Mo[(size_t)lu * ldm + i], t[lu], acc[u]);
+        if (l + u * CB_WARPS >= rv) break;
+        acc[0] = fma(x0[e0 + u], t[(l + u * CB_WARPS) * CC + cl], acc[0]);
       }
     }
-    for (; l < r; l += CB_WARPS) acc[0] = fma(Mo[(size_t)l * ldm + i], t[l], acc[0]);
+  }
+  if (valid) {
+    int l = warp + PRE * CB_WARPS;
+    for (; l + (CB_UNROLL - 1) * CB_WARPS < rv; l += CB_UNROLL * CB_WARPS) {
+      T x[CB_UNROLL];
+#pragma unroll
+      for (int u = 0; u < CB_UNROLL; ++u) {
+        const int col = (l + u * CB_WARPS) * CC + cl;
+        x[u] = col < r ? Mo[(size_t)col * ldm + i] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < CB_UNROLL; ++u) acc[u] = fma(x[u], t[(l + u * CB_WARPS) * CC + cl], acc[u]);
+    }
+    for (; l < rv; l += CB_WARPS) {
+      const int col = l * CC + cl;
+      acc[0] = fma(col < r ? Mo[(size_t)col * ldm + i] : T(0), t[col], acc[0]);
+    }
   }
   T lr = T(0);
 #pragma unroll
   for (int u = 0; u < CB_UNROLL; ++u) lr += acc[u];
-  red[warp][lane] = lr;
-  // the Gram partials: warp w sums slots w, w + CB_WARPS, ...
-  T kw = T(0);
-  if (valid) {
-    int p = warp;
-    for (; p + 7 * CB_WARPS < nsplit; p += 8 * CB_WARPS) {
-      T x[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = part[(size_t)(p + u * CB_WARPS) * m + i];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) kw += x[u];
-    }
-    for (; p < nsplit; p += CB_WARPS) kw += part[(size_t)p * m + i];
+  for (int o = ROWS; o < 32; o <<= 1) {
+    lr += __shfl_xor_sync(0xffffffffu, lr, o);
+    kw += __shfl_xor_sync(0xffffffffu, kw, o);
   }
-  redk[warp][lane] = kw;
+  if (cl == 0) {
+    red[warp][rl] = lr;
+    redk[warp][rl] = kw;
+  }
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x < ROWS) {
     T gv = T(0);
     if (valid) {
       T low = T(0), kv = T(0);
 #pragma unroll
-      for (int w = 0; w < CB_WARPS; ++w) { low += red[w][lane]; kv += redk[w][lane]; }
-      kv = fma(sn2, s[i], kv);
+      for (int w = 0; w < CB_WARPS; ++w) { low += red[w][rl]; kv += redk[w][rl]; }
+      kv = fma(sn2, si, kv);
       gv = fma(-a2, low, kv);
       g[i] = gv;
     }
-    gsh[lane] = gv;
+    gsh[rl] = gv;
   }
   __syncthreads();
-  const T gi = gsh[lane];
-  const T si = valid ? s[i] : T(0);
-  constexpr int CB_QB = 8;   // dots per warp whose loads are in flight together
-  for (int q0 = warp; q0 < j + 4; q0 += CB_QB * CB_WARPS) {
-    T pr[CB_QB];
+  const T gi = gsh[rl];
+  for (int q0 = warp * CC; q0 < j + 4; q0 += QB * CB_WARPS * CC) {
+    T pr[QB];
 #pragma unroll
-    for (int u = 0; u < CB_QB; ++u) {
-      const int q = q0 + u * CB_WARPS;
-      T x = T(0);
-      if (valid && q < j + 4) {
-        if (q < j) x = V[(size_t)q * ldv + i] * gi;
-        else if (q == j) x = si * gi;
-        else if (q == j + 1) x = si * r0[i];
-        else if (q == j + 2) x = gi * v[i];
-        else x = si * si;
+    for (int u = 0; u < QB; ++u) {
+      const int q = q0 + u * CB_WARPS * CC + cl;
+      T a = si, b = si;                                // q == j + 3
+      if (q < j) {
+        a = q0 == warp * CC ? xq[u] : (valid ? V[(size_t)q * ldv + i] : T(0));
+        b = gi;
+      } else if (q == j) {
+        b = gi;
+      } else if (q == j + 1) {
+        b = r0i;
+      } else if (q == j + 2) {
+        a = gi;
+        b = vi;
       }
-      pr[u] = x;
+      pr[u] = (valid && q < j + 4) ? a * b : T(0);
     }
+    if constexpr (CC == 1) {
+      const T tot = warp_sum_t<QB>(pr);
+      const int q = q0 + warp_sum_idx<QB>(lane) * CB_WARPS;
+      if (lane % (32 / QB) == 0 && q < j + 4) dpart[(size_t)q * gridDim.x + blockIdx.x] = tot;
+    } else {
 #pragma unroll
-    for (int u = 0; u < CB_QB; ++u) {
-      const int q = q0 + u * CB_WARPS;
-      if (q >= j + 4) break;   // uniform across the warp
-      const T tot = warp_sum(pr[u]);
-      if (lane == 0) dpart[(size_t)q * gridDim.x + blockIdx.x] = tot;
+      for (int u = 0; u < QB; ++u) {
+        const int q = q0 + u * CB_WARPS * CC + cl;
+        if (q - cl >= j + 4) break;   // uniform across the warp
+        T tot = pr[u];
+#pragma unroll
+        for (int o = ROWS / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        if (rl == 0 && q < j + 4) dpart[(size_t)q * gridDim.x + blockIdx.x] = tot;
+      }
     }
   }
 }
@@ -475,12 +580,11 @@ template <class T> __device__ __forceinline__ double dot_part(const T* __restric
 
 // Sum of the per-block partials part[q * nblk + b] over b for q in [0, nq), in a fixed order, into
 // out[q] (shared memory) -- and, if dots != null, into dots[q] in FP64.  Each warp takes UP_QB values
-// of q at a time so that their loads are in flight together.
+// of q at a time, BB partials per lane, so that their loads are in flight together.
 constexpr int UP_QB = 4;
-template <class T>
-__device__ __forceinline__ void sum_partials(const T* __restrict__ part, int nblk, int nq, T* out, double* dots) {
+template <int BB, class T>
+__device__ __forceinline__ void sum_partials_bb(const T* __restrict__ part, int nblk, int nq, T* out, double* dots) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  constexpr int BB = 8;   // partials per lane and value whose loads are in flight together
   for (int q0 = warp * UP_QB; q0 < nq; q0 += nw * UP_QB) {
     T acc[UP_QB];
 #pragma unroll
@@ -500,76 +604,115 @@ __device__ __forceinline__ void sum_partials(const T* __restrict__ part, int nbl
         for (int e = 0; e < BB; ++e)
           if (b0 + 32 * e < nblk) acc[u] += x[u][e];
     }
+    const T t = warp_sum_t<UP_QB>(acc);
+    const int q = q0 + warp_sum_idx<UP_QB>(lane);
+    if (lane % (32 / UP_QB) == 0 && q < nq) {
+      out[q] = t;
+      if (dots) dots[q] = double(t);
+    }
+  }
+}
+template <class T>
+__device__ __forceinline__ void sum_partials(const T* __restrict__ part, int nblk, int nq, T* out, double* dots) {
+  // (FP64 additions that are switched off cost as much as ones that are not: no more of them than partials)
+  if (sizeof(T) == 8 && nblk <= 64) sum_partials_bb<1>(part, nblk, nq, out, dots);
+  else sum_partials_bb<8>(part, nblk, nq, out, dots);
+}
+
+// Row block of the CG update kernels: ROWS rows, UP_THREADS / ROWS threads per row, each summing every
+// (UP_THREADS / ROWS)-th term of a row's sum over the previous directions (the loads of a warp stay coalesced:
+// its 32 threads take 32 consecutive rows of one column).
+constexpr int UP_THREADS = 256, UP_ROWS = 64, UP_ROWS_SMALL = 32;
+constexpr int UP_VB = 8;   // previous directions per thread whose V, GV loads are in flight together
+
+// This thread's values of up to UP_VB directions q0, q0 + SPLIT, ... < j of V and GV.
+template <int SPLIT, class T>
+__device__ __forceinline__ void load_dirs(const T* V, const T* GV, int ldv, int i, bool valid, int q0, int j,
+                                          T (&xv)[UP_VB], T (&xg)[UP_VB]) {
 #pragma unroll
-    for (int u = 0; u < UP_QB; ++u) {
-      const T t = warp_sum(acc[u]);
-      if (lane == 0 && q0 + u < nq) {
-        out[q0 + u] = t;
-        if (dots) dots[q0 + u] = double(t);
-      }
+  for (int e = 0; e < UP_VB; ++e) {
+    const int q = q0 + SPLIT * e;
+    xv[e] = ldcg_if(valid && q < j, V + (size_t)q * ldv + i);
+    xg[e] = ldcg_if(valid && q < j, GV + (size_t)q * ldv + i);
+  }
+}
+// d -= V c, gd -= GV c over this thread's directions sp, sp + SPLIT, ...; the first UP_VB of them are in xv, xg.
+template <int SPLIT, class T>
+__device__ __forceinline__ void orth_pass(const T* V, const T* GV, int ldv, int i, bool valid, int sp, int j,
+                                          const T* c, const T (&xv)[UP_VB], const T (&xg)[UP_VB], T& d, T& gd) {
+#pragma unroll
+  for (int e = 0; e < UP_VB; ++e) {
+    const int q = sp + SPLIT * e;
+    if (q >= j) break;
+    d = fma(-xv[e], c[q], d);
+    gd = fma(-xg[e], c[q], gd);
+  }
+  for (int q0 = sp + SPLIT * UP_VB; q0 < j; q0 += SPLIT * UP_VB) {
+    T yv[UP_VB], yg[UP_VB];
+    load_dirs<SPLIT>(V, GV, ldv, i, valid, q0, j, yv, yg);
+#pragma unroll
+    for (int e = 0; e < UP_VB; ++e) {
+      const int q = q0 + SPLIT * e;
+      if (q >= j) break;
+      d = fma(-yv[e], c[q], d);
+      gd = fma(-yg[e], c[q], gd);
     }
   }
 }
 
-// Row block of the CG update kernels: UP_ROWS rows, UP_SPLIT threads per row, each summing every
-// UP_SPLIT-th term of a row's sum over the previous directions (the loads of a warp stay coalesced:
-// its 32 threads take 32 consecutive rows of one column).
-constexpr int UP_THREADS = 256, UP_ROWS = 64, UP_SPLIT = UP_THREADS / UP_ROWS;
-static_assert(UP_ROWS % 32 == 0, "rows per lane");
-constexpr int UP_VB = 8;   // previous directions per thread whose V, GV loads are in flight together
-
 // First G-orthogonalisation pass of CG iteration j.  The first-pass dots are summed from the
-// combine blocks' partials (FP64, fixed order; block 0 also stores all j + 4 of them in dots1):
+// combine blocks' partials (fixed order; block 0 also stores all j + 4 of them in dots1):
 // c = V^T G s, then d = s - V c, G d = g - GV c, parked unnormalised in column j of V and GV.
 // The block then forms its rows' share of the second-pass dots (q < j: V[:, q] . G d; j: d . G d)
 // into dpart2[q * gridDim.x + block].
-template <class T>
+template <class T, int ROWS>
 __global__ void __launch_bounds__(UP_THREADS)
-k_cg_upd1(int j, const T* __restrict__ dpart1, int nblk1, double* __restrict__ dots1, T* __restrict__ V,
-          T* __restrict__ GV, int ldv, const T* __restrict__ s, const T* __restrict__ g, int m,
-          T* __restrict__ dpart2, const int* __restrict__ active) {
+k_cg_upd1(int j, const T* __restrict__ dpart1, int nblk1, double* __restrict__ dots1, T* V, T* GV, int ldv,
+          const T* __restrict__ s, const T* __restrict__ g, int m, T* __restrict__ dpart2,
+          const int* __restrict__ active) {
+  constexpr int SPLIT = UP_THREADS / ROWS, RT = ROWS / 32;   // (RT rows per lane in the dots)
+  constexpr int NW = UP_THREADS / 32, PQ = 2;                // passes of the dots whose loads are made ahead
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rl = threadIdx.x % ROWS, sp = threadIdx.x / ROWS;
+  const int row0 = blockIdx.x * ROWS;
+  const int i = row0 + rl;
+  const bool valid = i < m;
+  const int nrow = min(ROWS, m - row0);
+  T xv[UP_VB], xg[UP_VB], xd[PQ][UP_QB][RT];
+  load_dirs<SPLIT>(V, GV, ldv, i, valid, sp, j, xv, xg);
+  auto load_dots = [&](int q0, T (&x)[UP_QB][RT]) {
+#pragma unroll
+    for (int u = 0; u < UP_QB; ++u)
+#pragma unroll
+      for (int e = 0; e < RT; ++e) {
+        const int t = lane + 32 * e, q = q0 + u;
+        x[u][e] = ldcg_if(t < nrow && q < j, V + (size_t)q * ldv + row0 + t);
+      }
+  };
+#pragma unroll
+  for (int p = 0; p < PQ; ++p) load_dots((warp + p * NW) * UP_QB, xd[p]);
+  const T si = ldcg_if(valid, s + i);
+  const int act = ldcg_i(active);
   pdl_wait();
   pdl_trigger();
-  if (!*active) return;
+  if (!act) return;
   __shared__ T c[1024 + 4];
-  __shared__ T sd[UP_SPLIT][UP_ROWS], sgd[UP_SPLIT][UP_ROWS];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  __shared__ T sd[SPLIT][ROWS], sgd[SPLIT][ROWS];
+  const T gi = sp == 0 && valid ? g[i] : T(0);
   sum_partials(dpart1, nblk1, (blockIdx.x == 0) ? j + 4 : j, c, blockIdx.x == 0 ? dots1 : nullptr);
   __syncthreads();
-  const int rl = threadIdx.x % UP_ROWS, sp = threadIdx.x / UP_ROWS;
-  const int row0 = blockIdx.x * UP_ROWS;
-  const int i = row0 + rl;
   T d = T(0), gd = T(0);
-  if (i < m) {
-    for (int q0 = sp; q0 < j; q0 += UP_SPLIT * UP_VB) {
-      T xv[UP_VB], xg[UP_VB];
-#pragma unroll
-      for (int e = 0; e < UP_VB; ++e) {
-        const int q = q0 + UP_SPLIT * e;
-        xv[e] = q < j ? V[(size_t)q * ldv + i] : T(0);
-        xg[e] = q < j ? GV[(size_t)q * ldv + i] : T(0);
-      }
-#pragma unroll
-      for (int e = 0; e < UP_VB; ++e) {
-        const int q = q0 + UP_SPLIT * e;
-        if (q < j) {
-          const T cq = c[q];
-          d = fma(-xv[e], cq, d);
-          gd = fma(-xg[e], cq, gd);
-        }
-      }
-    }
-  }
+  orth_pass<SPLIT>(V, GV, ldv, i, valid, sp, j, c, xv, xg, d, gd);
   sd[sp][rl] = d;
   sgd[sp][rl] = gd;
   __syncthreads();
   if (sp == 0) {
     d = T(0); gd = T(0);
-    if (i < m) {
-      d = s[i];
-      gd = g[i];
+    if (valid) {
+      d = si;
+      gd = gi;
 #pragma unroll
-      for (int u = 0; u < UP_SPLIT; ++u) { d += sd[u][rl]; gd += sgd[u][rl]; }
+      for (int u = 0; u < SPLIT; ++u) { d += sd[u][rl]; gd += sgd[u][rl]; }
       V[(size_t)j * ldv + i] = d;
       GV[(size_t)j * ldv + i] = gd;
     }
@@ -577,37 +720,30 @@ k_cg_upd1(int j, const T* __restrict__ dpart1, int nblk1, double* __restrict__ d
     sgd[0][rl] = gd;
   }
   __syncthreads();
-  const int nrow = min(UP_ROWS, m - row0);
-  constexpr int RT = UP_ROWS / 32;   // rows per lane
-  for (int q0 = warp * UP_QB; q0 <= j; q0 += nw * UP_QB) {
+  T dl[RT], gl[RT];
+#pragma unroll
+  for (int e = 0; e < RT; ++e) { dl[e] = sd[0][lane + 32 * e]; gl[e] = sgd[0][lane + 32 * e]; }
+  auto dots = [&](int q0, const T (&x)[UP_QB][RT]) {
     T acc[UP_QB];
 #pragma unroll
-    for (int u = 0; u < UP_QB; ++u) acc[u] = T(0);
-    T x[UP_QB][RT];
-#pragma unroll
-    for (int u = 0; u < UP_QB; ++u)
-#pragma unroll
-      for (int e = 0; e < RT; ++e) {
-        const int t = lane + 32 * e, q = q0 + u;
-        x[u][e] = (t < nrow && q < j) ? V[(size_t)q * ldv + row0 + t] : T(0);
-      }
-#pragma unroll
-    for (int e = 0; e < RT; ++e) {
-      const int t = lane + 32 * e;
-      if (t >= nrow) continue;
-      const T gt = sgd[0][t];
-#pragma unroll
-      for (int u = 0; u < UP_QB; ++u) {
-        const int q = q0 + u;
-        if (q < j) acc[u] = fma(x[u][e], gt, acc[u]);
-        else if (q == j) acc[u] = fma(sd[0][t], gt, acc[u]);
-      }
-    }
-#pragma unroll
     for (int u = 0; u < UP_QB; ++u) {
-      const T t = warp_sum(acc[u]);
-      if (lane == 0 && q0 + u <= j) dpart2[(size_t)(q0 + u) * gridDim.x + blockIdx.x] = t;
+      acc[u] = T(0);
+#pragma unroll
+      for (int e = 0; e < RT; ++e) acc[u] = fma(q0 + u == j ? dl[e] : x[u][e], gl[e], acc[u]);
     }
+    const T t = warp_sum_t<UP_QB>(acc);
+    const int q = q0 + warp_sum_idx<UP_QB>(lane);
+    if (lane % (32 / UP_QB) == 0 && q <= j) dpart2[(size_t)q * gridDim.x + blockIdx.x] = t;
+  };
+#pragma unroll
+  for (int p = 0; p < PQ; ++p) {
+    const int q0 = (warp + p * NW) * UP_QB;
+    if (q0 <= j) dots(q0, xd[p]);
+  }
+  for (int q0 = (warp + PQ * NW) * UP_QB; q0 <= j; q0 += NW * UP_QB) {
+    T x[UP_QB][RT];
+    load_dots(q0, x);
+    dots(q0, x);
   }
 }
 
@@ -615,94 +751,98 @@ k_cg_upd1(int j, const T* __restrict__ dpart1, int nblk1, double* __restrict__ d
 //   c2 = V^T G d;  d <- d - V c2;  eta = d^T G d - |c2|^2;  alpha = s^T (r0 - G v) = s^T r0 - g^T v;
 //   V[:, j] = d / sqrt(eta);  GV[:, j] = G d / sqrt(eta);  v += (alpha / eta) d;  r -= (alpha / eta) G d.
 // Every block sums the second-pass dots from the k_cg_upd1 partials, recomputes the scalars and
-// takes the same stop decision.  With Snext (CG policy, no re-orthogonalisation) the next action
-// -- the updated residual -- is written to s and to column j + 1 of S here.
-template <class T>
+// takes the same stop decision.  The next action, if it is known by then, is written to s here: a given one
+// (snext_rep: replayed actions; snext_col: a stored column), or, with only Snext (CG policy without
+// re-orthogonalisation), the updated residual; Snext also receives it as column j + 1 of S.
+template <class T, int ROWS>
 __global__ void __launch_bounds__(UP_THREADS)
 k_cg_upd2(int j, const double* __restrict__ dots1, const T* __restrict__ dpart2, int nblk2,
-          T* __restrict__ V, T* __restrict__ GV, int ldv, T* __restrict__ r, T* __restrict__ v,
-          T* __restrict__ s, T* __restrict__ Q, int m,
-          double bd_tol, double rtol2_r0sq, int use_rtol, int* __restrict__ active,
+          T* V, T* GV, int ldv, T* r, T* v, T* s, T* __restrict__ Q, int m,
+          double bd_tol, double rtol2_r0sq, int use_rtol, int* active,
           double* __restrict__ eta_out, double* __restrict__ alpha_out, int* __restrict__ count,
-          T* __restrict__ Snext) {
+          T* Snext, const double* __restrict__ snext_rep, const T* snext_col) {
+  constexpr int SPLIT = UP_THREADS / ROWS;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rl = threadIdx.x % ROWS, sp = threadIdx.x / ROWS;
+  const int i = blockIdx.x * ROWS + rl;
+  const bool valid = i < m, own = sp == 0 && valid;
+  T xv[UP_VB], xg[UP_VB];
+  load_dirs<SPLIT>(V, GV, ldv, i, valid, sp, j, xv, xg);
+  const T ri = ldcg_if(own, r + i), vi = ldcg_if(own, v + i), si = ldcg_if(own && Q, s + i);
+  T sn = T(0);
+  if (snext_rep) sn = T(ldcg_if(own, snext_rep + i));
+  else if (snext_col) sn = ldcg_if(own, snext_col + i);
+  const int act = ldcg_i(active);
   pdl_wait();
   pdl_trigger();
-  if (!*active) return;
+  if (!act) return;
   __shared__ T c[1024 + 4];
-  __shared__ double sh[3];
+  __shared__ double sh[2];
   __shared__ T shc[3];             // 1 / sqrt(eta), alpha / eta, 1 / |s| (formed once, in FP64)
-  __shared__ T sd[UP_SPLIT][UP_ROWS], sgd[UP_SPLIT][UP_ROWS];
+  __shared__ int stop_sh;
+  __shared__ T sd[SPLIT][ROWS], sgd[SPLIT][ROWS];
+  const T dj = ldcg_if(own, V + (size_t)j * ldv + i), gdj = ldcg_if(own, GV + (size_t)j * ldv + i);
+  double sg = 0.0, a1 = 0.0, a2 = 0.0, ss = 0.0;
+  if (warp < 4) {
+    sg = ldcg_if(true, dots1 + j);
+    a1 = ldcg_if(true, dots1 + j + 1);
+    a2 = ldcg_if(true, dots1 + j + 2);
+    ss = ldcg_if(true, dots1 + j + 3);
+  }
   sum_partials(dpart2, nblk2, j + 1, c, nullptr);
   __syncthreads();
-  double ccp = 0.0;
-  for (int q = threadIdx.x; q < j; q += blockDim.x) ccp = fma(double(c[q]), double(c[q]), ccp);
-  const double cc = block_sum(ccp);
-  if (threadIdx.x == 0) {
-    const double sg = dots1[j];
-    const double eta = double(c[j]) - cc;
-    const double alpha = dots1[j + 1] - dots1[j + 2];
-    int stop = !(eta > bd_tol * sg) || !isfinite(eta) || !isfinite(alpha);
-    if (use_rtol && dots1[j + 3] <= rtol2_r0sq) stop = 1;
-    sh[0] = eta; sh[1] = alpha; sh[2] = stop;
-    if (!stop) {
-      shc[0] = T(1.0 / sqrt(eta));
-      shc[1] = T(alpha / eta);
-      shc[2] = T(1.0 / sqrt(dots1[j + 3]));
+  // The scalars, one warp (on an SM partition of its own) per FP64 division or root: 0: 1 / sqrt(eta),
+  // 1: alpha / eta, 2: 1 / |s|, 3: the stop decision.
+  if (warp < 4) {
+    double eta = 0.0;
+    if (warp != 2) {
+      double ccp = 0.0;
+      for (int q = lane; q < j; q += 32) ccp = fma(double(c[q]), double(c[q]), ccp);
+      eta = double(c[j]) - warp_sum(ccp);
     }
-  }
-  __syncthreads();
-  const double eta = sh[0], alpha = sh[1];
-  const int rl = threadIdx.x % UP_ROWS, sp = threadIdx.x / UP_ROWS;
-  const int i = blockIdx.x * UP_ROWS + rl;
-  if (sh[2] != 0.0) {
-    // breakdown / converged: this direction is not used; clear the parked column
-    if (sp == 0 && i < m) { V[(size_t)j * ldv + i] = T(0); GV[(size_t)j * ldv + i] = T(0); }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *active = 0;
-    return;
+    const double alpha = a1 - a2;
+    if (lane == 0) {
+      if (warp == 0) { sh[0] = eta; shc[0] = T(1.0 / sqrt(eta)); }
+      else if (warp == 1) { sh[1] = alpha; shc[1] = T(alpha / eta); }
+      else if (warp == 2) { if (Q) shc[2] = T(1.0 / sqrt(ss)); }
+      else {
+        int stop = !(eta > bd_tol * sg) || !isfinite(eta) || !isfinite(alpha);
+        if (use_rtol && ss <= rtol2_r0sq) stop = 1;
+        stop_sh = stop;
+      }
+    }
   }
   T d = T(0), gd = T(0);
-  if (i < m) {
-    for (int q0 = sp; q0 < j; q0 += UP_SPLIT * UP_VB) {
-      T xv[UP_VB], xg[UP_VB];
-#pragma unroll
-      for (int e = 0; e < UP_VB; ++e) {
-        const int q = q0 + UP_SPLIT * e;
-        xv[e] = q < j ? V[(size_t)q * ldv + i] : T(0);
-        xg[e] = q < j ? GV[(size_t)q * ldv + i] : T(0);
-      }
-#pragma unroll
-      for (int e = 0; e < UP_VB; ++e) {
-        const int q = q0 + UP_SPLIT * e;
-        if (q < j) {
-          const T cq = c[q];
-          d = fma(-xv[e], cq, d);
-          gd = fma(-xg[e], cq, gd);
-        }
-      }
-    }
-  }
+  orth_pass<SPLIT>(V, GV, ldv, i, valid, sp, j, c, xv, xg, d, gd);
   sd[sp][rl] = d;
   sgd[sp][rl] = gd;
   __syncthreads();
-  if (sp == 0 && i < m) {
-    d = V[(size_t)j * ldv + i];
-    gd = GV[(size_t)j * ldv + i];
+  if (stop_sh) {
+    // breakdown / converged: this direction is not used; clear the parked column
+    if (own) { V[(size_t)j * ldv + i] = T(0); GV[(size_t)j * ldv + i] = T(0); }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *active = 0;
+    return;
+  }
+  if (own) {
+    d = dj;
+    gd = gdj;
 #pragma unroll
-    for (int u = 0; u < UP_SPLIT; ++u) { d += sd[u][rl]; gd += sgd[u][rl]; }
+    for (int u = 0; u < SPLIT; ++u) { d += sd[u][rl]; gd += sgd[u][rl]; }
     const T inv = shc[0];
     const T coef = shc[1];
     V[(size_t)j * ldv + i] = d * inv;
     GV[(size_t)j * ldv + i] = gd * inv;
-    v[i] = fma(coef, d, v[i]);
-    const T rn = fma(-coef, gd, r[i]);
+    v[i] = fma(coef, d, vi);
+    const T rn = fma(-coef, gd, ri);
     r[i] = rn;
-    if (Q) Q[(size_t)j * ldv + i] = s[i] * shc[2];
-    if (Snext) {
-      s[i] = rn;
-      Snext[i] = rn;
+    if (Q) Q[(size_t)j * ldv + i] = si * shc[2];
+    if (snext_rep || snext_col || Snext) {
+      const T val = snext_rep || snext_col ? sn : rn;
+      s[i] = val;
+      if (Snext) Snext[i] = val;
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) { eta_out[j] = eta; alpha_out[j] = alpha; *count = j + 1; }
+  if (blockIdx.x == 0 && threadIdx.x == 0) { eta_out[j] = sh[0]; alpha_out[j] = sh[1]; *count = j + 1; }
 }
 
 // Projection coefficients of the action on the orthonormal basis Q of the previous actions:
@@ -1596,30 +1736,46 @@ void gram_matvec(int ker, const C4<T>* Xo, const T* s, int m, T sf2, T* part, co
   }
 }
 
+static bool cg_small(int m, size_t es) { return es == 8 && m <= CG64_SMALL_MAX; }
+static int cg_blocks1(int m, size_t es) { return (int)cdiv(m, cg_small(m, es) ? CB_ROWS_SMALL : CB_ROWS); }
+static int cg_blocks2(int m, size_t es) { return (int)cdiv(m, cg_small(m, es) ? UP_ROWS_SMALL : UP_ROWS); }
 template <class T>
 void cg_combine(const T* part, int nsplit, const T* s, T sn2, const T* Mo, int ldm, int r, const T* t, T a2, int m,
                 T* g, const T* V, int ldv, int j, const T* r0, const T* v, T* dpart1, const int* active,
                 cudaStream_t st) {
   const int tz = std::max(1, (m + GV_CHUNK - 1) / GV_CHUNK);
-  launch_pdl(k_cg_combine<T>, dim3(cdiv(m, CB_ROWS)), dim3(CB_WARPS * 32), std::max(r, 1) * sizeof(T), st, 
-      part, nsplit, s, sn2, Mo, ldm, r, t, tz, a2, m, g, V, ldv, j, r0, v, dpart1, active);
+  auto fn = k_cg_combine<T, CB_ROWS>;
+  const size_t smem = std::max(cg_small(m, sizeof(T)) ? (r + 3) / 4 * 4 : r, 1) * sizeof(T);
+  if constexpr (sizeof(T) == 8)
+    if (cg_small(m, 8)) fn = k_cg_combine<T, CB_ROWS_SMALL>;
+  launch_pdl(fn, dim3(cg_blocks1(m, sizeof(T))), dim3(CB_WARPS * 32), smem, st, part, nsplit, s, sn2, Mo, ldm,
+              r, t, tz, a2, m, g, V, ldv, j, r0, v, dpart1, active);
 }
-size_t cg_dpart_elems(int m, int budget) {
-  return (size_t)(budget + 4) * cdiv(std::max(m, 1), CB_ROWS) + (size_t)(budget + 1) * cdiv(std::max(m, 1), UP_ROWS);
+size_t cg_dpart2_offset(int m, int budget, size_t elem_size) { return (size_t)(budget + 4) * cg_blocks1(m, elem_size); }
+size_t cg_dpart_elems(int mmax, int budget) {
+  // (the small FP64 blocks of a step with fewer observations can outnumber the blocks of the largest step)
+  const int mb = std::max(mmax, 1), ms = std::min(mb, CG64_SMALL_MAX);
+  return (size_t)(budget + 4) * std::max(cg_blocks1(mb, 4), cg_blocks1(ms, 8)) +
+         (size_t)(budget + 1) * std::max(cg_blocks2(mb, 4), cg_blocks2(ms, 8));
 }
 template <class T>
 void cg_upd1(int j, const T* dpart1, double* dots1, T* V, T* GV, int ldv, const T* s, const T* g, int m,
              T* dpart2, const int* active, cudaStream_t st) {
-  launch_pdl(k_cg_upd1<T>, dim3(cdiv(m, UP_ROWS)), dim3(UP_THREADS), 0, st, j, dpart1, (int)cdiv(m, CB_ROWS), dots1, V, GV, ldv, s, g, m,
-                                                        dpart2, active);
+  auto fn = k_cg_upd1<T, UP_ROWS>;
+  if constexpr (sizeof(T) == 8)
+    if (cg_small(m, 8)) fn = k_cg_upd1<T, UP_ROWS_SMALL>;
+  launch_pdl(fn, dim3(cg_blocks2(m, sizeof(T))), dim3(UP_THREADS), 0, st, j, dpart1, cg_blocks1(m, sizeof(T)), dots1, V, GV,
+             ldv, s, g, m, dpart2, active);
 }
 template <class T>
 void cg_upd2(int j, const double* dots1, const T* dpart2, T* V, T* GV, int ldv, T* r, T* v, T* s, T* Q,
              int m, double bd_tol, double rtol2_r0sq, int use_rtol, int* active, double* eta, double* alpha,
-             int* count, T* Snext, cudaStream_t st) {
-  launch_pdl(k_cg_upd2<T>, dim3(cdiv(m, UP_ROWS)), dim3(UP_THREADS), 0, st, j, dots1, dpart2, (int)cdiv(m, UP_ROWS), V, GV, ldv, r, v,
-                                                        s, Q, m, bd_tol, rtol2_r0sq, use_rtol, active, eta, alpha,
-                                                        count, Snext);
+             int* count, T* Snext, const double* snext_rep, const T* snext_col, cudaStream_t st) {
+  auto fn = k_cg_upd2<T, UP_ROWS>;
+  if constexpr (sizeof(T) == 8)
+    if (cg_small(m, 8)) fn = k_cg_upd2<T, UP_ROWS_SMALL>;
+  launch_pdl(fn, dim3(cg_blocks2(m, sizeof(T))), dim3(UP_THREADS), 0, st, j, dots1, dpart2, cg_blocks2(m, sizeof(T)), V, GV,
+             ldv, r, v, s, Q, m, bd_tol, rtol2_r0sq, use_rtol, active, eta, alpha, count, Snext, snext_rep, snext_col);
 }
 template <class T>
 void cg_reorth(const T* Q, int ldq, int j, T* s, int m, double* qd, T* S, int lds, const int* active, cudaStream_t st) {
@@ -2191,7 +2347,7 @@ void check_finite(const double* x, size_t n, int* err, cudaStream_t st) {
   template void cg_upd1<T>(int, const T*, double*, T*, T*, int, const T*, const T*, int, T*,                    \
                            const int*, cudaStream_t);                                                            \
   template void cg_upd2<T>(int, const double*, const T*, T*, T*, int, T*, T*, T*, T*, int, double, double,       \
-                           int, int*, double*, double*, int*, T*, cudaStream_t);                                 \
+                           int, int*, double*, double*, int*, T*, const double*, const T*, cudaStream_t);                                 \
   template void cg_reorth<T>(const T*, int, int, T*, int, double*, T*, int, const int*, cudaStream_t);          \
   template void cg_select<T>(int, const T*, const double*, int, T*, T*, int, const int*, cudaStream_t);          \
   template void cg_init<T>(const double*, const double*, const int*, int, T*, T*, T*, double*, cudaStream_t);    \
