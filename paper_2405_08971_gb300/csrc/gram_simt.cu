@@ -60,12 +60,12 @@ template <int CPT, int RPT> struct F32Tile {
 
 // One stage's products: acc += (RPT rows at ty RPT) x (CPT columns F32Tile::col(tx, .)), 16 terms each.
 template <int CPT, int RPT>
-__device__ __forceinline__ void stage_fma(const float* Ks, const float* Bs, int tx, int ty,
+__device__ __forceinline__ void stage_fma(const float* Ks, const float* Bs, int buf, int tx, int ty,
                                           uint64_t (&acc)[CPT][RPT / 2]) {
   using F = F32Tile<CPT, RPT>;
 #pragma unroll 4
   for (int kk = 0; kk < GS_KS; ++kk) {
-    const float* kp = Ks + (size_t)kk * F::LDK + ty * RPT;
+    const float* kp = Ks + (size_t)(buf * GS_KS + kk) * F::LDK + ty * RPT;
     uint64_t kr[RPT / 2];
     if constexpr (RPT % 4 == 0) {
 #pragma unroll
@@ -78,7 +78,7 @@ __device__ __forceinline__ void stage_fma(const float* Ks, const float* Bs, int 
 #pragma unroll
       for (int q = 0; q < RPT / 2; ++q) kr[q] = *reinterpret_cast<const uint64_t*>(kp + 2 * q);
     }
-    const float* bp = Bs + kk * F::LDB;
+    const float* bp = Bs + (buf * GS_KS + kk) * F::LDB;
     float b[CPT];
 #pragma unroll
     for (int q = 0; q < F::N4; ++q) {
@@ -211,7 +211,7 @@ k_gram_block_f32(int fn, const C4<float>* __restrict__ Xr, int nr, const C4<floa
     bar();
     int buf = 0;
     for (int st = first; st < nst; st += step, buf ^= 1) {
-      stage_fma<CPT, RPT>(Ks + (size_t)buf * GS_KS * F::LDK, Bs + buf * GS_KS * F::LDB, tx, ty, acc);
+      stage_fma<CPT, RPT>(Ks, Bs, buf, tx, ty, acc);
       if (st + step < nst) {
         eval(buf ^ 1);
         store_b(buf ^ 1);
@@ -295,7 +295,7 @@ k_gemm_nn_f32(int M, int N, int K, float alpha, const float* __restrict__ A, int
     bar();
     int buf = 0;
     for (int st = first; st < nst; st += step, buf ^= 1) {
-      stage_fma<CPT, RPT>(Ks + (size_t)buf * GS_KS * F::LDK, Bs + buf * GS_KS * F::LDB, tx, ty, acc);
+      stage_fma<CPT, RPT>(Ks, Bs, buf, tx, ty, acc);
       if (st + step < nst) {
         store(buf ^ 1);
         if (st + 2 * step < nst) load(st + 2 * step);
