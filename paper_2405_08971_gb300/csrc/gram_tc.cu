@@ -12,16 +12,19 @@
 // accumulate it in FP32 from the same correlation values.
 //
 // Four operand modes (template parameter MD):
-//   BF16      one BF16 MMA per slice and N chunk (kind::f16); 64-column slices, 128-byte swizzle.
+//   BF16      one BF16 MMA per slice and N chunk (kind::f16); 32-column slices.
 //   FP16 x3   every operand is carried as hi = fp16(x) plus lo = fp16(x - hi) (22 significant
 //             bits; B is scaled per column by a power of two into [0.5, 1) first, undone in the
 //             epilogue), and hi*hi + hi*lo + lo*hi accumulate in the same TMEM columns: FP32-class
-//             products at three MMAs per slice; 32-column slices, 64-byte swizzle (the doubled
-//             operands must still fit two pipeline stages in shared memory).
+//             products at three MMAs per slice; 32-column slices.
 //   TF32      one kind::tf32 MMA per slice (operands rounded to TF32: 11 significant bits, FP32
-//             exponent range); 32-column slices of 4-byte elements, 128-byte swizzle.
+//             exponent range); 16-column slices of 4-byte elements.
 //   TF32 x3   hi = tf32(x), lo = tf32(x - hi) and three kind::tf32 MMAs (about 22 significant
-//             bits, no scaling needed); 16-column slices, 64-byte swizzle.
+//             bits, no scaling needed); 16-column slices.
+// Slices are 64 bytes of every operand row (64-byte swizzle) in all modes: with 512 operand columns that leaves
+// room for 4 stages, where 128-byte rows left 2 (32,768 x 16,384 x 513 in BF16: 485 us with them, 364 us so).  A
+// BF16 or TF32 value costs little more than its evaluation, so there half of the producer warps fill a slice
+// (16 bytes per row and store) and two slices are filled at a time.
 // In every mode one MMA instruction consumes 32 bytes of K per operand row (16 16-bit or 8 32-bit
 // elements), so the descriptors advance by 32 bytes per K step whatever the element type.
 // Every mbarrier wait is bounded; on timeout the CTA raises the error flag and stops.
@@ -54,14 +57,15 @@ template <int MD> struct Mode {
   static constexpr bool TF32 = (MD == MD_TF32 || MD == MD_TF32X3);     // kind::tf32, 4-byte elements
   static constexpr bool SCALED = (MD == MD_F16X3);                     // per-column power-of-two scale of B
   static constexpr int ES = TF32 ? 4 : 2;             // operand element bytes
-  static constexpr int ROWB = SPLIT ? 64 : 128;       // bytes per tile row = swizzle span
+  static constexpr int ROWB = 64;                     // bytes per tile row = swizzle span
   static constexpr int BK = ROWB / ES;                // kernel columns per pipeline stage
   static constexpr int NPART = SPLIT ? 2 : 1;         // operand parts (hi, lo)
   static constexpr int A_TILE = BM * ROWB;            // bytes per A part
   static constexpr int C_STAGE = BK * 16;             // column coordinates and mean column, pair layout
-  static constexpr int CPT = BK / 8;                  // columns per producer thread and slice
+  static constexpr int GROUPS = SPLIT ? 1 : 2;        // producer groups, each filling every GROUPS-th slice
+  static constexpr int CPT = BK * GROUPS / 8;         // columns per producer thread and slice
   static constexpr uint32_t SBO = 8 * ROWB;           // 8-row group stride
-  static constexpr uint64_t LAYOUT = SPLIT ? 4 : 2;   // descriptor swizzle: 64-byte / 128-byte
+  static constexpr uint64_t LAYOUT = 4;               // descriptor swizzle: 64-byte
   // instruction descriptor format fields: FP32 accumulator (bit 4); A and B types in bits 7..9 and
   // 10..12: FP16 = 0, BF16 = 1 (kind::f16), TF32 = 2 (kind::tf32)
   static constexpr uint32_t FMT = (1u << 4) | (MD == MD_BF16 ? ((1u << 7) | (1u << 10)) : 0u) |
@@ -131,6 +135,28 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
   return false;
 }
 
+// The same by a whole warp, each lane for its own barrier; the result is uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag, long long limit) {
+  for (long long it = 0; it < limit; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (__all_sync(0xffffffffu, ok)) return true;
+    if (__any_sync(0xffffffffu, lds32(abort_flag))) return false;
+  }
+  sts32(abort_flag, 1);
+  return false;
+}
+// One lane of a converged warp, the same at every call
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 // Position in a ring of S stages: the stage and the parity of its current use.  (Counted up: a modulo of the
 // slice number by the runtime stage count costs about as many instructions as a slice's own work.)
 struct Ring {
@@ -157,18 +183,13 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
-// Shared-memory matrix descriptor: K-major, swizzled rows of ROWB bytes, 8-row groups SBO apart.
-// The K step of an MMA (16 elements = 32 bytes) is taken by advancing the start address.
-template <int MD>
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;                           // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(Mode<MD>::SBO >> 4) << 32;        // stride byte offset
-  d |= (uint64_t)1 << 46;                           // descriptor version
-  d |= Mode<MD>::LAYOUT << 61;                      // swizzle mode
-  return d;
-}
+// Shared-memory matrix descriptor: K-major, swizzled rows of ROWB bytes, 8-row groups SBO apart.  Low word:
+// start address / 16 (bits 0..13) and leading byte offset (1, unused for swizzled K-major); high word: stride
+// byte offset / 16, descriptor version (bit 46) and swizzle mode (bits 61..63).
+// The K step of an MMA (32 bytes of every row) is taken by advancing the start address.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+template <int MD> constexpr uint32_t SDESC_HI =
+    (Mode<MD>::SBO >> 4) | (1u << 14) | ((uint32_t)Mode<MD>::LAYOUT << 29);
 
 // Byte offset of byte `b` of row `row` in a swizzled tile: the 16-byte chunk index is XORed with
 // the row's phase (row & 7 for 128-byte rows, (row >> 1) & 3 for 64-byte rows).
@@ -186,19 +207,40 @@ __host__ __device__ constexpr uint32_t idesc(int n) {
   return Mode<MD>::FMT | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-// D (TMEM) += A * B, or D = A * B when acc == 0; kind::tf32 for the TF32 modes, kind::f16 otherwise.
+// D (TMEM) += A * B, or D = A * B when acc == 0; kind::tf32 for the TF32 modes, kind::f16 otherwise.  A and B by
+// the low words of their descriptors.
 template <int MD>
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc) {
   if constexpr (Mode<MD>::TF32) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %3, p;\n}\n"
+        ::"r"(d_tmem), "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(SDESC_HI<MD>)
         : "memory");
   } else {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n"
+        ::"r"(d_tmem), "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(SDESC_HI<MD>)
         : "memory");
+  }
+}
+// All MMAs of one slice: a, b = low descriptor words of the stage's hi parts, npad operand columns (at most 256
+// per instruction); with acc0 == 0 the first of each accumulator column overwrites.
+template <int MD>
+__device__ __forceinline__ void mma_slice(uint32_t tmem, uint32_t a, uint32_t b, int npad, uint32_t acc0) {
+  using M = Mode<MD>;
+  const uint32_t lo = (uint32_t)npad * (M::ROWB / 16);   // from the hi to the lo part of B
+  for (int c0 = 0; c0 < npad; c0 += 256, b += 256 * (M::ROWB / 16), tmem += 256) {
+    const uint32_t id = idesc<MD>(min(256, npad - c0));
+#pragma unroll
+    for (int kk = 0; kk < M::ROWB / 32; ++kk) {
+      mma<MD>(tmem, a + 2 * kk, b + 2 * kk, id, kk == 0 ? acc0 : 1u);
+      if constexpr (M::SPLIT) {
+        mma<MD>(tmem, a + 2 * kk, b + lo + 2 * kk, id, 1u);
+        mma<MD>(tmem, a + M::A_TILE / 16 + 2 * kk, b + 2 * kk, id, 1u);
+      }
+    }
   }
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -310,14 +352,14 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
   uint32_t abort_flag = smem_u32(tmem_holder + 1);
   float* mean_part = reinterpret_cast<float*>(tmem_holder + 4);     // [2][8][BM]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const long long total = (long long)P.ntiles * P.nk;
   const long long u0 = total * blockIdx.x / gridDim.x;
   const long long u1 = total * (blockIdx.x + 1) / gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(smem_u32(&fullA[s]), NPROD_WARPS);
+      mbar_init(smem_u32(&fullA[s]), NPROD_WARPS / M::GROUPS);
       mbar_init(smem_u32(&fullB[s]), 1);
       mbar_init(smem_u32(&fullC[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
@@ -340,11 +382,14 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
 
   if (warp < NPROD_WARPS) {
     // ------------------------------------------------------------ kernel-tile producers + epilogue
-    // Producer role: warp w computes rows {rh*32 + lane, rh*32 + lane + 64} (rh = w & 1) for the
-    // CPT-column group cg = w >> 1 of every slice, two columns at a time in packed f32x2
-    // arithmetic.  Epilogue role: warp w reads TMEM lanes 32*(w & 3).. (the lane group it may
+    // Producer role: the 16 / GROUPS warps of group g fill the slices g, g + GROUPS, ... of the CTA's
+    // range; in one, warp w computes rows {rh*32 + lane, rh*32 + lane + 64} (rh = w & 1) for the
+    // CPT-column group cg, two columns at a time in packed f32x2 arithmetic.  The number of stages is a
+    // multiple of GROUPS, so a stage always belongs to the same group, whose warps see every phase of its
+    // barriers.  Epilogue role: warp w reads TMEM lanes 32*(w & 3).. (the lane group it may
     // access) for the column chunks qt, qt + NQ, ... (qt = w >> 2).
-    const int rh = warp & 1, cg = warp >> 1;
+    constexpr int G = M::GROUPS;
+    const int rh = warp & 1, cg = (warp >> 1) % (8 / G), grp = (warp >> 1) / (8 / G);
     const int lg = warp & 3;                        // TMEM lane group of this warp
     const int qt = warp >> 2;                       // which NQ-th of the 32-column epilogue chunks
     const int rl = lg * 32 + lane;                  // epilogue row within the tile (= TMEM lane)
@@ -352,7 +397,8 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     long long u = u0;
     int tcount = 0;
     bool ok = true;
-    Ring ring;
+    int s = grp, next = grp;                        // this group's next stage and slice of the CTA's range
+    uint32_t ph = 0;
     const uint32_t fullC0 = smem_u32(fullC), fullA0 = smem_u32(fullA);
     // this thread's parts of a stage: coordinates and mean column of its column group, its two operand rows
     constexpr int NPAIR = M::CPT / 2;
@@ -374,11 +420,11 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
         rx1 = f2_make(x1.x, x1.x); ry1 = f2_make(x1.y, x1.y); rz1 = f2_make(x1.z, x1.z);
       }
       uint64_t macc0 = 0ull, macc1 = 0ull;          // (even, odd column) partial means, FP32 pairs
-      for (int left = (int)(uend - u); left > 0; --left, ++u, ring.next(S)) {
-        const int s = ring.s;
+      ok = true;
+      for (const int seg = (int)(uend - u0); next < seg; next += G) {
         // fullC completes only after the TMA warp saw empty[s] (the MMAs of this stage's previous
         // use are done) and its copies landed, so it also releases the A stage to the producers.
-        ok = mbar_wait(fullC0 + 8 * s, ring.ph, abort_flag, P.wait_limit);
+        ok = mbar_wait(fullC0 + 8 * s, ph, abort_flag, P.wait_limit);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         const uint32_t cp = cp0 + s * M::C_STAGE;
@@ -427,11 +473,13 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(fullA0 + 8 * s);
+        if ((s += G) >= S) { s -= S; ph ^= 1; }
       }
+      u = uend;
       // ---- end of this CTA's part of the tile: every producer warp arrives here, also on abort
       const uint32_t mp = mp0 + (tcount & 1) * (8 * BM * 4);
-      sts32f(mp + (cg * BM + pr0) * 4, f2_sum(macc0));
-      sts32f(mp + (cg * BM + pr1) * 4, f2_sum(macc1));
+      sts32f(mp + ((warp >> 1) * BM + pr0) * 4, f2_sum(macc0));
+      sts32f(mp + ((warp >> 1) * BM + pr1) * 4, f2_sum(macc1));
       ok = producers_all(ok && !lds32(abort_flag));
       if (!ok) break;
       if (qt == 0 && row < P.nr) {
@@ -489,20 +537,18 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
       long long issued = 0;
       Ring ring;
       int kt = (int)(u0 % P.nk);
-      for (long long u = u0; u < u1; ++u, ring.next(S)) {
+      const uint32_t empty0 = smem_u32(empty), fullB0 = smem_u32(fullB), fullC0 = smem_u32(fullC);
+      const uint32_t b0 = smem_u32(B_base), c0 = smem_u32(C_base), box_bytes = (uint32_t)P.boxh * M::ROWB;
+      for (long long left = u1 - u0; left > 0; --left, ring.next(S)) {
         const int s = ring.s;
-        if (!mbar_wait(smem_u32(&empty[s]), ring.ph ^ 1, abort_flag, P.wait_limit)) break;
-        const uint32_t cb = smem_u32(&fullC[s]);
+        if (!mbar_wait(empty0 + 8 * s, ring.ph ^ 1, abort_flag, P.wait_limit)) break;
+        const uint32_t cb = fullC0 + 8 * s, bb = fullB0 + 8 * s;
         mbar_expect_tx(cb, M::C_STAGE);
-        bulk_load(smem_u32(C_base + (size_t)s * M::C_STAGE), P.Xc + (size_t)kt * M::BK, M::C_STAGE, cb);
-        const uint32_t bb = smem_u32(&fullB[s]);
+        bulk_load(c0 + s * M::C_STAGE, P.Xc + (size_t)kt * M::BK, M::C_STAGE, cb);
         mbar_expect_tx(bb, P.b_stage_bytes);
-        // B rows (operand columns) 0..npad-1 hold the hi part, npad..2 npad-1 the lo part
-        for (int part = 0; part < M::NPART; ++part)
-          for (int b = 0; b < P.nbox; ++b)
-            tma_load_2d(smem_u32(B_base + (size_t)s * P.b_stage_bytes +
-                                 ((size_t)part * P.npad + (size_t)b * P.boxh) * M::ROWB),
-                        &tmapB, kt * M::BK, part * P.npad + b * P.boxh, bb);
+        // B rows (operand columns) 0..npad-1 hold the hi part, npad..2 npad-1 the lo part; boxes of boxh rows
+        uint32_t dst = b0 + s * P.b_stage_bytes;
+        for (int b = 0, y = 0; b < P.nbox; ++b, y += P.boxh, dst += box_bytes) tma_load_2d(dst, &tmapB, kt * M::BK, y, bb);
         ++issued;
         if (++kt == P.nk) kt = 0;
       }
@@ -518,55 +564,50 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     }
   } else if (warp == MMA_WARP) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      long long u = u0;
-      int tcount = 0;
-      Ring ring;
-      while (u < u1 && ok) {
-        const long long tend = (u / P.nk + 1) * P.nk;
-        const long long uend = u1 < tend ? u1 : tend;
-        if (tcount > 0) {   // the epilogue of the previous tile must have read the accumulator out
-          ok = mbar_wait(smem_u32(tfree), (tcount - 1) & 1, abort_flag, P.wait_limit);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-        bool first = true;
-        for (int left = (int)(uend - u); left > 0; --left, ++u, ring.next(S)) {
-          const int s = ring.s;
-          ok = mbar_wait(smem_u32(&fullA[s]), ring.ph, abort_flag, P.wait_limit) &&
-               mbar_wait(smem_u32(&fullB[s]), ring.ph, abort_flag, P.wait_limit);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_u32(A_base + (size_t)s * M::NPART * M::A_TILE);
-          const uint32_t b0 = smem_u32(B_base + (size_t)s * P.b_stage_bytes);
-          const uint32_t blo = (uint32_t)P.npad * M::ROWB;   // offset of the lo part of B
-          for (int c0 = 0; c0 < P.npad; c0 += 256) {
-            const int nn = min(256, P.npad - c0);
-            const uint32_t id = idesc<MD>(nn);
-            const uint32_t d = tmem + (uint32_t)c0;
-#pragma unroll
-            for (int kk = 0; kk < M::ROWB / 32; ++kk) {
-              const uint64_t ah = sdesc<MD>(a0 + kk * 32);
-              const uint64_t bh = sdesc<MD>(b0 + (uint32_t)c0 * M::ROWB + kk * 32);
-              mma<MD>(d, ah, bh, id, (first && kk == 0) ? 0u : 1u);
-              if constexpr (M::SPLIT) {
-                mma<MD>(d, ah, sdesc<MD>(b0 + blo + (uint32_t)c0 * M::ROWB + kk * 32), id, 1u);
-                mma<MD>(d, sdesc<MD>(a0 + M::A_TILE + kk * 32), bh, id, 1u);
-              }
-            }
-          }
-          first = false;
-          mma_commit(smem_u32(&empty[s]));
-        }
+    // The whole warp runs the loop and one lane issues: its control flow and operands are uniform, so the
+    // descriptors stay in uniform registers, which is where tcgen05.mma reads them, and one wait looks at
+    // both barriers of a stage (lane 1: B).  This warp paces the pipeline: as a single-lane loop with a wait
+    // per barrier it took 1,220 cycles per slice (706 of them to issue 6 MMAs), and every other role waited
+    // for it (65,536 x 8,192 x 65, FP16 x3: 555 us, 407 us this way; factor products 65,536 x 512 x 576: 187, 163;
+    // 512 x 577 x 65,536: 255, 236).
+    const bool leader = elect_one();
+    bool ok = true;
+    long long u = u0;
+    int tcount = 0;
+    Ring ring;
+    const uint32_t full0 = smem_u32(lane == 1 ? fullB : fullA), empty0 = smem_u32(empty);
+    const uint32_t a0 = sdesc_lo(smem_u32(A_base)), b0 = sdesc_lo(smem_u32(B_base));
+    const uint32_t d = __shfl_sync(0xffffffffu, tmem, 0);
+    while (u < u1) {
+      const long long tend = (u / P.nk + 1) * P.nk;
+      const long long uend = u1 < tend ? u1 : tend;
+      if (tcount > 0) {   // the epilogue of the previous tile must have read the accumulator out
+        ok = mbar_wait_warp(smem_u32(tfree), (tcount - 1) & 1, abort_flag, P.wait_limit);
         if (!ok) break;
-        mma_commit(smem_u32(done));
-        ++tcount;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      // every MMA issued above has completed before TMEM is released (also after an abort)
-      mma_commit(smem_u32(fin));
-      mbar_drain(smem_u32(fin), 0);
+      uint32_t acc = 0;
+      for (int left = (int)(uend - u); left > 0; --left, ring.next(S)) {
+        const int s = ring.s;
+        ok = mbar_wait_warp(full0 + 8 * s, ring.ph, abort_flag, P.wait_limit);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t as = a0 + s * (M::NPART * M::A_TILE / 16), bs = b0 + s * (P.b_stage_bytes >> 4);
+        if (leader) {
+          mma_slice<MD>(d, as, bs, P.npad, acc);
+          mma_commit(empty0 + 8 * s);
+        }
+        acc = 1;
+      }
+      if (!ok) break;
+      u = uend;
+      if (leader) mma_commit(smem_u32(done));
+      ++tcount;
     }
+    // every MMA issued above has completed before TMEM is released (also after an abort)
+    if (leader) mma_commit(smem_u32(fin));
+    __syncwarp();
+    mbar_drain(smem_u32(fin), 0);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -664,7 +705,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 3 * S + 3);
   uint32_t abort_flag = smem_u32(tmem_holder + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const int units = P.ntiles * P.nchunks * P.kchunks;
   constexpr bool preB = PREB;
   if (threadIdx.x == 0) {
@@ -715,7 +756,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
       // loaded PF slices ahead (a ring of registers indexed statically: the loop over the slices is unrolled
       // PF times), so that the loads' latency overlaps the conversion, the stores and the waits for free
       // stages.  One slice per turn and PF = 3: 512 x 577 x 65,536 306 us, 65,536 x 512 x 576 200 us; this way
-      // 255 and 187 us.
+      // 255 and 187 us (then still paced by the MMA warp; now 236 and 163).
       constexpr int PF = PREB ? 4 : 2;
       int ak = ks0 * 16 + ar_kq * 4, bk = ks0 * 16 + (tid & 3) * 4;      // K of the next loads
       const size_t arow = min(row0 + ar_row, P.M - 1);
@@ -866,52 +907,44 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm_tc(const GemmParams P) {
         mbar_drain(smem_u32(&fullB[(int)(q % S)]), (uint32_t)((q / S) & 1));
     }
   } else if (warp == MMA_WARP) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      Ring ring;
-      int tcount = 0;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int kc = u / (P.ntiles * P.nchunks);
-        int ks0, ks1;
-        chunk_range(P, kc, ks0, ks1);
-        if (tcount > 0) {
-          ok = mbar_wait(smem_u32(tfree), (tcount - 1) & 1, abort_flag, P.wait_limit);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-        for (int ks = ks0; ks < ks1; ++ks, ring.next(S)) {
-          const int s = ring.s;
-          ok = mbar_wait(smem_u32(&fullA[s]), ring.ph, abort_flag, P.wait_limit);
-          if (ok && preB) ok = mbar_wait(smem_u32(&fullB[s]), ring.ph, abort_flag, P.wait_limit);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_u32(A_base + (size_t)s * M::NPART * M::A_TILE);
-          const uint32_t b0 = smem_u32(B_base + (size_t)s * P.b_stage_bytes);
-          const uint32_t blo = (uint32_t)P.npad * M::ROWB;
-          for (int c0 = 0; c0 < P.npad; c0 += 256) {
-            const int nn = min(256, P.npad - c0);
-            const uint32_t id = idesc<MD>(nn);
-            const uint32_t d = tmem + (uint32_t)c0;
-#pragma unroll
-            for (int kk = 0; kk < M::ROWB / 32; ++kk) {
-              const uint64_t ah = sdesc<MD>(a0 + kk * 32);
-              const uint64_t bh = sdesc<MD>(b0 + (uint32_t)c0 * M::ROWB + kk * 32);
-              mma<MD>(d, ah, bh, id, (ks == ks0 && kk == 0) ? 0u : 1u);
-              mma<MD>(d, ah, sdesc<MD>(b0 + blo + (uint32_t)c0 * M::ROWB + kk * 32), id, 1u);
-              mma<MD>(d, sdesc<MD>(a0 + M::A_TILE + kk * 32), bh, id, 1u);
-            }
-          }
-          mma_commit(smem_u32(&empty[s]));
-        }
+    // the MMA issuer: see k_gram_tc
+    const bool leader = elect_one();
+    bool ok = true;
+    Ring ring;
+    const uint32_t full0 = smem_u32(preB && lane == 1 ? fullB : fullA), empty0 = smem_u32(empty);
+    const uint32_t a0 = sdesc_lo(smem_u32(A_base)), b0 = sdesc_lo(smem_u32(B_base));
+    const uint32_t d = __shfl_sync(0xffffffffu, tmem, 0);
+    int tcount = 0;
+    for (int u = blockIdx.x; u < units; u += gridDim.x) {
+      const int kc = u / (P.ntiles * P.nchunks);
+      int ks0, ks1;
+      chunk_range(P, kc, ks0, ks1);
+      if (tcount > 0) {
+        ok = mbar_wait_warp(smem_u32(tfree), (tcount - 1) & 1, abort_flag, P.wait_limit);
         if (!ok) break;
-        mma_commit(smem_u32(done));
-        ++tcount;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      // every MMA issued above has completed before TMEM is released
-      mma_commit(smem_u32(fin));
-      mbar_drain(smem_u32(fin), 0);
+      uint32_t acc = 0;
+      for (int left = ks1 - ks0; left > 0; --left, ring.next(S)) {
+        const int s = ring.s;
+        ok = mbar_wait_warp(full0 + 8 * s, ring.ph, abort_flag, P.wait_limit);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t as = a0 + s * (M::NPART * M::A_TILE / 16), bs = b0 + s * (P.b_stage_bytes >> 4);
+        if (leader) {
+          mma_slice<MD>(d, as, bs, P.npad, acc);
+          mma_commit(empty0 + 8 * s);
+        }
+        acc = 1;
+      }
+      if (!ok) break;
+      if (leader) mma_commit(smem_u32(done));
+      ++tcount;
     }
+    // every MMA issued above has completed before TMEM is released
+    if (leader) mma_commit(smem_u32(fin));
+    __syncwarp();
+    mbar_drain(smem_u32(fin), 0);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1096,13 +1129,16 @@ Layout plan_layout(int wtc) {
   using M = Mode<MD>;
   Layout L;
   L.npad = std::max(16, round_up(wtc, 16));
-  L.nbox = (L.npad + 255) / 256;           // npad <= 512: one or two boxes per part
-  L.boxh = L.npad / L.nbox;                // a multiple of 8: boxes start on swizzle-atom boundaries
+  // as few boxes of at most 256 rows over the parts' NPART * npad rows as leave whole groups of 8 (boxes start on
+  // swizzle-atom boundaries)
+  const int brows = M::NPART * L.npad;
+  for (L.nbox = (brows + 255) / 256; brows % (8 * L.nbox); ++L.nbox) {}
+  L.boxh = brows / L.nbox;
   L.b_stage_bytes = (uint32_t)(M::NPART * L.npad * M::ROWB);
   const size_t per_stage = (size_t)M::NPART * M::A_TILE + L.b_stage_bytes + M::C_STAGE;
   const size_t fixed = 1024 /*alignment slack*/ + 64 * 8 + 64 + 2 * 8 * BM * 4;
   const size_t budget = 220 * 1024;
-  L.stages = (int)std::min<size_t>(8, (budget - fixed) / per_stage);
+  L.stages = (int)std::min<size_t>(8, (budget - fixed) / per_stage) / M::GROUPS * M::GROUPS;
   L.tmem_cols = 32;
   while (L.tmem_cols < L.npad) L.tmem_cols *= 2;
   L.smem = fixed + (size_t)L.stages * per_stage;
@@ -1162,7 +1198,7 @@ int launch(int ker, const C4<float>* Xr, int nr, int nc, const void* Bp, int ldp
                                                            : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
   CUresult cr = encode(&map, dt, 2,
                        const_cast<void*>(Bp), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       M::SPLIT ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                       CU_TENSOR_MAP_SWIZZLE_64B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return 6;
 
