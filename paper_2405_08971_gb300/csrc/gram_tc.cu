@@ -18,13 +18,15 @@
 //             epilogue), and hi*hi + hi*lo + lo*hi accumulate in the same TMEM columns: FP32-class
 //             products at three MMAs per slice; 32-column slices.
 //   TF32      one kind::tf32 MMA per slice (operands rounded to TF32: 11 significant bits, FP32
-//             exponent range); 16-column slices of 4-byte elements.
+//             exponent range); 32-column slices of 4-byte elements (128 bytes of a row: with 16
+//             columns the waits of a slice weigh twice as much, and all 16 producer warps fill one).
 //   TF32 x3   hi = tf32(x), lo = tf32(x - hi) and three kind::tf32 MMAs (about 22 significant
 //             bits, no scaling needed); 16-column slices.
-// Slices are 64 bytes of every operand row (64-byte swizzle) in all modes: with 512 operand columns that leaves
-// room for 4 stages, where 128-byte rows left 2 (32,768 x 16,384 x 513 in BF16: 485 us with them, 364 us so).  A
-// BF16 or TF32 value costs little more than its evaluation, so there half of the producer warps fill a slice
-// (16 bytes per row and store) and two slices are filled at a time.
+// Slices are 64 bytes of every operand row (64-byte swizzle) in the other modes: with 512 operand columns that leaves
+// room for 4 stages, where 128-byte rows left 2 (32,768 x 16,384 x 513 in BF16: 485 us with them, 364 us so).  Half
+// of the producer warps fill a slice, with 16-byte stores, and two slices are filled at a time: a warp pays the
+// wait, the vote and the proxy fence of a slice for 16 values per lane instead of 8, and the stores meet no bank
+// conflicts (65,536 x 8,192 x 65 in FP16 x3: 465 us for the whole call with all warps on one slice, 394 us so).
 // In every mode one MMA instruction consumes 32 bytes of K per operand row (16 16-bit or 8 32-bit
 // elements), so the descriptors advance by 32 bytes per K step whatever the element type.
 // Every mbarrier wait is bounded; on timeout the CTA raises the error flag and stops.
@@ -57,15 +59,16 @@ template <int MD> struct Mode {
   static constexpr bool TF32 = (MD == MD_TF32 || MD == MD_TF32X3);     // kind::tf32, 4-byte elements
   static constexpr bool SCALED = (MD == MD_F16X3);                     // per-column power-of-two scale of B
   static constexpr int ES = TF32 ? 4 : 2;             // operand element bytes
-  static constexpr int ROWB = 64;                     // bytes per tile row = swizzle span
+  static constexpr int ROWB = TF32 && !SPLIT ? 128 : 64;   // bytes per tile row = swizzle span
   static constexpr int BK = ROWB / ES;                // kernel columns per pipeline stage
   static constexpr int NPART = SPLIT ? 2 : 1;         // operand parts (hi, lo)
   static constexpr int A_TILE = BM * ROWB;            // bytes per A part
   static constexpr int C_STAGE = BK * 16;             // column coordinates and mean column, pair layout
-  static constexpr int GROUPS = SPLIT ? 1 : 2;        // producer groups, each filling every GROUPS-th slice
-  static constexpr int CPT = BK * GROUPS / 8;         // columns per producer thread and slice
+  static constexpr int CPT = 16 / ES;                 // columns per producer thread and slice: 16 bytes of a row
+  static constexpr int GROUPS = ROWB == 64 ? 2 : 1;   // producer groups, each filling every GROUPS-th slice
+  static constexpr int MEAN_RUN = SPLIT ? 16 : 1 << 20;   // slices between flushes of the mean's running sums
   static constexpr uint32_t SBO = 8 * ROWB;           // 8-row group stride
-  static constexpr uint64_t LAYOUT = 4;               // descriptor swizzle: 64-byte
+  static constexpr uint64_t LAYOUT = ROWB == 64 ? 4 : 2;   // descriptor swizzle: 64-byte / 128-byte
   // instruction descriptor format fields: FP32 accumulator (bit 4); A and B types in bits 7..9 and
   // 10..12: FP16 = 0, BF16 = 1 (kind::f16), TF32 = 2 (kind::tf32)
   static constexpr uint32_t FMT = (1u << 4) | (MD == MD_BF16 ? ((1u << 7) | (1u << 10)) : 0u) |
@@ -101,9 +104,6 @@ __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
 }
 __device__ __forceinline__ void sts32f(uint32_t a, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
@@ -324,6 +324,25 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
   }
 }
 
+// The running sum r into the sum h and the rounding errors l (two_sum, in FP32 pairs); r starts again at 0.
+// The filter and smoother carry the mean column through hundreds of steps, so it is summed to about FP32 rounding
+// whatever the order of its terms: runs of 16 slices, then error-free (in the split modes; the rounded operands of
+// the others leave nothing to gain).
+__device__ __forceinline__ void mean_flush(uint64_t& r, uint64_t& h, uint64_t& l) {
+  const uint64_t t = f2_add(h, r), b = f2_sub(t, h);
+  l = f2_add(l, f2_add(f2_sub(h, f2_sub(t, b)), f2_sub(r, b)));
+  h = t;
+  r = 0ull;
+}
+
+// Both halves' sum; an infinite or NaN sum has no rounding errors to add.
+__device__ __forceinline__ float mean_total(uint64_t h, uint64_t l) {
+  float h0, h1, l0, l1;
+  f2_split(h, h0, h1);
+  f2_split(l, l0, l1);
+  return (fabsf(h0) <= FLT_MAX ? h0 + l0 : h0) + (fabsf(h1) <= FLT_MAX ? h1 + l1 : h1);
+}
+
 // Persistent schedule (stream-K): the work is the sequence of (row tile, K slice) units, tile-major;
 // CTA b takes units [total*b/G, total*(b+1)/G).  With G <= ntiles every CTA covers at least one full
 // tile's worth of slices, so a tile is shared by at most two CTAs; those add their partial sums
@@ -419,74 +438,79 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
         rx0 = f2_make(x0.x, x0.x); ry0 = f2_make(x0.y, x0.y); rz0 = f2_make(x0.z, x0.z);
         rx1 = f2_make(x1.x, x1.x); ry1 = f2_make(x1.y, x1.y); rz1 = f2_make(x1.z, x1.z);
       }
-      uint64_t macc0 = 0ull, macc1 = 0ull;          // (even, odd column) partial means, FP32 pairs
+      // (even, odd column) partial means, FP32 pairs: a running sum of up to MEAN_RUN slices on top of the sum
+      // so far and its rounding errors
+      uint64_t macc0 = 0ull, macc1 = 0ull, mh0 = 0ull, mh1 = 0ull, ml0 = 0ull, ml1 = 0ull;
       ok = true;
-      for (const int seg = (int)(uend - u0); next < seg; next += G) {
-        // fullC completes only after the TMA warp saw empty[s] (the MMAs of this stage's previous
-        // use are done) and its copies landed, so it also releases the A stage to the producers.
-        ok = mbar_wait(fullC0 + 8 * s, ph, abort_flag, P.wait_limit);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        const uint32_t cp = cp0 + s * M::C_STAGE;
-        // 16-bit modes: one packed word per column pair and part; TF32 modes: one word per column
-        uint32_t pk0[2 * NPAIR], pk1[2 * NPAIR], pl0[2 * NPAIR], pl1[2 * NPAIR];
+      const int seg = (int)(uend - u0);
+      while (next < seg && ok) {
+        for (const int lim = min(seg, next + M::MEAN_RUN * G); next < lim; next += G) {
+          // fullC completes only after the TMA warp saw empty[s] (the MMAs of this stage's previous
+          // use are done) and its copies landed, so it also releases the A stage to the producers.
+          ok = mbar_wait(fullC0 + 8 * s, ph, abort_flag, P.wait_limit);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const uint32_t cp = cp0 + s * M::C_STAGE;
+          // 16-bit modes: one packed word per column pair and part; TF32 modes: one word per column
+          uint32_t pk0[4], pk1[4];
+          [[maybe_unused]] uint32_t pl0[4], pl1[4];
 #pragma unroll
-        for (int q = 0; q < NPAIR; ++q) {
-          const ulonglong2 xy = lds128(cp + q * 32), zw = lds128(cp + q * 32 + 16);
-          const uint64_t cz = zw.x, w2 = zw.y;
-          const uint64_t k0 = kpair<KER>(rx0, ry0, rz0, xy.x, xy.y, cz);
-          const uint64_t k1 = kpair<KER>(rx1, ry1, rz1, xy.x, xy.y, cz);
-          macc0 = f2_fma(k0, w2, macc0);
-          macc1 = f2_fma(k1, w2, macc1);
-          if constexpr (M::TF32) {
-            float a0, b0v, a1, b1v;
-            f2_split(k0, a0, b0v);
-            f2_split(k1, a1, b1v);
-            pk0[2 * q] = tf32_rna(a0); pk0[2 * q + 1] = tf32_rna(b0v);
-            pk1[2 * q] = tf32_rna(a1); pk1[2 * q + 1] = tf32_rna(b1v);
-            if constexpr (M::SPLIT) {   // x - hi is exact in FP32; lo keeps its leading 11 bits
-              pl0[2 * q] = tf32_rna(a0 - __uint_as_float(pk0[2 * q]));
-              pl0[2 * q + 1] = tf32_rna(b0v - __uint_as_float(pk0[2 * q + 1]));
-              pl1[2 * q] = tf32_rna(a1 - __uint_as_float(pk1[2 * q]));
-              pl1[2 * q + 1] = tf32_rna(b1v - __uint_as_float(pk1[2 * q + 1]));
+          for (int q = 0; q < NPAIR; ++q) {
+            const ulonglong2 xy = lds128(cp + q * 32), zw = lds128(cp + q * 32 + 16);
+            const uint64_t cz = zw.x, w2 = zw.y;
+            const uint64_t k0 = kpair<KER>(rx0, ry0, rz0, xy.x, xy.y, cz);
+            const uint64_t k1 = kpair<KER>(rx1, ry1, rz1, xy.x, xy.y, cz);
+            macc0 = f2_fma(k0, w2, macc0);
+            macc1 = f2_fma(k1, w2, macc1);
+            if constexpr (M::TF32) {
+              float a0, b0v, a1, b1v;
+              f2_split(k0, a0, b0v);
+              f2_split(k1, a1, b1v);
+              pk0[2 * q] = tf32_rna(a0); pk0[2 * q + 1] = tf32_rna(b0v);
+              pk1[2 * q] = tf32_rna(a1); pk1[2 * q + 1] = tf32_rna(b1v);
+              if constexpr (M::SPLIT) {   // x - hi is exact in FP32; lo keeps its leading 11 bits
+                pl0[2 * q] = tf32_rna(a0 - __uint_as_float(pk0[2 * q]));
+                pl0[2 * q + 1] = tf32_rna(b0v - __uint_as_float(pk0[2 * q + 1]));
+                pl1[2 * q] = tf32_rna(a1 - __uint_as_float(pk1[2 * q]));
+                pl1[2 * q + 1] = tf32_rna(b1v - __uint_as_float(pk1[2 * q + 1]));
+              }
+            } else if constexpr (M::SPLIT) {
+              pk0[q] = f2_f16(k0);
+              pk1[q] = f2_f16(k1);
+              pl0[q] = f2_f16(f2_sub(k0, f16x2_to_f2(pk0[q])));
+              pl1[q] = f2_f16(f2_sub(k1, f16x2_to_f2(pk1[q])));
+            } else {
+              pk0[q] = f2_bf16(k0);
+              pk1[q] = f2_bf16(k1);
             }
-          } else if constexpr (M::SPLIT) {
-            pk0[q] = f2_f16(k0);
-            pk1[q] = f2_f16(k1);
-            pl0[q] = f2_f16(f2_sub(k0, f16x2_to_f2(pk0[q])));
-            pl1[q] = f2_f16(f2_sub(k1, f16x2_to_f2(pk1[q])));
-          } else {
-            pk0[q] = f2_bf16(k0);
-            pk1[q] = f2_bf16(k1);
           }
-        }
-        const uint32_t ast = a0 + s * (M::NPART * M::A_TILE);
-        if constexpr (M::SPLIT) {   // 8 bytes per row and part (4 fp16 or 2 tf32 values)
-          sts64(ast + o0, pk0[0], pk0[1]);
-          sts64(ast + o1, pk1[0], pk1[1]);
-          sts64(ast + M::A_TILE + o0, pl0[0], pl0[1]);
-          sts64(ast + M::A_TILE + o1, pl1[0], pl1[1]);
-        } else {                    // 16 bytes per row (8 bf16 or 4 tf32 values)
+          const uint32_t ast = a0 + s * (M::NPART * M::A_TILE);
           sts128(ast + o0, pk0[0], pk0[1], pk0[2], pk0[3]);
           sts128(ast + o1, pk1[0], pk1[1], pk1[2], pk1[3]);
+          if constexpr (M::SPLIT) {
+            sts128(ast + M::A_TILE + o0, pl0[0], pl0[1], pl0[2], pl0[3]);
+            sts128(ast + M::A_TILE + o1, pl1[0], pl1[1], pl1[2], pl1[3]);
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(fullA0 + 8 * s);
+          if ((s += G) >= S) { s -= S; ph ^= 1; }
         }
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(fullA0 + 8 * s);
-        if ((s += G) >= S) { s -= S; ph ^= 1; }
+        mean_flush(macc0, mh0, ml0);
+        mean_flush(macc1, mh1, ml1);
       }
       u = uend;
       // ---- end of this CTA's part of the tile: every producer warp arrives here, also on abort
       const uint32_t mp = mp0 + (tcount & 1) * (8 * BM * 4);
-      sts32f(mp + ((warp >> 1) * BM + pr0) * 4, f2_sum(macc0));
-      sts32f(mp + ((warp >> 1) * BM + pr1) * 4, f2_sum(macc1));
+      sts32f(mp + ((warp >> 1) * BM + pr0) * 4, mean_total(mh0, ml0));
+      sts32f(mp + ((warp >> 1) * BM + pr1) * 4, mean_total(mh1, ml1));
       ok = producers_all(ok && !lds32(abort_flag));
       if (!ok) break;
       if (qt == 0 && row < P.nr) {
-        float m = lds32f(mp + rl * 4);
+        double md = 0.0;
 #pragma unroll
-        for (int j = 1; j < 8; ++j) m += lds32f(mp + (j * BM + rl) * 4);
-        m *= P.sf2;
+        for (int j = 0; j < 8; ++j) md += (double)lds32f(mp + (j * BM + rl) * 4);
+        const float m = (float)((double)P.sf2 * md);
         float* dst = P.Out + (size_t)P.wtc * P.ldo + row;
         if (split) atomicAdd(dst, m);
         else *dst = m;
@@ -1228,7 +1252,7 @@ int launch(int ker, const C4<float>* Xr, int nr, int nc, const void* Bp, int ldp
                                                            : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
   CUresult cr = encode(&map, dt, 2,
                        const_cast<void*>(Bp), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       CU_TENSOR_MAP_SWIZZLE_64B,
+                       M::ROWB == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return 6;
 
