@@ -507,10 +507,18 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
       ok = producers_all(ok && !lds32(abort_flag));
       if (!ok) break;
       if (qt == 0 && row < P.nr) {
-        double md = 0.0;
+        float m;
+        if constexpr (M::SPLIT) {
+          double md = 0.0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) md += (double)lds32f(mp + (j * BM + rl) * 4);
-        const float m = (float)((double)P.sf2 * md);
+          for (int j = 0; j < 8; ++j) md += (double)lds32f(mp + (j * BM + rl) * 4);
+          m = (float)((double)P.sf2 * md);
+        } else {
+          m = lds32f(mp + rl * 4);
+#pragma unroll
+          for (int j = 1; j < 8; ++j) m += lds32f(mp + (j * BM + rl) * 4);
+          m *= P.sf2;
+        }
         float* dst = P.Out + (size_t)P.wtc * P.ldo + row;
         if (split) atomicAdd(dst, m);
         else *dst = m;
