@@ -600,7 +600,8 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
     // descriptors stay in uniform registers, which is where tcgen05.mma reads them, and one wait looks at
     // both barriers of a stage (lane 1: B).  This warp paces the pipeline: as a single-lane loop with a wait
     // per barrier it took 1,220 cycles per slice (706 of them to issue 6 MMAs), and every other role waited
-    // for it (65,536 x 8,192 x 65, FP16 x3: 555 us, 407 us this way; factor products 65,536 x 512 x 576: 187, 163;
+    // for it (65,536 x 8,192 x 65, FP16 x3: 555 us, 407 us this way, 338 us with
+    // two producer groups besides; factor products 65,536 x 512 x 576: 187, 163;
     // 512 x 577 x 65,536: 255, 236).
     const bool leader = elect_one();
     bool ok = true;
