@@ -63,13 +63,14 @@ __device__ __forceinline__ int ld_relaxed_int(const int* p) {
 }
 constexpr long long kPollLimit = 4000000LL;
 
-// Power of two that brings a matrix of largest magnitude amax (its bit pattern) to about 1, and its inverse;
-// 1 for a zero, denormal or non-finite matrix.
-__device__ __forceinline__ void pow2_scale(unsigned long long amax, double& sc, double& inv) {
-  const long long ex = (long long)(amax >> 52) & 0x7FF;
-  if (ex == 0 || ex > 2045) { sc = inv = 1.0; return; }
-  sc = __longlong_as_double((2046 - ex) << 52);
-  inv = __longlong_as_double(ex << 52);
+// Power of two that brings a largest magnitude amax (its bit pattern; as far as the exponent range goes, a zero or
+// denormal one too) to about 2^target, and its inverse; 1 for a non-finite one.
+__device__ __forceinline__ void pow2_scale(unsigned long long amax, int target, double& sc, double& inv) {
+  const int ex = (int)(amax >> 52) & 0x7FF;
+  if (ex == 2047) { sc = inv = 1.0; return; }
+  const long long E = max(1, min(2045, 2046 + target - ex));
+  sc = __longlong_as_double(E << 52);
+  inv = __longlong_as_double((2046 - E) << 52);
 }
 
 // *amax = largest magnitude of the N x N matrix, as a bit pattern (zero before the launch)
@@ -114,9 +115,12 @@ k_absmax(const double* __restrict__ A, int lda, int N, unsigned long long* __res
 // them): 152 blocks polling the same lines queue at their L2 slices (N = 576: 2.73 ms with one replica, 2.52
 // with 4, 2.66 with 16).  N = 576 takes 2.52 ms, N = 288 0.94 ms; 2.79 and 1.15 ms with scaled reflectors,
 // whose scalars stood between the column pass and the exchange, shuffle sums and pairs of 16 bytes a value.
-// The matrix is scaled by a power of two, which keeps the unscaled reflectors' products in range; a column
-// below 1e-140 of the matrix is left alone (tau = 0).  v and tau are kept for the back-transformation, v
+// The matrix is scaled by a power of two to about 2^TD_SCALE, which keeps the unscaled reflectors' products in
+// range: they go up to N^1.5 c^3 (2^936 at N = 2,048) and, for a decoupled block far below the rest, down to c^3 and
+// its reciprocal.  A column whose square is below TD_TINY (2^-620 of the matrix) is left alone (tau = 0).  v and tau are kept for the back-transformation, v
 // below the subdiagonal of column k.
+constexpr int TD_SCALE = 300;                // exponents: the scaled matrix,
+constexpr double TD_TINY = 0x1p-640;         // and the squared norm of a column that is left alone
 constexpr int TD_VEC = 128;                  // threads of the vector work: 4 warps, the owner warps
 constexpr int TD_THREADS = TD_VEC + 32;      // warp 4: block reductions and scalars
 constexpr int TD_MAX_SLOTS = 64;             // owned columns per block
@@ -200,7 +204,7 @@ __device__ __forceinline__ TdScalars td_scalars(double c1, double sigma) {
   TdScalars r;
   const double x = fma(c1, c1, sigma);
   // (comparisons on the bit patterns: they stay off the FP64 pipe)
-  if (__double_as_longlong(sigma) == 0 || __double_as_longlong(x) < __double_as_longlong(1e-280)) {
+  if (__double_as_longlong(sigma) == 0 || __double_as_longlong(x) < __double_as_longlong(TD_TINY)) {
     r.gamma = 1.0; r.gt = r.tau = 0.0; r.beta = c1;
     return r;
   }
@@ -281,7 +285,7 @@ k_tridiag(double* __restrict__ A, int lda, int N, double* __restrict__ d, double
   const int maxcol = (int)blockIdx.x + G * ((N - 1 - (int)blockIdx.x) / G);
   const size_t rep = (size_t)N * (N + 1);     // words of a replica of the slots
   double msc, minv;
-  pow2_scale(*amax, msc, minv);
+  pow2_scale(*amax, TD_SCALE, msc, minv);
   if (N <= 2) {
     if (blockIdx.x == 0 && tid == 0) {
       d[0] = A[0];
@@ -546,6 +550,10 @@ __host__ __device__ inline size_t prep_smem_bytes(int K) { return (size_t)K * (4
 //      by rank when a rotation moved one.
 //   5. The kept columns are grouped by their row support (child 1 only, both, child 2 only) for the
 //      eigenvector product of phase 5.
+// Poles, rho and with them the distances of phases 2 to 4 are in units of a power of two near the merge's
+// largest magnitude (W.rho[lo + 1] takes them back): the secular function divides by distances of rho z^2, 1e-30
+// of that magnitude, and squares them, which leaves FP64's range for a matrix (or a decoupled block of one) below
+// 2^-430 or above 2^506 in its own units.  Eigenvalues go in and out unscaled.
 // (device function: every thread of the block calls it; psm holds prep_smem_bytes(K))
 __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N, DcWork W, double* psm) {
   const int lo = mg.lo, mid = mg.mid, K = mg.hi - mg.lo, n1 = mg.mid - mg.lo;
@@ -576,7 +584,11 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
   zz = block_sum(zz);
   double zn, rzn;
   fast_sqrt(fmax(zz, 1e-280), zn, rzn);
-  const double rho = fabs(rho0) * zz;
+  // the children's spectra ascend: their ends have the largest magnitudes
+  const double lmax = fmax(fmax(fabs(sLam[0]), fabs(sLam[n1 - 1])), fmax(fabs(sLam[n1]), fabs(sLam[K - 1])));
+  double sc, isc;
+  pow2_scale((unsigned long long)__double_as_longlong(fmax(lmax, fabs(rho0) * zz)), 0, sc, isc);
+  const double rho = fabs(rho0) * sc * zz;
   // 1. merge by rank (ties: child 1 first)
   for (int t = threadIdx.x; t < K; t += blockDim.x) {
     const long long kt = sKey[t];
@@ -591,7 +603,7 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
       pos = (t - n1) + a;
     }
     sPerm[pos] = t;
-    sD[pos] = sLam[t];
+    sD[pos] = sc * sLam[t];
     sZ[pos] = sZr[t] * rzn;
     sType[pos] = (t < n1) ? 1 : 3;
   }
@@ -707,7 +719,7 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
   }
   for (int q = threadIdx.x; q < K - kp; q += blockDim.x) {
     const int j = sDefl[q];
-    W.Dd[lo + q] = sD[j];
+    W.Dd[lo + q] = isc * sD[j];
     W.cold[lo + q] = lo + sPerm[j];
   }
   // 5. kept columns grouped by row support: child 1 only, both children, child 2 only
@@ -726,6 +738,7 @@ __device__ void dc_prep(const MergeDesc mg, const double* __restrict__ e, int N,
       W.gcnt[2 * lo] = tot[0];
       W.gcnt[2 * lo + 1] = tot[1];
       W.rho[lo] = rho;
+      W.rho[lo + 1] = isc;
       W.Kp[lo] = kp;
     }
   }
@@ -947,7 +960,7 @@ __device__ void dc_secular_root(int lo, int i, int N, DcWork W, int* err, int la
     if (it == 199 && !conv && lane == 0) atomicExch(err, kErrSecular);
   }
   for (int j = lane; j < Kp; j += LANES) delta[j] = (Dk[j] - Dorg) - tau;
-  if (lane == 0) W.lamk[lo + i] = Dorg + tau;
+  if (lane == 0) W.lamk[lo + i] = W.rho[lo + 1] * (Dorg + tau);
 }
 template <int LANES>
 __global__ void k_dc_secular(const MergeDesc* __restrict__ merges, const int* __restrict__ mergeof, int N, DcWork W,
