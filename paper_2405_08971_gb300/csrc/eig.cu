@@ -124,8 +124,8 @@ constexpr double TD_TINY = 0x1p-640;         // and the squared norm of a column
 constexpr int TD_VEC = 128;                  // threads of the vector work: 4 warps, the owner warps
 constexpr int TD_THREADS = TD_VEC + 32;      // warp 4: block reductions and scalars
 constexpr int TD_MAX_SLOTS = 64;             // owned columns per block
-// Replicas of the exchange slots (template parameter REP): 4 up to order 1,024, one above, where the slots
-// (8 N^2 bytes a replica) would begin to count among the workspace.
+// Replicas of the exchange slots (template parameter REP; N (N + 1) words each): 4 up to order 1,024, one above,
+// where the fill of 32 N^2 bytes would begin to count.
 inline int td_replicas(int N) { return N <= 1024 ? 4 : 1; }
 constexpr int TD_BATCH = 5;                  // exchange entries a thread polls with their loads in flight together
 
@@ -1652,17 +1652,19 @@ inline size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
+// Workspace of every order up to nmax: each part grows with the order.  (The exchange slots of the
+// tridiagonalisation, whose replicas drop from 4 to 1 above order 1,024, have no part of their own: they lie over
+// Q, Qtmp, Delta and the reflector groups, at least 4 N^2 + 17 N words that are first written after it.)
 size_t eig_workspace_bytes(int nmax) {
   size_t N = std::max(nmax, 1);
   size_t b = 0;
   b += align_up((3 * N + 1) * sizeof(double));    // d, e, tau, largest magnitude
-  b += align_up(td_replicas((int)N) * N * (N + 1) * sizeof(double));    // exchange slots of the tridiagonalisation, (S, C) per entry
   b += 3 * align_up(N * N * sizeof(double));      // Q, Qtmp, Delta
+  b += align_up((N / RB + 2) * RB * N * sizeof(float2));    // reflector groups as double-FP32 pairs
   b += 10 * align_up(N * sizeof(double));         // lam, lamk, lamtmp, Dw, Zw, Dk, Zk, Dd, rho, spare
   b += align_up(4 * N * sizeof(double));          // rot
   b += align_up((N / RB + 2) * RB * RB * sizeof(double));   // back-transform T blocks
   b += align_up((N / RB + 2) * RB * RB * sizeof(float2));   // T blocks as double-FP32 pairs
-  b += align_up((N / RB + 2) * RB * N * sizeof(float2));    // reflector groups as double-FP32 pairs
   b += 7 * align_up(N * sizeof(int));             // colk, cold, perm, Kp, nrot, gperm, spare
   b += align_up(2 * N * sizeof(int));             // gcnt
   return b + 4096;
@@ -1682,12 +1684,13 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   double* e = d + N;
   double* tau = e + N;
   unsigned long long* amax = (unsigned long long*)(tau + N);
-  const size_t slot_bytes = td_replicas(N) * (size_t)N * (N + 1) * sizeof(double);
-  double* slots = (double*)take(slot_bytes);
   DcWork W;
   W.Q = (double*)take((size_t)N * N * sizeof(double));
   W.Qtmp = (double*)take((size_t)N * N * sizeof(double));
   W.Delta = (double*)take((size_t)N * N * sizeof(double));
+  float2* Vff = (float2*)take(((size_t)N / RB + 2) * RB * (size_t)N * sizeof(float2));
+  double* slots = W.Q;
+  const size_t slot_bytes = td_replicas(N) * (size_t)N * (N + 1) * sizeof(double);
   W.lam = (double*)take(N * sizeof(double));
   W.lamk = (double*)take(N * sizeof(double));
   W.Df = (float2*)take(N * sizeof(float2));
@@ -1701,7 +1704,6 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   W.rot = (double*)take(4 * N * sizeof(double));
   W.Tm = (double*)take(((size_t)N / RB + 2) * RB * RB * sizeof(double));
   float2* Tff = (float2*)take(((size_t)N / RB + 2) * RB * RB * sizeof(float2));
-  float2* Vff = (float2*)take(((size_t)N / RB + 2) * RB * (size_t)N * sizeof(float2));
   W.colk = (int*)take(N * sizeof(int));
   W.cold = (int*)take(N * sizeof(int));
   W.rank = (int*)take(N * sizeof(int));
@@ -1712,8 +1714,6 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
   W.mergeof = nullptr;
 
   cudaMemsetAsync(slots, 0xFF, slot_bytes, st);      // every slot empty
-  // Q and Qtmp (adjacent): a merge's row tiles that straddle its children read zeros outside them
-  cudaMemsetAsync(W.Q, 0, (size_t)((char*)W.Qtmp - (char*)W.Q) + (size_t)N * N * sizeof(double), st);
   cudaMemsetAsync(d, 0, (3 * (size_t)N + 1) * sizeof(double), st);
   k_absmax<<<std::min(N, 304), 256, 0, st>>>(A, lda, N, amax); note_launch();
 
@@ -1744,6 +1744,8 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
     if (ce != cudaSuccess) return 1000 + (int)ce;
   }
   if (marks) cudaEventRecord(marks[0], st);
+  // Q and Qtmp (adjacent): a merge's row tiles that straddle its children read zeros outside them
+  cudaMemsetAsync(W.Q, 0, (size_t)((char*)W.Qtmp - (char*)W.Q) + (size_t)N * N * sizeof(double), st);
   // 2. divide and conquer; the T matrices of the back-transformation ride on the first launch of small merges
   const bool ff = sizeof(T) == sizeof(double) && assembly == kAssemblyFF && N >= 3 &&
                   (size_t)(2 * RB + CB) * N * sizeof(float2) <= 227 * 1024;   // (the double-buffered staging fits)
