@@ -1344,6 +1344,29 @@ uint8_t* bpre_scratch(size_t bytes) {
   return t_bpre;
 }
 
+}  // namespace
+
+// The last chunks of a split K range (kchunks chunks of kslices slices, nk in all; base_units output tiles; at most
+// cap chunks of partial sums fit).  A last round of units with few of them would leave most SMs idle for a whole unit's
+// time: the chunks those units belong to are cut finer instead, one round of short units (512 x 577 x 65,536: 768
+// units of 64 slices are 5.05 rounds of 152 CTAs; 756 of them and 144 of 6 slices are 5.1).  More output tiles than
+// CTAs leave no room for that: such products keep the even split.  Returns 1 with out = {chunks of kslices, slices of
+// each later chunk, chunks in all}, or 0.
+extern "C" int cakf_split_tail(int base_units, int nk, int kslices, int kchunks, int slots, size_t cap, int* out) {
+  const int left = (base_units * kchunks) % slots, drop = (left + base_units - 1) / base_units;
+  if (base_units > slots || left == 0 || left > slots / 4 || drop >= kchunks) return 0;
+  const int per_unit = slots / base_units, kfull = kchunks - drop, tail = nk - kfull * kslices;
+  const int ktail = std::max(1, (tail + per_unit - 1) / per_unit);
+  const int total = kfull + (tail + ktail - 1) / ktail;
+  if (ktail >= kslices || (size_t)total > cap) return 0;
+  out[0] = kfull;
+  out[1] = ktail;
+  out[2] = total;
+  return 1;
+}
+
+namespace {
+
 int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A, int lda, const float* B, int ldb,
                    float beta, float* C_f32, int ldc, bool force_split, float* part, size_t part_floats,
                    int* kchunks_out, int* Mpad_out, int* err, cudaStream_t st) {
@@ -1384,18 +1407,12 @@ int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A
   const bool split = force_split || P.kchunks > 1;
   P.kfull = P.kchunks;
   P.ktail = P.kslices;
-  // a last round of units with few of them would leave most SMs idle for a whole unit's time: the chunks those
-  // units belong to are cut finer instead, one round of short units (512 x 577 x 65,536: 768 units of 64 slices
-  // are 5.05 rounds of 152 CTAs; 756 of them and 144 of 6 slices are 5.1)
-  const int left = (base_units * P.kchunks) % slots, drop = (left + base_units - 1) / base_units;
-  if (split && left > 0 && left <= slots / 4 && drop < P.kchunks) {
-    const int kfull = P.kchunks - drop, tail = P.nk - kfull * P.kslices;
-    const int ktail = std::max(1, (tail + slots / base_units - 1) / (slots / base_units));
-    const int total = kfull + (tail + ktail - 1) / ktail;
-    if (ktail < P.kslices && (size_t)total * N * P.Mpad <= part_floats) {
-      P.kfull = kfull;
-      P.ktail = ktail;
-      P.kchunks = total;
+  if (split) {
+    int tail[3];
+    if (cakf_split_tail(base_units, P.nk, P.kslices, P.kchunks, slots, part_floats / ((size_t)N * P.Mpad), tail)) {
+      P.kfull = tail[0];
+      P.ktail = tail[1];
+      P.kchunks = tail[2];
     }
   }
   if (split && !part) return 11;
