@@ -6,6 +6,7 @@
 #include <string>
 #include "cakf.h"
 #include "internal.h"
+#include "fp64_ops.cuh"
 
 namespace cakf {
 namespace {
@@ -47,6 +48,16 @@ __global__ void __launch_bounds__(PROBE_THREADS) k_probe_dfma(int iters, double*
 #pragma unroll
   for (int c = 0; c < PROBE_CHAINS; ++c) acc += v[c];
   if (acc == 12345.678) out[blockIdx.x * blockDim.x + threadIdx.x] = acc;
+}
+
+// Row i of x (32 NV values): out[i] = warp_sum_int of it, lane l holding values NV l .. NV l + NV - 1.
+template <int NV>
+__global__ void __launch_bounds__(32) k_probe_warp_sum(const double* x, double* out) {
+  double v[NV];
+#pragma unroll
+  for (int u = 0; u < NV; ++u) v[u] = x[((size_t)blockIdx.x * 32 + threadIdx.x) * NV + u];
+  const double s = warp_sum_int<NV>(v);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 template <class F>
@@ -100,4 +111,14 @@ extern "C" int cakf_probe_peaks(double* mufu_ops_per_s, double* fp64_flops_per_s
   *mufu_ops_per_s = threads * it_mufu * PROBE_CHAINS * 2.0 / (ms_mufu * 1e-3);
   *fp64_flops_per_s = threads * it_dfma * PROBE_CHAINS * 2.0 / (ms_dfma * 1e-3);
   return CAKF_OK;
+}
+
+// The eigensolver's integer warp sum by itself, for its test: rows of 32 nv values (nv 1 or 4), device arrays.
+extern "C" int cakf_probe_warp_sum(int32_t nv, int32_t rows, const double* x, double* out) {
+  if ((nv != 1 && nv != 4) || rows < 1 || !x || !out)
+    return set_last_error(CAKF_ERR_ARG, "cakf_probe_warp_sum: invalid argument");
+  if (nv == 1) k_probe_warp_sum<1><<<rows, 32>>>(x, out);
+  else k_probe_warp_sum<4><<<rows, 32>>>(x, out);
+  const cudaError_t ce = cudaDeviceSynchronize();
+  return ce == cudaSuccess ? CAKF_OK : set_last_error(CAKF_ERR_CUDA, cudaGetErrorString(ce));
 }
