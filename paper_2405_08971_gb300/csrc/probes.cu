@@ -60,6 +60,13 @@ __global__ void __launch_bounds__(32) k_probe_warp_sum(const double* x, double* 
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
+__global__ void __launch_bounds__(256) k_probe_roots(const double* x, int n, double* sq, double* rs, double* rc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  fast_sqrt(fabs(x[i]), sq[i], rs[i]);
+  rc[i] = fast_rcp(x[i]);
+}
+
 template <class F>
 double time_ms(F launch, cudaStream_t st) {
   cudaEvent_t e0, e1;
@@ -119,6 +126,15 @@ extern "C" int cakf_probe_warp_sum(int32_t nv, int32_t rows, const double* x, do
     return set_last_error(CAKF_ERR_ARG, "cakf_probe_warp_sum: invalid argument");
   if (nv == 1) k_probe_warp_sum<1><<<rows, 32>>>(x, out);
   else k_probe_warp_sum<4><<<rows, 32>>>(x, out);
+  const cudaError_t ce = cudaDeviceSynchronize();
+  return ce == cudaSuccess ? CAKF_OK : set_last_error(CAKF_ERR_CUDA, cudaGetErrorString(ce));
+}
+
+// The eigensolver's roots and reciprocals by themselves, for their test: sqrt|x|, 1 / sqrt|x| and 1 / x of n values,
+// device arrays.
+extern "C" int cakf_probe_roots(int32_t n, const double* x, double* sq, double* rs, double* rc) {
+  if (n < 1 || !x || !sq || !rs || !rc) return set_last_error(CAKF_ERR_ARG, "cakf_probe_roots: invalid argument");
+  k_probe_roots<<<(n - 1) / 256 + 1, 256>>>(x, n, sq, rs, rc);
   const cudaError_t ce = cudaDeviceSynchronize();
   return ce == cudaSuccess ? CAKF_OK : set_last_error(CAKF_ERR_CUDA, cudaGetErrorString(ce));
 }
