@@ -24,9 +24,14 @@ __device__ __forceinline__ float approx_exp_neg(float s) {   // exp(-s) via ex2.
 
 // ---- programmatic dependent launch.  A kernel started by launch_pdl may become resident while the
 // kernel before it in the stream is still running; pdl_wait() returns once that kernel has completed
-// and its writes are visible, so every such kernel calls it before it touches memory, and then
-// pdl_trigger() so that the next kernel's launch overlaps this one.  (Without the launch attribute
-// both are no-ops.)
+// and its writes are visible.  Every such kernel, in every block and thread, calls pdl_wait() first and
+// pdl_trigger() only after it, so that the next kernel's launch overlaps this one's work.  That order
+// is what the next kernel may rely on: when it starts, every block of this one has passed its wait, so
+// whatever was launched before this one has completed.  The CG kernels do rely on it: before their own
+// pdl_wait() they read (past L1) what was written two launches earlier or before, and never what the
+// kernel in front writes; they write nothing before it.  A kernel that triggers before it waits, or
+// leaves without waiting, must not stand in front of them.  (Without the launch attribute both calls
+// are no-ops and the order is the stream's.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

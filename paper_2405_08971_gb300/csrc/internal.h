@@ -12,9 +12,9 @@ namespace cakf {
 long long launch_count();
 void note_launch(long long k = 1);
 
-// Launch of a kernel that begins with pdl_wait(); pdl_trigger(); with programmatic stream
-// serialisation, so that its launch overlaps the previous kernel in the stream (the chains of short
-// dependent kernels of the CG loop and the eigensolver).  Counts the launch.
+// Launch of a kernel that calls pdl_wait() and then pdl_trigger() (the contract stands beside them in
+// common.cuh) with programmatic stream serialisation, so that its launch overlaps the previous kernel in
+// the stream (the chain of short dependent kernels of the CG loop).  Counts the launch.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args&&... args) {
