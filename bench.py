@@ -396,7 +396,7 @@ def main():
                                 "peak_source": peak_note.format("FP64 FMA chains, 2 flops each"),
                                 "launches": prof["eig_calls"], "avg_ms": tri_ms / prof["eig_calls"],
                                 "ms_total": tri_ms,
-                                "note": "one cross-block exchange per Householder column (epoch-tagged word pairs, no grid barrier): bound by its latency chain, not by FP64 throughput"}
+                                "note": "one cross-block exchange per Householder column (write-once words, no grid barrier): bound by its latency chain, not by FP64 throughput"}
     # tensor-core / SIMT Gram x block (filter finalize): kernel entries on MUFU (sqrt + exp2 each)
     if prof["gram_block_launches"]:
         gb_ms = prof["gram_block_ms"]
@@ -418,7 +418,7 @@ def main():
             ent["tensor_frac"] = mmas * tfl / tpk
             ent["tensor_peak_source"] = (f"{pk_src} bf16_tflops_sustained" + (" x 1.1/2.25 (nominal TF32/BF16)" if tf32 else "")
                                          + f"; {mmas} MMA(s) per algorithmic flop")
-        kernels["k_gram_tc" if args.precision in tc_modes else "k_gram_block_simt"] = ent
+        kernels["k_gram_tc" if args.precision in tc_modes else "k_gram_block_f64" if args.precision == "fp64" else "k_gram_block_f32"] = ent
     # CG Gram matvec (sampled every 8th iteration): m (m + 1) / 2 unique kernel entries per launch
     # (the symmetric Gram is evaluated once per entry pair), 2 MUFU operations each
     if prof["cg_matvec_launches"]:

@@ -324,6 +324,8 @@ int cakf_factor_gemm(int32_t trans_a, int32_t M, int32_t N, int32_t K, double al
  * `keep` eigenpairs of the N x N symmetric matrix A (the Gram M^T M of a downdate factor in the
  * filter and smoother), the same device code the filter and smoother run.
  *   A       DEVICE, N*N doubles, column-major (only read; a copy is factorised)
+ *   N       1 .. 1,446, or 1,610 with keep <= 508 (the back-transformation's shared memory; a larger order returns
+ *           CAKF_ERR_CUDA, as does a filter whose rank plus budget needs one)
  *   w_out   DEVICE, keep doubles: eigenvalues in descending order
  *   U_out   DEVICE, N*keep doubles, column-major: the matching orthonormal eigenvectors
  * Its workspace is kept per thread for the next call up to 64 MB and freed on return beyond (it is

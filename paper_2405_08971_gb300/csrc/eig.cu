@@ -1588,11 +1588,11 @@ size_t eig_workspace_bytes(int nmax) {
   b += align_up((3 * N + 1) * sizeof(double));    // d, e, tau, largest magnitude
   b += 3 * align_up(N * N * sizeof(double));      // Q, Qtmp, Delta
   b += align_up((N / RB + 2) * RB * N * sizeof(float2));    // reflector groups as double-FP32 pairs
-  b += 10 * align_up(N * sizeof(double));         // lam, lamk, lamtmp, Dw, Zw, Dk, Zk, Dd, rho, spare
+  b += 10 * align_up(N * sizeof(double));         // lam, lamk, Df, zf, Zw, Dk, Zk, Dd, rho, z2
   b += align_up(4 * N * sizeof(double));          // rot
   b += align_up((N / RB + 2) * RB * RB * sizeof(double));   // back-transform T blocks
   b += align_up((N / RB + 2) * RB * RB * sizeof(float2));   // T blocks as double-FP32 pairs
-  b += 7 * align_up(N * sizeof(int));             // colk, cold, perm, Kp, nrot, gperm, spare
+  b += 7 * align_up(N * sizeof(int));             // colk, cold, rank, Kp, nrot, gperm, spare
   b += align_up(2 * N * sizeof(int));             // gcnt
   return b + 4096;
 }

@@ -323,7 +323,7 @@ k_gemm_nn_f32(int M, int N, int K, float alpha, const float* __restrict__ A, int
 
 // FP64.  A block owns 32 rows (one per lane) and up to 72 columns, column w + 8 u with warp w.  What
 // counts is the number of FP64 instructions (a warp-wide one takes 19 cycles of its SM): a kernel
-// value costs about 37 of them, so it is evaluated once per 72 columns, columns are not padded (a
+// value costs about 41 of them (Matern-5/2: 74 per value at 33 columns, by the instruction counters), so it is evaluated once per 72 columns, columns are not padded (a
 // warp skips the ones beyond the width), and the cluster split keeps every SM busy.
 // 4,097 x 2,000 x 33 takes 1,340 us, against 3,350 us for 64 x 64 tiles (65 blocks, 64 columns computed).
 template <int KER, bool DER> __device__ __forceinline__ double kfn(const C4<double>& a, const C4<double>& b, double sf2) {
@@ -497,7 +497,10 @@ void gram_block_fn(int fn, const C4<T>* Xr, int nr, const C4<T>* Xc, int nc, con
                    T* Out, int ldo, cudaStream_t st) {
   if (nr <= 0 || width <= 0) return;
   const int nchunk = (width + GS_MAX_COLS - 1) / GS_MAX_COLS, cw = (width + nchunk - 1) / nchunk;
-  const int per = (cw + 7) / 8;                         // columns per thread (FP32) or warp (FP64)
+  // columns per thread (FP32) or warp (FP64), rounded up to an odd count: the filter's and smoother's blocks are
+  // i + 1 columns wide, i mostly a multiple of 16 (33 and 65 columns are 5 and 9 without padding).  Even
+  // counts would spare a width of 16, 32 or 64 a third to a ninth of its FP32 products; FP64 skips them anyway
+  const int per = (cw + 7) / 8;
 #define CAKF_GS(NAME)                                                                                             \
   if (per <= 1) NAME<1>(fn, Xr, nr, Xc, nc, B, ldb, width, cw, nchunk, sf2, Out, ldo, st);                        \
   else if (per <= 3) NAME<3>(fn, Xr, nr, Xc, nc, B, ldb, width, cw, nchunk, sf2, Out, ldo, st);                   \

@@ -3,8 +3,8 @@
 //   Out[i, c] = sf2 * sum_j corr(xr_i, xc_j) B[j, c]     (Out, B column-major; corr a Matern correlation)
 //
 // The kernel matrix is never stored.  The work is the sequence of (128-row tile, K slice) units,
-// split evenly over a persistent grid of one CTA per SM.  Per slice, 16 producer warps evaluate the
-// 128-row correlation tile from coordinates staged in shared memory and write it in the swizzled
+// split evenly over a persistent grid of one CTA per SM.  Per slice, 8 of the 16 producer warps (all 16 in
+// the plain TF32 mode) evaluate the 128-row correlation tile from coordinates staged in shared memory and write it in the swizzled
 // K-major layout the tensor core reads; a TMA warp stages the matching slice of the packed B
 // operand; one thread issues tcgen05.mma (M = 128, N <= 256 per instruction, K = 16) accumulating
 // in TMEM (up to 512 FP32 columns); the producer warps drain TMEM in the epilogue.  The last column
@@ -662,7 +662,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
 // TF32 parts and write the swizzled K-major operand layout; one thread issues the MMAs; the
 // producer warps drain TMEM.  A unit covering all of K writes alpha acc + beta C directly; with K
 // split over chunks (and every TN product, whose output is FP64) each unit writes its FP32 partial
-// tile and k_gemm_reduce sums the chunks in FP64.
+// tile and k_gemm_reduce sums the chunks (FP32 pairs of eight, then FP64).
 struct GemmParams {
   const float* A;
   int lda, transA;
@@ -1014,7 +1014,8 @@ k_gemm_prep_b(const float* __restrict__ B, int ldb, int K, int N, int cw, int np
   }
 }
 
-// C[row + col * ldc] = alpha * sum_kc part[(kc * N + col) * Mpad + row] + beta * C  (FP64 sums)
+// C[row + col * ldc] = alpha * sum_kc part[(kc * N + col) * Mpad + row] + beta * C  (eight
+// chunks at a time as an FP32 sum and its rounding errors, then FP64)
 template <class OutT>
 __global__ void k_gemm_reduce(const float* __restrict__ part, int kchunks, int M, int N, int Mpad, double alpha,
                               double beta, OutT* __restrict__ C, int ldc) {
@@ -1397,7 +1398,7 @@ int gemm_tc_launch(int transA, int Mr, int N, int K, float alpha, const float* A
     const size_t per_chunk = (size_t)N * P.Mpad;
     const int cap = part ? (int)std::min<size_t>(4096, part_floats / std::max<size_t>(per_chunk, 1)) : 1;
     // enough chunks to fill the GPU, and at most 64 slices (1,024 K values) per chunk so that the
-    // FP32 accumulation chains in TMEM stay short; the chunks are summed in FP64
+    // FP32 accumulation chains in TMEM stay short; k_gemm_reduce sums the chunks
     const int want = std::max((slots + base_units - 1) / base_units, (P.nk + 63) / 64);
     kchunks = std::max(1, std::min({want, cap, std::max(1, P.nk / 4)}));
     if (force_split && cap < 1) return 11;

@@ -216,7 +216,8 @@ int gram_block_tc(int ker, int kind, const C4<float>* Xr, int nr, const C4<float
 // per product, FP32 accumulation):
 //   gemm_tc_nn: C (M x N, float) = alpha A B + beta C, A M x K (lda), B K x N (ldb), column-major;
 //   gemm_tc_tn: C (na x nb, double) = alpha A^T B + beta C, A K x na, B K x nb, with the K range
-//               split over CTAs; part (part_bytes) holds the FP32 partial tiles, summed in FP64.
+//               split over CTAs; part (part_bytes) holds the FP32 partial tiles, summed in FP32
+//               pairs of eight and then FP64.
 // Return 0 on success (launch errors otherwise); a timed-out wait raises the device flag err.
 int gemm_tc_nn(int M, int N, int K, float alpha, const float* A, int lda, const float* B, int ldb, float beta,
                float* C, int ldc, int* err, cudaStream_t st);

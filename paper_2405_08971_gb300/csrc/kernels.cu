@@ -185,9 +185,9 @@ k_gram_matvec(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int 
 // The FP64 matvec for few observations, where even 32 x 32 tiles leave most SMs idle: every entry is
 // evaluated (no symmetry), a block takes 32 rows (one per lane) and MVS_W * cpw columns (cpw per
 // warp), and its sum goes to the slot of its column group, so the slots per row number
-// ceil(m / (MVS_W cpw)) and no column sums are needed.  An FP64 Matern value is about 60 dependent
-// FP64 operations (a warp-wide one takes 19 cycles of the SM's FP64 pipe), so what counts is how many
-// SMs share the values.
+// ceil(m / (MVS_W cpw)) and no column sums are needed.  An FP64 Matern-5/2 value is about 41
+// FP64 instructions, most of them a dependent chain (a warp-wide one takes 19 cycles of the SM's FP64 pipe), so
+// what counts is how many SMs share the values.
 template <int KER, class T>
 __global__ void __launch_bounds__(MVS_W * 32)
 k_gram_matvec_rows(const C4<T>* __restrict__ Xo, const T* __restrict__ s, int m, int nslot, int cpw, T sf2,
@@ -1863,7 +1863,7 @@ void gemm_tn(const T* A, int lda, int na, const T* B, int ldb, int nb, int K, do
              int ldc, double* part, size_t part_elems, cudaStream_t st) {
   if (na <= 0 || nb <= 0) return;
   if (sizeof(T) == 4 && t_gemm_mode == 2 && (double)na * nb * K > 2e7 && K >= 64) {
-    // FP32 operands on the tensor cores (split TF32), FP32 partial tiles summed in FP64
+    // FP32 operands on the tensor cores (split TF32), FP32 partial tiles summed by k_gemm_reduce
     if (gemm_tc_tn((const float*)A, lda, na, (const float*)B, ldb, nb, K, alpha, beta, C, ldc, part,
                    part_elems * sizeof(double), t_gemm_err, st) == 0)
       return;
