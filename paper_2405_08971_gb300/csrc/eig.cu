@@ -413,16 +413,22 @@ struct DcWork {
   int *colk, *cold, *rank, *Kp, *nrot, *mergeof, *gperm, *gcnt;
 };
 
-__global__ void k_dc_init(const double* __restrict__ d, const double* __restrict__ e, int N, double* lam,
-                          double* Q, double* Qtmp) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
+// Eigenvalues of the leaves, and Q = Qtmp = I: a merge's row tiles that straddle its children
+// read zeros outside them, and a leaf without a merge at the deepest level is valid in both.  (Both lie under
+// the exchange slots, so they are filled here, after the tridiagonalisation; as a memset of its own the fill took
+// 7 us of a call at N = 576 and 12 at 288.)
+__global__ void __launch_bounds__(256)
+k_dc_init(const double* __restrict__ d, const double* __restrict__ e, int N, double* lam, double* Q, double* Qtmp) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (t >= N) return;
+  const double one = t == j ? 1.0 : 0.0;
+  Q[(size_t)j * N + t] = one;
+  Qtmp[(size_t)j * N + t] = one;
+  if (t != j) return;
   double v = d[j];
   if (j > 0) v -= fabs(e[j - 1]);
   if (j + 1 < N) v -= fabs(e[j]);
   lam[j] = v;
-  Q[(size_t)j * N + j] = 1.0;
-  Qtmp[(size_t)j * N + j] = 1.0;    // (a leaf without a merge at the deepest level is valid in both)
 }
 
 // Order-preserving integer key of a double (IEEE bit pattern; negative values mirrored), so the
@@ -1671,14 +1677,12 @@ int eig_sym_topk(double* A, int lda, int N, int nkeep, double* w, T* U, int ldu,
     if (ce != cudaSuccess) return 1000 + (int)ce;
   }
   if (marks) cudaEventRecord(marks[0], st);
-  // Q and Qtmp (adjacent): a merge's row tiles that straddle its children read zeros outside them
-  cudaMemsetAsync(W.Q, 0, (size_t)((char*)W.Qtmp - (char*)W.Q) + (size_t)N * N * sizeof(double), st);
   // 2. divide and conquer; the T matrices of the back-transformation ride on the first launch of small merges
   const bool ff = sizeof(T) == sizeof(double) && assembly == kAssemblyFF && N >= 3 &&
                   (size_t)(2 * RB + CB) * N * sizeof(float2) <= 227 * 1024;   // (the double-buffered staging fits)
   const TmatArgs ta{A, lda, tau, W.Tm, ff ? Vff : nullptr, ff ? Tff : nullptr};
   int tmat_blocks = N >= 3 ? (N - 2 + RB - 1) / RB : 0;
-  k_dc_init<<<(N + 255) / 256, 256, 0, st>>>(d, e, N, W.lam, W.Q, W.Qtmp); note_launch();
+  k_dc_init<<<dim3((N + 255) / 256, N), 256, 0, st>>>(d, e, N, W.lam, W.Q, W.Qtmp); note_launch();
   const Plan& pl = pe->plan;
   const int nlev = (int)pl.level_off.size() - 1;
   for (int lv = 0; lv < nlev; ++lv) {
