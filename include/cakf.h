@@ -328,9 +328,9 @@ int cakf_factor_gemm(int32_t trans_a, int32_t M, int32_t N, int32_t K, double al
  *           CAKF_ERR_CUDA, as does a filter whose rank plus budget needs one)
  *   w_out   DEVICE, keep doubles: eigenvalues in descending order
  *   U_out   DEVICE, N*keep doubles, column-major: the matching orthonormal eigenvectors
- * Its workspace is kept per thread for the next call up to 64 MB and freed on return beyond (it is
- * meant for verification and tools, not for the hot loop).  Errors: CAKF_ERR_ARG, CAKF_ERR_OOM, CAKF_ERR_CUDA, CAKF_ERR_TIMEOUT,
- * CAKF_ERR_NUMERIC (secular iteration without convergence or non-finite values).
+ * Its workspace is kept per thread for the next call up to 64 MB (outside cakf_set_device_memory_limit, which
+ * counts contexts) and freed on return beyond; it is meant for verification and tools, not for the hot loop.
+ * Errors: CAKF_ERR_ARG, CAKF_ERR_OOM, CAKF_ERR_CUDA, CAKF_ERR_TIMEOUT, CAKF_ERR_NUMERIC (secular iteration without convergence or non-finite values).
  */
 int cakf_eig_topk(const double* A, int32_t N, int32_t keep, double* w_out, double* U_out, void* cuda_stream);
 
